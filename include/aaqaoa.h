@@ -540,8 +540,10 @@ int aaqaoa_launch_count(const aaqaoa_plan *plan, int *launches);
 /*
  * Launch profiling. While enabled, the plan records a CUDA event pair on its
  * stream around every kernel launch and keeps, per kernel kind, the launch
- * count and the bytes each launch has to move (statevector tiles loaded plus
- * stored). aaqaoa_profile_read synchronises the stream and returns the summed
+ * count and the bytes of the statevectors each launch loads plus stores, whole
+ * statevectors of 2^n amplitudes (the tiled passes of a MaxCut plan move half of
+ * that: they keep the half of the flip-symmetric state with vertex n - 1 on
+ * side 0, the other half being psi(x) = psi(~x)). aaqaoa_profile_read synchronises the stream and returns the summed
  * event durations (ms), launches and bytes of one kind:
  *   0 forward tiled pass, 1 adjoint tiled pass, 2 whole-circuit (small n)
  *   kernel, 3 aggregation over a stored state, 4 parameter tables.
@@ -553,7 +555,7 @@ int aaqaoa_profile_read(aaqaoa_plan *plan, int kind, double *ms_total, int *laun
 /*
  * aaqaoa_stats -- all kinds of aaqaoa_profile_read at once: per kind (index
  * as above) the launches recorded since profiling was enabled, their summed
- * event durations (ms) and the bytes they had to move. out: host struct.
+ * event durations (ms) and their bytes, counted as above. out: host struct.
  * Synchronises the plan's stream (so the plan is not const). INVALID_ARG for
  * a NULL plan or out; all zero when profiling was never enabled.
  */
@@ -571,7 +573,7 @@ int aaqaoa_stats(aaqaoa_plan *plan, aaqaoa_stats_t *out);
  * cut-function work -- phase, lambda = O phi, energy, dE/dgamma, inverse
  * phase; bit 1: a fused layer boundary; bit 2: the cluster low pass; bit 3:
  * the turnaround pass of a gradient evaluation), event duration (ms) and
- * bytes to move. kind, flags, ms, bytes: host arrays of at least max entries, each may
+ * bytes, counted as above. kind, flags, ms, bytes: host arrays of at least max entries, each may
  * be NULL. *count (host int) receives the number of records, also when it
  * exceeds max. Synchronises the plan's stream. INVALID_ARG for a NULL plan
  * or count, or max < 0.

@@ -92,6 +92,7 @@ struct Pass {
     int wide;    // tensor-map form (rows of more than 128 bytes)
     int skip_last = 0;  // low pass done after register stage 1
     int qubits = 0;     // butterflies of this pass
+    int pair = 0;       // spans vertex n - 1 of a half state: a tile and the mirrored tile
     int cluster = 0;    // the 14-qubit low pass of a cluster of 4 CTAs (complex64 adjoint)
 };
 
@@ -152,7 +153,15 @@ struct aaqaoa_plan {
     int tab_len() const { return wsum + 1; }  // cut values 0..sum of edge weights
     int out_stride() const { return 1 + 2 * p; }
     bool small() const { return n <= T(); }
-    int tiles() const { return small() ? 1 : 1 << (n - T()); }
+    // Index bits of the stored state. The tiled passes of a MaxCut plan keep the
+    // half of the flip-symmetric state with vertex n - 1 on side 0 (see k_pass)
+    bool half() const { return !ising && !small(); }
+    int bits() const { return half() ? n - 1 : n; }
+    size_t amps() const { return (size_t)1 << bits(); }
+    // a launch record's bytes count whole statevectors, whatever part is stored
+    double state_bytes() const { return (double)((size_t)1 << n) * (double)amp(); }
+    double sym() const { return half() ? 2.0 : 1.0; }  // what a sum over the stored amplitudes counts
+    int tiles() const { return small() ? 1 : 1 << (bits() - T()); }
     bool fuse = true;  // fuse layer boundaries into one pass where the plan allows
     int *err_shared = nullptr;  // set when the plan is part of a multi-graph batch
     const GraphFns *pt_dev = nullptr;  // set for a group of same-n graphs: point b is graph b
@@ -259,8 +268,8 @@ Layout layout(const aaqaoa_plan *pl, int batch, bool grad)
     return L;
 }
 
-// 5-D view of B statevectors for tiles of 2^T amplitudes: rows of 2^cb
-// contiguous amplitudes along qubits s..s+T-cb-1. A 128-byte segment holds
+// 5-D view of B statevectors of 2^n stored amplitudes for boxes of 2^T: rows of
+// 2^cb contiguous amplitudes along qubits s..s+T-cb-1. A 128-byte segment holds
 // 2^cbmin amplitudes. Nine row qubits (cb = cbmin) need two box dimensions
 // (32 x 16 rows); up to eight fit one (wide form, rows of 2^(cb-cbmin)
 // segments).
@@ -333,8 +342,10 @@ int make_cluster_map(CUtensorMap *map, void *base, int n, int B, bool load)
 // big_last (the adjoint's passes): the larger high groups come last, so that
 // the adjoint's last group can be the forward's last, smaller one (the pair a
 // turnaround pass takes).
+// half: the state is kept as its flip-symmetric half, and the last high group,
+// the one with qubit n - 1, runs as a pair pass.
 bool layer_passes(int n, int T, int cbmin, int hbmax, int L2, int L, int K, std::vector<Pass> &v,
-                  bool cluster_low = false, bool big_last = false)
+                  bool cluster_low = false, bool big_last = false, bool half = false)
 {
     v.clear();
     const bool cl = cluster_low && L == CLUSTER_LOW_QUBITS && T + 2 == CLUSTER_LOW_QUBITS;
@@ -353,6 +364,7 @@ bool layer_passes(int n, int T, int cbmin, int hbmax, int L2, int L, int K, std:
             return false;
         Pass hp{s, T - h, 0, (1 << h) - 1, 0};
         hp.qubits = h;
+        hp.pair = half && k == K - 1;
         v.push_back(hp);
         s += h;
     }
@@ -380,7 +392,7 @@ void build_passes(aaqaoa_plan *pl)
         pass_geometry(pl->c128, nv, &T, &CB, &HB);
         const int L2 = low_two_stage_bits(pl->c128, nv);
         default_layer(pl->n, T, CB, HB, L2, &L, &K, nv == 2);
-        layer_passes(pl->n, T, CB, HB, L2, L, K, nv == 1 ? pl->passes : pl->bwd_passes, false, nv == 2);
+        layer_passes(pl->n, T, CB, HB, L2, L, K, nv == 1 ? pl->passes : pl->bwd_passes, false, nv == 2, pl->half());
     }
 }
 
@@ -570,6 +582,7 @@ PassArgs forward_args(const aaqaoa_plan *pl, int obs, int B, const Step &sp, siz
     a.cb = ps.cb;
     a.wide_rows = ps.wide;
     a.is_low = ps.is_low;
+    a.pair = ps.pair;
     a.hmask = ps.hmask;
     a.skip_last = ps.skip_last;
     a.layer = sp.layer;
@@ -588,7 +601,7 @@ PassArgs forward_args(const aaqaoa_plan *pl, int obs, int B, const Step &sp, siz
         a.post |= POST_RESCALE;
     if (last && mode != FWD_STATE) {
         a.slot_idx[0] = 0;
-        a.slot_scale[0] = 1.0;
+        a.slot_scale[0] = pl->sym();
     }
     if (sp.layer2 >= 0) {
         a.fuse = 1;
@@ -618,7 +631,7 @@ int enqueue_forward(aaqaoa_plan *pl, int B, int obs, FwdMode mode)
             a.drop_first_load = 1;
             pl->inject = 0;
         }
-        const double S = (double)B * (double)((size_t)1 << pl->n) * (double)pl->amp();
+        const double S = (double)B * pl->state_bytes();
         ProfScope ps_(pl, PK_FWD, S * ((a.load ? 1 : 0) + (a.write ? 1 : 0)), pass_flags(a));
         CKL(launch_pass(pl->c128, 1, pl->map_phi[sp.k], pl->map_phi[sp.k], a, grid, pl->stream), "forward pass");
         pl->launches++;
@@ -632,10 +645,10 @@ int enqueue_backward(aaqaoa_plan *pl, int B, int obs)
 {
     int T, CB, HB;
     pass_geometry(pl->c128, 2, &T, &CB, &HB);
-    const int tiles = 1 << (pl->n - T);
+    const int tiles = 1 << (pl->bits() - T);
     const int grid = pass_grid((long long)tiles * B);
     const int chunk = B > 1 ? (int)(((long long)tiles * B + grid - 1) / grid) : 0;
-    const double S = (double)B * (double)((size_t)1 << pl->n) * (double)pl->amp();
+    const double S = (double)B * pl->state_bytes();
     const Turn tn = turnaround(pl);
     const int lp = pl->p - 1;  // the last layer: the adjoint's first
     if (tn.kb >= 0) {
@@ -654,6 +667,7 @@ int enqueue_backward(aaqaoa_plan *pl, int B, int obs)
         a.cb = ps.cb;
         a.wide_rows = ps.wide;
         a.is_low = 0;
+        a.pair = ps.pair;
         a.hmask = ps.hmask;
         a.layer = a.layer2 = a.tab_layer = lp;
         a.sign_s = 1.0;
@@ -666,9 +680,9 @@ int enqueue_backward(aaqaoa_plan *pl, int B, int obs)
         a.post = POST_REDUCE | POST_RESCALE | POST_LAMBDA;
         a.fuse = 1;
         a.slot_idx[0] = 0;  // the energy
-        a.slot_scale[0] = 1.0;
+        a.slot_scale[0] = pl->sym();
         a.slot_idx[2] = 1 + pl->p + lp;  // dE/dbeta of the last layer, this group's share
-        a.slot_scale[2] = 2.0;
+        a.slot_scale[2] = 2.0 * pl->sym();
         if (pl->inject == AAQAOA_FAULT_DROP_TILE) {
             a.drop_first_load = 1;
             pl->inject = 0;
@@ -694,6 +708,7 @@ int enqueue_backward(aaqaoa_plan *pl, int B, int obs)
         a.cb = ps.cb;
         a.wide_rows = ps.wide;
         a.is_low = ps.is_low;
+        a.pair = ps.pair;
         a.hmask = ps.hmask;
         a.skip_last = ps.skip_last;
         a.layer = l;
@@ -708,23 +723,23 @@ int enqueue_backward(aaqaoa_plan *pl, int B, int obs)
         a.post = sp.last_of_layer ? (POST_GAMMA | (l > 0 ? POST_PHASE_CONJ : 0)) : 0;
         a.write = !(sp.last_of_layer && l == 0);
         a.slot_idx[0] = 1 + pl->p + l;
-        a.slot_scale[0] = 2.0;
+        a.slot_scale[0] = 2.0 * pl->sym();
         if (sp.last_of_layer) {
             a.slot_idx[1] = 1 + l;
-            a.slot_scale[1] = 2.0;
+            a.slot_scale[1] = 2.0 * pl->sym();
         }
         if (sp.layer2 >= 0) {  // the next layer (l - 1) starts on the same qubits
             a.fuse = 1;
             a.layer2 = sp.layer2;
             a.slot_idx[2] = 1 + pl->p + sp.layer2;
-            a.slot_scale[2] = 2.0;
+            a.slot_scale[2] = 2.0 * pl->sym();
         }
         if (ps.cluster) {  // one launch per point, each over that point's cluster tiles
             for (int b = 0; b < B; b++) {
                 PassArgs ab = a;
                 ab.B = 1;
                 ab.chunk = 0;
-                ab.tile0 = b << (pl->n - CLUSTER_LOW_QUBITS);
+                ab.tile0 = b << (pl->bits() - CLUSTER_LOW_QUBITS);
                 ab.cs = a.cs + (size_t)b * pl->p;
                 ab.out = a.out + (size_t)b * pl->out_stride();
                 ProfScope ps_(pl, PK_ADJ, S / B * (a.nvec_io + 2), pass_flags(a) | 4);
@@ -803,12 +818,14 @@ int enqueue_aggregate(aaqaoa_plan *pl, int obs, int agg)
     AggArgs a;
     memset(&a, 0, sizeof a);
     a.n = pl->n;
-    a.chunks = pl->n < 10 ? 0 : ((uint64_t)1 << (pl->n - 10));
+    a.bits = pl->bits();
+    a.scale = pl->sym();
+    a.chunks = pl->n < 10 ? 0 : pl->amps() >> 10;
     a.state = pl->d_phi();
     a.partials = pl->d_partials();
     a.counter = pl->d_counter_agg();
     a.out_energy = pl->d_out();
-    const double S = (double)((size_t)1 << pl->n) * (double)pl->amp();
+    const double S = pl->state_bytes();
     if (agg == AAQAOA_AGG_SINGLEPASS) {
         a.obs = pl->obs[obs];
         ProfScope ps_(pl, PK_AGG, S);
@@ -1167,6 +1184,7 @@ int aaqaoa_prepare_ising(int n, int num_edges, const int32_t *edges, const doubl
         }
     }
     pl->ising = true;
+    build_passes(pl);  // an Ising state is kept whole: no pair passes
     pl->wsum = 0;  // the phase tables carry only the butterfly scale (one entry)
     pl->ising_w.assign(edge_weight, edge_weight + num_edges);
     if (field)
@@ -1225,7 +1243,8 @@ int build_maps(aaqaoa_plan *pl)
     pass_geometry(pl->c128, 1, &T, &CB, &HB);
     for (size_t k = 0; k < pl->passes.size(); k++) {
         Pass &ps = pl->passes[k];
-        int r = make_map(&pl->map_phi[k], pl->d_phi(), pl->n, ps.s, ps.cb, T, CB, pl->amp(), pl->cap, &ps.wide);
+        int r = make_map(&pl->map_phi[k], pl->d_phi(), pl->bits(), ps.s, ps.cb, T - ps.pair, CB, pl->amp(), pl->cap,
+                         &ps.wide);
         if (r)
             return r;
     }
@@ -1235,17 +1254,19 @@ int build_maps(aaqaoa_plan *pl)
             Pass &ps = pl->bwd_passes[k];
             if (ps.cluster) {
                 for (int j = 0; j < 4; j++) {
-                    int r = make_cluster_map(&pl->map_bcl[k][j], j % 2 ? pl->d_lam() : pl->d_phi(), pl->n, pl->cap,
+                    int r = make_cluster_map(&pl->map_bcl[k][j], j % 2 ? pl->d_lam() : pl->d_phi(), pl->bits(), pl->cap,
                                              j < 2);
                     if (r)
                         return r;
                 }
                 continue;
             }
-            int r = make_map(&pl->map_bphi[k], pl->d_phi(), pl->n, ps.s, ps.cb, T, CB, pl->amp(), pl->cap, &ps.wide);
+            int r = make_map(&pl->map_bphi[k], pl->d_phi(), pl->bits(), ps.s, ps.cb, T - ps.pair, CB, pl->amp(),
+                             pl->cap, &ps.wide);
             if (r)
                 return r;
-            r = make_map(&pl->map_blam[k], pl->d_lam(), pl->n, ps.s, ps.cb, T, CB, pl->amp(), pl->cap, &ps.wide);
+            r = make_map(&pl->map_blam[k], pl->d_lam(), pl->bits(), ps.s, ps.cb, T - ps.pair, CB, pl->amp(), pl->cap,
+                         &ps.wide);
             if (r)
                 return r;
         }
@@ -1297,7 +1318,7 @@ static int set_layers(aaqaoa_plan *pl, const int plan4[4])
             L = plan4[2 * (nv - 1)];
         if (plan4[2 * (nv - 1) + 1] > 0)
             K = plan4[2 * (nv - 1) + 1];
-        if (!layer_passes(pl->n, T, CB, HB, L2, L, K, v[nv - 1], nv == 2 && !pl->c128, nv == 2))
+        if (!layer_passes(pl->n, T, CB, HB, L2, L, K, v[nv - 1], nv == 2 && !pl->c128, nv == 2, pl->half()))
             return fail(AAQAOA_ERR_INVALID_ARG, "%s plan: low pass of %d qubits + %d high passes does not tile n=%d",
                         nv == 1 ? "forward" : "adjoint", L, K, pl->n);
     }
@@ -1697,7 +1718,7 @@ int aaqaoa_statevector(aaqaoa_plan *pl, const double *gamma, const double *beta,
         if ((r = enqueue_forward(pl, 1, AAQAOA_OBS_FULL, FWD_STATE)))
             return r;
         // the passes store the twisted, shifted-angle state: map it back
-        CKL(launch_untwist(pl->c128, pl->d_phi(), pl->n, pl->d_cs(), pl->p, pl->ising ? 1 : 0, pl->stream),
+        CKL(launch_untwist(pl->c128, pl->d_phi(), pl->n, pl->bits(), pl->d_cs(), pl->p, pl->ising ? 1 : 0, pl->stream),
             "statevector export");
         pl->launches++;
     }
@@ -1735,7 +1756,9 @@ int aaqaoa_edge_zz(aaqaoa_plan *pl, const double *gamma, const double *beta, dou
         AggArgs a;
         memset(&a, 0, sizeof a);
         a.n = pl->n;
-        a.chunks = pl->n < 10 ? 0 : ((uint64_t)1 << (pl->n - 10));
+        a.bits = pl->bits();
+        a.scale = pl->sym();
+        a.chunks = pl->n < 10 ? 0 : pl->amps() >> 10;
         a.state = pl->d_phi();
         a.partials = pl->d_partials();
         a.counter = pl->d_counter_agg();
@@ -1835,7 +1858,7 @@ int aaqaoa_sample(aaqaoa_plan *pl, const double *gamma, const double *beta, int 
     }
     pl->state_valid = true;
     CK(cudaMemcpyAsync(pl->d_samp_u(), u, (size_t)K * sizeof(double), cudaMemcpyHostToDevice, pl->stream));
-    CKL(launch_sample(pl->c128, pl->d_phi(), pl->n, pl->d_samp_sums(), pl->d_samp_total(), K, pl->d_samp_u(),
+    CKL(launch_sample(pl->c128, pl->d_phi(), pl->n, pl->bits(), pl->d_samp_sums(), pl->d_samp_total(), K, pl->d_samp_u(),
                       pl->d_samp_x(), cut_out ? pl->d_samp_cut() : nullptr, pl->cost, pl->stream),
         "sampling");
     pl->launches += 3;
@@ -2100,8 +2123,8 @@ extern "C" int aaqaoa_expect_static(aaqaoa_plan *pl, const double *gamma, const 
             return fail(AAQAOA_ERR_UNSUPPORTED, "%d passes per layer", np);
         int wide[8];
         for (int k = 0; k < np; k++)
-            if ((r = make_map(&maps[k], d_phi, pl->n, pl->passes[k].s, pl->passes[k].cb, pl->T(), pl->CB(), pl->amp(),
-                              1, &wide[k])))
+            if ((r = make_map(&maps[k], d_phi, pl->bits(), pl->passes[k].s, pl->passes[k].cb,
+                              pl->T() - pl->passes[k].pair, pl->CB(), pl->amp(), 1, &wide[k])))
                 return r;
         const int grid = pass_grid(pl->tiles());
         const std::vector<Step> sched = layer_schedule(p, pl->passes, plan_fuses(pl), false, !pl->c128);

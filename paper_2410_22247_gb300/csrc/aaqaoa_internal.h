@@ -69,7 +69,9 @@ struct PassArgs {
     int wide_rows;    // tensor map form: 1 when a row spans more than 128 bytes
     int is_low;       // tile is contiguous and its low bits are transformed here
     int hmask;        // which local high bits (bit j = local bit cb + j) get a butterfly
-    int tiles;        // tiles per statevector = 2^(n - tile bits)
+    int pair;         // the tile's top local bit is vertex n - 1 of a state kept as its
+                      // flip-symmetric half: a tile and the mirrored tile (see k_pass)
+    int tiles;        // tiles per stored statevector (a power of two)
     int B;            // statevectors (parameter points) in this launch
     int chunk;        // 0: CTAs interleave tiles; else each CTA takes `chunk` consecutive tiles
     int skip_last;    // low pass whose qubits all lie in register stages 0 and 1 (no third stage)
@@ -148,7 +150,9 @@ struct SmallGraph {
 // Aggregation over a stored statevector.
 struct AggArgs {
     int n;
-    uint64_t chunks;     // number of 1024-amplitude chunks (per state)
+    int bits;            // index bits of the stored state: n, or n - 1 for a flip-symmetric half
+    double scale;        // 2^(n - bits): what a sum over the stored amplitudes stands for
+    uint64_t chunks;     // number of 1024-amplitude chunks (per stored state)
     const void *state;
     double *partials;    // [T][grid]
     unsigned *counter;
@@ -192,10 +196,10 @@ int launch_agg_fused(bool c128, const AggArgs &a, cudaStream_t st, int grid);
 int launch_agg_terms(bool c128, const AggArgs &a, cudaStream_t st, int grid);
 int agg_grid(bool c128);
 size_t small_multi_smem_bytes(bool c128, int max_n, int max_tab);
-int launch_untwist(bool c128, void *psi, int n, const double2 *cs, int p, int noshift, cudaStream_t st);
+int launch_untwist(bool c128, void *psi, int n, int bits, const double2 *cs, int p, int noshift, cudaStream_t st);
 int launch_maxcut(const CostFn &cost, int n, unsigned long long *d_key, cudaStream_t st);
 size_t sample_chunk_count(int n);
-int launch_sample(bool c128, const void *psi, int n, double *d_sums, double *d_total, int K, const double *d_u,
+int launch_sample(bool c128, const void *psi, int n, int bits, double *d_sums, double *d_total, int K, const double *d_u,
                   unsigned long long *d_x, int *d_cut, const CostFn &cost, cudaStream_t st);
 int launch_small_multi(bool c128, const SmallGraph *d_graphs, int G, int p, int obs, int max_n, int max_tab,
                        const double *d_gamma, const double *d_beta, double *d_energy, cudaStream_t st);

@@ -317,12 +317,12 @@ __global__ void __maxnreg__((Geo<float, 2>::MAXREG))
             C a[NR], l[NR];
             C *sv0 = reinterpret_cast<C *>(sm + (size_t)q * 2 * TB);
             C *sv1 = reinterpret_cast<C *>(sm + (size_t)q * 2 * TB + TB);
-            load_regs<R, 2, 2>(sv0, sb2, a);
-            load_regs<R, 2, 2>(sv1, sb2, l);
+            load_regs<R, 2, 2>(sv0, sb2, sb2, a);
+            load_regs<R, 2, 2>(sv1, sb2, sb2, l);
             R run3 = run_after2;
-            mix_regs<R, 2, 3>(P, X.cb, X.tq, X.f, run3, a, l, acc0);
-            store_regs<R, 2, 2>(sv0, sb2, a);
-            store_regs<R, 2, 2>(sv1, sb2, l);
+            mix_regs<R, 2, 3>(P, X, X.tq, X.f, run3, a, l, acc0);
+            store_regs<R, 2, 2>(sv0, sb2, sb2, a);
+            store_regs<R, 2, 2>(sv1, sb2, sb2, l);
             fence_proxy_async_smem();
             mbar_arrive(&done[q]);
             return true;
@@ -355,14 +355,14 @@ __global__ void __maxnreg__((Geo<float, 2>::MAXREG))
             pending = -1;
             compute_sync<NTHR>();
             // stage 2: local bits 8..11, then the exchange
-            load_regs<R, 2, 2>(X.sv0, sb2, a);
-            load_regs<R, 2, 2>(X.sv1, sb2, l);
+            load_regs<R, 2, 2>(X.sv0, sb2, sb2, a);
+            load_regs<R, 2, 2>(X.sv1, sb2, sb2, l);
             fence_proxy_async_smem();  // these reads precede the peers' asynchronous stores
             compute_sync<NTHR>();      // this CTA's stage-2 reads are done
             if (tid < CLUSTER_CTAS)
                 mbar_arrive_remote(map_to_cta(smem_u32(&xl[q]), (uint32_t)tid));
             open_tile = (long long)k;
-            mix_regs<R, 2, 2>(P, X.cb, X.tq, X.f, X.run, a, l, acc0);
+            mix_regs<R, 2, 2>(P, X, X.tq, X.f, X.run, a, l, acc0);
             run_after2 = X.run;
             const bool wl = mbar_wait_cluster_bounded(&xl[q], par);
             if (compute_sync_or<NTHR>(!wl)) {
@@ -761,6 +761,7 @@ __device__ void agg_finish(const AggArgs &A, int nslots, double (*vals), double 
             a += __ldcg(A.partials + (size_t)t * gridDim.x + i);
         block_sum2<NTHR>(a, dummy, red);
         if (threadIdx.x == 0) {
+            a *= A.scale;
             if (A.num_terms == 0) {
                 *A.out_energy += a;
             } else {
@@ -774,7 +775,9 @@ __device__ void agg_finish(const AggArgs &A, int nslots, double (*vals), double 
         *A.counter = 0u;
 }
 
-// E += sum_x |psi_x|^2 O(x) over a stored state (one read).
+// E += sum_x |psi_x|^2 O(x) over a stored state (one read). A flip-symmetric
+// half (A.bits = n - 1) holds the states with vertex n - 1 on side 0; O and
+// every Z_u Z_v are equal on the other half, so the sum counts twice.
 template <typename R>
 __global__ void __launch_bounds__(256) k_agg_fused(const __grid_constant__ AggArgs A)
 {
@@ -784,8 +787,8 @@ __global__ void __launch_bounds__(256) k_agg_fused(const __grid_constant__ AggAr
     const int lane = threadIdx.x & 31;
     const C *st = reinterpret_cast<const C *>(A.state);
     double acc = 0.0;
-    if (A.n < 10) {
-        const int N = 1 << A.n;
+    if (A.bits < 10) {
+        const int N = 1 << A.bits;
         if (blockIdx.x == 0)
             for (int x = threadIdx.x; x < N; x += 256)
                 acc += (double)((st[x].x * st[x].x + st[x].y * st[x].y) * (R)cut_direct(A.obs, A.n, (uint32_t)x));
@@ -829,8 +832,8 @@ __global__ void __launch_bounds__(256) k_agg_terms(const __grid_constant__ AggAr
     for (int t = 0; t < T; t++)
         acc_s[t * 256 + threadIdx.x] = 0.0;
     const C *st = reinterpret_cast<const C *>(A.state);
-    if (A.n < 10) {
-        const int N = 1 << A.n;
+    if (A.bits < 10) {
+        const int N = 1 << A.bits;
         if (blockIdx.x == 0)
             for (int x = threadIdx.x; x < N; x += 256) {
                 const double pr = (double)(st[x].x * st[x].x + st[x].y * st[x].y);
@@ -1072,11 +1075,12 @@ int launch_small(bool c128, const SmallArgs &a, int B, cudaStream_t st)
 // circuit with every mixer layer l whose |sin beta_l| > |cos beta_l| rotated
 // by beta_l - pi/2 instead of beta_l. With K such layers
 //   psi = (-i)^(n K) (X^n)^K psi',
-// so psi(x) = (-i)^(nK) i^(-|y|) psi~(y), y = x with all bits flipped when K
-// is odd, else y = x. In place; for odd K each thread handles a pair (x, ~x).
-// Ising plans never rotate by beta_l - pi/2 (noshift): K = 0.
+// and X^n psi' = psi' for a MaxCut state, kept as its half with vertex n - 1
+// on side 0 (bits = n - 1): psi(x) = (-i)^(nK) i^(-|x|) psi~(x) there, in
+// place, and psi(~x) = psi(x) fills the buffer's other half. Ising plans keep
+// the whole state and never rotate by beta_l - pi/2 (noshift): K = 0.
 template <typename R>
-__global__ void k_untwist(typename CT<R>::T *psi, int n, const double2 *cs, int p, int noshift)
+__global__ void k_untwist(typename CT<R>::T *psi, int n, int bits, const double2 *cs, int p, int noshift)
 {
     using C = typename CT<R>::T;
     int K = 0;
@@ -1087,18 +1091,12 @@ __global__ void k_untwist(typename CT<R>::T *psi, int n, const double2 *cs, int 
         e &= 3;
         return e == 0 ? v : e == 1 ? mkc<C>(-v.y, v.x) : e == 2 ? mkc<C>(-v.x, -v.y) : mkc<C>(v.y, -v.x);
     };
-    const uint64_t N = 1ull << n, full = N - 1;
-    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    if (K & 1) {
-        for (uint64_t x = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; x < N / 2; x += stride) {
-            const uint64_t y = x ^ full;
-            const C vx = psi[x], vy = psi[y];
-            psi[x] = turn(vy, ph - __popcll(y));
-            psi[y] = turn(vx, ph - __popcll(x));
-        }
-    } else {
-        for (uint64_t x = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; x < N; x += stride)
-            psi[x] = turn(psi[x], ph - __popcll(x));
+    const uint64_t N = 1ull << bits, stride = (uint64_t)gridDim.x * blockDim.x;
+    for (uint64_t x = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; x < N; x += stride) {
+        const C v = turn(psi[x], ph - __popcll(x));
+        psi[x] = v;
+        if (bits < n)
+            psi[(N << 1) - 1 - x] = v;
     }
 }
 
@@ -1164,15 +1162,17 @@ int launch_maxcut(const CostFn &cost, int n, unsigned long long *d_key, cudaStre
 // the cumulative mass before the chunk; then one warp per sample finds the
 // chunk by binary search and the amplitude inside it by a lane scan. Sample k
 // is the smallest x whose cumulative mass exceeds u_k * total (the last index
-// if rounding leaves none).
+// if rounding leaves none). Of a flip-symmetric state the half with the top
+// bit clear is stored (bits = n - 1): psi(x) = psi(~x), and chunk c of the
+// other half holds the amplitudes of chunk nchunks - 1 - c backwards.
 constexpr int SAMPLE_BITS = 12;
 
 template <typename R>
-__global__ void __launch_bounds__(256) k_sample_chunks(const typename CT<R>::T *psi, int n, double *sums)
+__global__ void __launch_bounds__(256) k_sample_chunks(const typename CT<R>::T *psi, int n, int bits, double *sums)
 {
     __shared__ double red[2][32];
     const int cb = n < SAMPLE_BITS ? n : SAMPLE_BITS;
-    const uint64_t nchunks = 1ull << (n - cb), len = 1ull << cb;
+    const uint64_t all = 1ull << (n - cb), nchunks = bits < n ? all / 2 : all, len = 1ull << cb;
     for (uint64_t c = blockIdx.x; c < nchunks; c += gridDim.x) {
         double s = 0.0;
         for (uint64_t i = threadIdx.x; i < len; i += blockDim.x) {
@@ -1181,8 +1181,11 @@ __global__ void __launch_bounds__(256) k_sample_chunks(const typename CT<R>::T *
         }
         double z = 0.0;
         block_sum2<256>(s, z, red);
-        if (threadIdx.x == 0)
+        if (threadIdx.x == 0) {
             sums[c] = s;
+            if (bits < n)
+                sums[all - 1 - c] = s;
+        }
         __syncthreads();
     }
 }
@@ -1218,7 +1221,7 @@ __global__ void __launch_bounds__(1024) k_sample_scan(double *v, uint64_t count,
 }
 
 template <typename R>
-__global__ void __launch_bounds__(256) k_sample_draw(const typename CT<R>::T *psi, int n, const double *prefix,
+__global__ void __launch_bounds__(256) k_sample_draw(const typename CT<R>::T *psi, int n, int bits, const double *prefix,
                                                      const double *total, int K, const double *u,
                                                      unsigned long long *x_out, int *cut_out,
                                                      const __grid_constant__ CostFn cost)
@@ -1229,6 +1232,10 @@ __global__ void __launch_bounds__(256) k_sample_draw(const typename CT<R>::T *ps
     const int cb = n < SAMPLE_BITS ? n : SAMPLE_BITS;
     const uint64_t nchunks = 1ull << (n - cb), len = 1ull << cb, N = 1ull << n;
     const uint64_t per = len >= 32 ? len / 32 : 1;  // amplitudes per lane
+    auto mass = [&](uint64_t x) {
+        const typename CT<R>::T a = psi[x >> bits ? N - 1 - x : x];
+        return (double)a.x * (double)a.x + (double)a.y * (double)a.y;
+    };
     for (int k = warp; k < K; k += nwarps) {
         const double t = u[k] * *total;
         uint64_t lo = 0, hi = nchunks;  // last chunk with prefix <= t
@@ -1245,10 +1252,8 @@ __global__ void __launch_bounds__(256) k_sample_draw(const typename CT<R>::T *ps
         const uint64_t base = c * len + (uint64_t)lane * per;
         double s = 0.0;
         if ((uint64_t)lane * per < len)
-            for (uint64_t i = 0; i < per; i++) {
-                const typename CT<R>::T a = psi[base + i];
-                s += (double)a.x * (double)a.x + (double)a.y * (double)a.y;
-            }
+            for (uint64_t i = 0; i < per; i++)
+                s += mass(base + i);
         double inc = s;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -1265,8 +1270,7 @@ __global__ void __launch_bounds__(256) k_sample_draw(const typename CT<R>::T *ps
             if (lane == L) {
                 double run = before;
                 for (uint64_t i = 0; i < per; i++) {
-                    const typename CT<R>::T a = psi[base + i];
-                    run += (double)a.x * (double)a.x + (double)a.y * (double)a.y;
+                    run += mass(base + i);
                     if (run > rem) {
                         x = base + i;
                         break;
@@ -1295,31 +1299,32 @@ __global__ void __launch_bounds__(256) k_sample_draw(const typename CT<R>::T *ps
 
 size_t sample_chunk_count(int n) { return (size_t)1 << (n < SAMPLE_BITS ? 0 : n - SAMPLE_BITS); }
 
-int launch_sample(bool c128, const void *psi, int n, double *d_sums, double *d_total, int K, const double *d_u,
+int launch_sample(bool c128, const void *psi, int n, int bits, double *d_sums, double *d_total, int K, const double *d_u,
                   unsigned long long *d_x, int *d_cut, const CostFn &cost, cudaStream_t st)
 {
     const uint64_t nchunks = sample_chunk_count(n);
-    const int g1 = (int)(nchunks < (uint64_t)(8 * device_sms()) ? nchunks : (uint64_t)(8 * device_sms()));
+    const uint64_t own = bits < n && nchunks > 1 ? nchunks / 2 : nchunks;
+    const int g1 = (int)(own < (uint64_t)(8 * device_sms()) ? own : (uint64_t)(8 * device_sms()));
     const int g3 = (K + 7) / 8 < 4 * device_sms() ? (K + 7) / 8 : 4 * device_sms();
     if (c128)
-        k_sample_chunks<double><<<g1, 256, 0, st>>>((const double2 *)psi, n, d_sums);
+        k_sample_chunks<double><<<g1, 256, 0, st>>>((const double2 *)psi, n, bits, d_sums);
     else
-        k_sample_chunks<float><<<g1, 256, 0, st>>>((const float2 *)psi, n, d_sums);
+        k_sample_chunks<float><<<g1, 256, 0, st>>>((const float2 *)psi, n, bits, d_sums);
     k_sample_scan<<<1, 1024, 0, st>>>(d_sums, nchunks, d_total);
     if (c128)
-        k_sample_draw<double><<<g3, 256, 0, st>>>((const double2 *)psi, n, d_sums, d_total, K, d_u, d_x, d_cut, cost);
+        k_sample_draw<double><<<g3, 256, 0, st>>>((const double2 *)psi, n, bits, d_sums, d_total, K, d_u, d_x, d_cut, cost);
     else
-        k_sample_draw<float><<<g3, 256, 0, st>>>((const float2 *)psi, n, d_sums, d_total, K, d_u, d_x, d_cut, cost);
+        k_sample_draw<float><<<g3, 256, 0, st>>>((const float2 *)psi, n, bits, d_sums, d_total, K, d_u, d_x, d_cut, cost);
     return (int)cudaGetLastError();
 }
 
-int launch_untwist(bool c128, void *psi, int n, const double2 *cs, int p, int noshift, cudaStream_t st)
+int launch_untwist(bool c128, void *psi, int n, int bits, const double2 *cs, int p, int noshift, cudaStream_t st)
 {
     const int grid = 4 * device_sms();
     if (c128)
-        k_untwist<double><<<grid, 256, 0, st>>>((double2 *)psi, n, cs, p, noshift);
+        k_untwist<double><<<grid, 256, 0, st>>>((double2 *)psi, n, bits, cs, p, noshift);
     else
-        k_untwist<float><<<grid, 256, 0, st>>>((float2 *)psi, n, cs, p, noshift);
+        k_untwist<float><<<grid, 256, 0, st>>>((float2 *)psi, n, bits, cs, p, noshift);
     return (int)cudaGetLastError();
 }
 

@@ -520,45 +520,50 @@ static_assert(split_ok<Geo<float, 1>, 0>() && split_ok<Geo<float, 1>, 1>() && sp
                   split_ok<Geo<double, 2>, 0>() && split_ok<Geo<double, 2>, 1>() && split_ok<Geo<double, 2>, 2>(),
               "shared-memory index split");
 
+// sb2: the base of the registers with the top register bit set (a pair pass's
+// last stage reads them from the mirrored thread's place; sb otherwise)
 template <typename R, int NV, int ST>
-__device__ __forceinline__ void load_regs(const typename CT<R>::T *sv, uint32_t sb,
+__device__ __forceinline__ void load_regs(const typename CT<R>::T *sv, uint32_t sb, uint32_t sb2,
                                           typename CT<R>::T (&a)[1 << Geo<R, NV>::RB])
 {
     using G = Geo<R, NV>;
     constexpr int NR = 1 << G::RB;
     constexpr uint32_t LOW = split_low<G, ST>();
-    const uint32_t sbh = sb & ~LOW, sbl = sb & LOW;
+    const uint32_t bh[2] = {sb & ~LOW, sb2 & ~LOW}, bl[2] = {sb & LOW, sb2 & LOW};
     if constexpr (std::is_same<R, float>::value && G::reg(ST, 0) == 0) {
 #pragma unroll
         for (int m = 0; m < NR; m += 2) {
-            const float4 v = *reinterpret_cast<const float4 *>(&sv[smem_index<G, ST>(sbh, sbl, m)]);
+            const int h = 2 * m >= NR;
+            const float4 v = *reinterpret_cast<const float4 *>(&sv[smem_index<G, ST>(bh[h], bl[h], m)]);
             a[m] = make_float2(v.x, v.y);
             a[m + 1] = make_float2(v.z, v.w);
         }
     } else {
 #pragma unroll
         for (int m = 0; m < NR; m++)
-            a[m] = sv[smem_index<G, ST>(sbh, sbl, m)];
+            a[m] = sv[smem_index<G, ST>(bh[2 * m >= NR], bl[2 * m >= NR], m)];
     }
 }
 
 template <typename R, int NV, int ST>
-__device__ __forceinline__ void store_regs(typename CT<R>::T *sv, uint32_t sb,
+__device__ __forceinline__ void store_regs(typename CT<R>::T *sv, uint32_t sb, uint32_t sb2,
                                            const typename CT<R>::T (&a)[1 << Geo<R, NV>::RB])
 {
     using G = Geo<R, NV>;
     constexpr int NR = 1 << G::RB;
     constexpr uint32_t LOW = split_low<G, ST>();
-    const uint32_t sbh = sb & ~LOW, sbl = sb & LOW;
+    const uint32_t bh[2] = {sb & ~LOW, sb2 & ~LOW}, bl[2] = {sb & LOW, sb2 & LOW};
     if constexpr (std::is_same<R, float>::value && G::reg(ST, 0) == 0) {
 #pragma unroll
-        for (int m = 0; m < NR; m += 2)
-            *reinterpret_cast<float4 *>(&sv[smem_index<G, ST>(sbh, sbl, m)]) =
+        for (int m = 0; m < NR; m += 2) {
+            const int h = 2 * m >= NR;
+            *reinterpret_cast<float4 *>(&sv[smem_index<G, ST>(bh[h], bl[h], m)]) =
                 make_float4(a[m].x, a[m].y, a[m + 1].x, a[m + 1].y);
+        }
     } else {
 #pragma unroll
         for (int m = 0; m < NR; m++)
-            sv[smem_index<G, ST>(sbh, sbl, m)] = a[m];
+            sv[smem_index<G, ST>(bh[2 * m >= NR], bl[2 * m >= NR], m)] = a[m];
     }
 }
 
@@ -653,6 +658,11 @@ struct StageCtx {
     const float *qrf;  // the same as floats
     uint64_t fixed;
     int s, cb, tid;  // high qubit s and contiguous bits cb of this pass's tiles
+    // a pass over vertex n - 1 of a half state (k_pass): 0 no, 1 the number of
+    // stored index bits is odd, 2 it is even; the sign of that vertex's
+    // rotation for register 0 of this tile
+    int pair = 0;
+    R psign = (R)1;
     bool first;
     R tq;          // t of the rotation: tan beta, or -cot beta when |sin| > |cos|
     R f;           // factor dropped by one butterfly: cos beta or sin beta
@@ -695,75 +705,110 @@ struct StageCtx {
 // producer warp computes them per tile), the t-only sums on the thread only
 // (computed once per launch), Qr on the stage only. What is left per thread
 // and tile is a subset sum over the 2^RB register states.
-template <typename G, int ST, typename V>
-__device__ __forceinline__ void cut_terms(const V *tc, const V *pt, int tid, V &base, V (&d)[G::RB])
+//
+// In a pair pass (StageCtx::pair) the registers of the mirrored tile hold the
+// states with their other tile bits flipped: in the first stage that is a
+// whole thread (its top thread bit), in the last stage the half of the
+// registers with the top register bit. For those, register state r stands for
+// ~r, and O(~r) = O(all set) - sum_{k in r} d_k + Qr[~r]: the same subset sum
+// from another base with the opposite sign.
+template <typename G, int ST>
+__device__ __forceinline__ int logical_tid(int tid, int pair)
 {
     constexpr int NTB = G::T - G::RB;
+    const bool flip = ST != G::NST - 1 && pair && ((tid >> (NTB - 1)) & 1);
+    return flip ? tid ^ ((1 << (NTB - 1)) - 1) : tid;
+}
+template <typename G, int ST, typename V>
+__device__ __forceinline__ void cut_terms(const V *tc, const V *pt, int tid, int pair, V &base, V (&d)[G::RB])
+{
+    constexpr int NTB = G::T - G::RB;
+    const int tl = logical_tid<G, ST>(tid, pair);
     base = tc[15] + pt[0];
 #pragma unroll
     for (int j = 0; j < NTB; j++)
-        if ((tid >> j) & 1)
+        if ((tl >> j) & 1)
             base += tc[G::thr(ST, j)];
 #pragma unroll
     for (int k = 0; k < G::RB; k++)
         d[k] = tc[G::reg(ST, k)] + pt[(1 + k) * G::NTHR];
+    if (tl != tid)
+#pragma unroll
+        for (int k = 0; k < G::RB; k++) {
+            base += d[k];
+            d[k] = -d[k];
+        }
+}
+
+// v[m] = base + sum_{k in m} d_k over the register states
+template <typename G, int ST, typename V>
+__device__ __forceinline__ void subset_sums(V base, V (&d)[G::RB], int pair, V (&v)[1 << G::RB])
+{
+    constexpr int RB = G::RB, H = 1 << (RB - 1);
+    V base2 = base + d[RB - 1];
+    v[0] = base;
+#pragma unroll
+    for (int m = 1; m < H; m++) {
+        const int top = hibit(m);
+        v[m] = v[m ^ (1 << top)] + d[top];
+    }
+    if (ST == G::NST - 1 && pair)
+#pragma unroll
+        for (int k = 0; k < RB - 1; k++) {
+            base2 += d[k];
+            d[k] = -d[k];
+        }
+    v[H] = base2;
+#pragma unroll
+    for (int m = 1; m < H; m++) {
+        const int top = hibit(m);
+        v[H | m] = v[H | (m ^ (1 << top))] + d[top];
+    }
 }
 
 // integer cut values (phase-table indices)
 template <typename G, int ST>
-__device__ __forceinline__ void cut_int(const int *tc, const int *pt, const int *qr, bool qz, int tid,
+__device__ __forceinline__ void cut_int(const int *tc, const int *pt, const int *qr, bool qz, int tid, int pair,
                                         int (&v)[1 << G::RB])
 {
     constexpr int RB = G::RB;
     int base, d[RB];
-    cut_terms<G, ST>(tc, pt, tid, base, d);
-    v[0] = base;
+    cut_terms<G, ST>(tc, pt, tid, pair, base, d);
+    subset_sums<G, ST>(base, d, pair, v);
+    if (!qz) {  // a mirrored thread's register m is state ~m
+        const int f = logical_tid<G, ST>(tid, pair) != tid ? (1 << RB) - 1 : 0;
 #pragma unroll
-    for (int m = 1; m < (1 << RB); m++) {
-        const int top = hibit(m);
-        v[m] = v[m ^ (1 << top)] + d[top];
+        for (int m = 0; m < (1 << RB); m++)
+            v[m] += qr[m ^ f];
     }
-    if (!qz)
-#pragma unroll
-        for (int m = 1; m < (1 << RB); m++)
-            v[m] += qr[m];
 }
 
 // cut values as multipliers of type R (exact: integers below 2^24)
 template <typename G, typename R, int ST>
 __device__ __forceinline__ void cut_real(const int *tc, const int *pt, const int *qr, const float *qrf, bool qz,
-                                         int tid, R (&v)[1 << G::RB])
+                                         int tid, int pair, R (&v)[1 << G::RB])
 {
     constexpr int RB = G::RB;
     int base, d[RB];
-    cut_terms<G, ST>(tc, pt, tid, base, d);
+    cut_terms<G, ST>(tc, pt, tid, pair, base, d);
+    const int f = logical_tid<G, ST>(tid, pair) != tid ? (1 << RB) - 1 : 0;
     if constexpr (std::is_same<R, float>::value) {
         float df[RB];
 #pragma unroll
         for (int k = 0; k < RB; k++)
             df[k] = (float)d[k];
-        v[0] = (float)base;
-#pragma unroll
-        for (int m = 1; m < (1 << RB); m++) {
-            const int top = hibit(m);
-            v[m] = v[m ^ (1 << top)] + df[top];
-        }
+        subset_sums<G, ST>((float)base, df, pair, v);
         if (!qz)
 #pragma unroll
-            for (int m = 1; m < (1 << RB); m++)
-                v[m] += qrf[m];
+            for (int m = 0; m < (1 << RB); m++)
+                v[m] += qrf[m ^ f];
     } else {
         int iv[1 << RB];
-        iv[0] = base;
-#pragma unroll
-        for (int m = 1; m < (1 << RB); m++) {
-            const int top = hibit(m);
-            iv[m] = iv[m ^ (1 << top)] + d[top];
-        }
+        subset_sums<G, ST>(base, d, pair, iv);
         if (!qz)
 #pragma unroll
-            for (int m = 1; m < (1 << RB); m++)
-                iv[m] += qr[m];
+            for (int m = 0; m < (1 << RB); m++)
+                iv[m] += qr[m ^ f];
 #pragma unroll
         for (int m = 0; m < (1 << RB); m++)
             v[m] = (R)iv[m];
@@ -779,13 +824,8 @@ __device__ __forceinline__ void ising_vals(const R *tc, const R *pt, const R *q,
 {
     constexpr int RB = G::RB;
     R base, d[RB];
-    cut_terms<G, ST, R>(tc, pt, tid, base, d);
-    v[0] = base;
-#pragma unroll
-    for (int m = 1; m < (1 << RB); m++) {
-        const int top = hibit(m);
-        v[m] = v[m ^ (1 << top)] + d[top];
-    }
+    cut_terms<G, ST, R>(tc, pt, tid, 0, base, d);
+    subset_sums<G, ST, R>(base, d, 0, v);
     if (!qz)
 #pragma unroll
         for (int m = 1; m < (1 << RB); m++)
@@ -855,8 +895,64 @@ __host__ __device__ constexpr int first_owned(int st)
     return k;
 }
 
+// The rotation of vertex n - 1 on a half state, between the two tiles of a
+// pair pass. With x = (1, x') the stored amplitude is the one of y = ~x' (all
+// stored bits flipped), and the twisted amplitude of x is g = i^(1-m)
+// (-1)^|x'| times the stored one (m stored bits; i^(1+|x'|) against i^|y|).
+// Register r of the tile meets register ~r of the mirrored one, so
+//   (a, b) <- (a - t g b, b + t conj(g) a),
+// g real for odd m, imaginary for even m, its sign alternating with the bit
+// count of r (compile time) from X.psign (register 0, per thread and tile).
+// The pair's term of dE/dbeta likewise: g [Re(conj l_b a) - Re(conj l_a b)],
+// or sigma [Im(conj l_b a) + Im(conj l_a b)] with g = i sigma.
+template <typename R, int NV, bool PHI>
+__device__ __forceinline__ R mix_mirror(int pair, R t, typename CT<R>::T (&a)[1 << Geo<R, NV>::RB],
+                                        typename CT<R>::T (&l)[1 << Geo<R, NV>::RB])
+{
+    using C = typename CT<R>::T;
+    constexpr int H = 1 << (Geo<R, NV>::RB - 1);
+    if (pair == 1) {
+        C ipp[2], ipn[2];
+        ipp[0] = ipp[1] = ipn[0] = ipn[1] = mkc<C>((R)0, (R)0);
+#pragma unroll
+        for (int r = 0; r < H; r++) {
+            const int m1 = 2 * H - 1 - r;
+            const bool odd = ((r ^ (r >> 1) ^ (r >> 2) ^ (r >> 3)) & 1) != 0;
+            const R tt = odd ? -t : t;
+            if constexpr (NV == 2 && !PHI) {
+                dot_acc(odd ? ipn[r & 1] : ipp[r & 1], l[m1], a[r]);
+                dot_acc(odd ? ipp[r & 1] : ipn[r & 1], l[r], a[m1]);
+                rot(l[r], l[m1], tt);
+            }
+            rot(a[r], a[m1], tt);
+        }
+        return ((ipp[0].x + ipp[0].y) + (ipp[1].x + ipp[1].y)) - ((ipn[0].x + ipn[0].y) + (ipn[1].x + ipn[1].y));
+    }
+    auto turn = [](C &u, C &v, R s) {  // (u, v) <- (u - i s v, v - i s u)
+        const C u0 = u;
+        u.x = fma(s, v.y, u.x);
+        u.y = fma(-s, v.x, u.y);
+        v.x = fma(s, u0.y, v.x);
+        v.y = fma(-s, u0.x, v.y);
+    };
+    R q[2] = {0, 0};
+#pragma unroll
+    for (int r = 0; r < H; r++) {
+        const int m1 = 2 * H - 1 - r;
+        const bool odd = ((r ^ (r >> 1) ^ (r >> 2) ^ (r >> 3)) & 1) != 0;
+        const R tt = odd ? -t : t;
+        if constexpr (NV == 2 && !PHI) {
+            q[odd] = fma(l[m1].x, a[r].y, fma(-l[m1].y, a[r].x, q[odd]));
+            q[odd] = fma(l[r].x, a[m1].y, fma(-l[r].y, a[m1].x, q[odd]));
+            turn(l[r], l[m1], tt);
+        }
+        turn(a[r], a[m1], tt);
+    }
+    return q[0] - q[1];
+}
+
 template <typename R, int NV, int ST, bool COT, int DUE, bool PHI = false>
-__device__ __forceinline__ void mix_regs_form(const PassRegs &A, int cb, R tq, R f, R &run,
+__device__ __forceinline__ void mix_regs_form(const PassRegs &A, int cb, R tq, R f, R &run, int pair, R psign,
                                               typename CT<R>::T (&a)[1 << Geo<R, NV>::RB],
                                               typename CT<R>::T (&l)[1 << Geo<R, NV>::RB], Acc<R> &acc)
 {
@@ -877,6 +973,13 @@ __device__ __forceinline__ void mix_regs_form(const PassRegs &A, int cb, R tq, R
             due = A.is_low;
         if (!due)
             continue;
+        if (!COT && ST == G::NST - 1 && k == RB - 1 && pair) {  // vertex n - 1 of a half state
+            const R q = psign * mix_mirror<R, NV, PHI>(pair, psign * tq, a, l);
+            if constexpr (NV == 2 && !PHI)
+                gb = fma(q, sc * sc, gb);
+            sc *= f;
+            continue;
+        }
         C ipp[2], ipn[2];
         ipp[0] = ipp[1] = ipn[0] = ipn[1] = mkc<C>((R)0, (R)0);
 #pragma unroll
@@ -912,15 +1015,26 @@ __device__ __forceinline__ void mix_regs_form(const PassRegs &A, int cb, R tq, R
 // cot (Ising plans only, decided per layer) selects the butterfly form once
 // for the whole stage, outside the unrolled loops
 template <typename R, int NV, int ST, bool IS = false, int DUE = -1, bool PHI = false>
-__device__ __forceinline__ void mix_regs(const PassRegs &A, int cb, R tq, R f, R &run,
+__device__ __forceinline__ void mix_regs(const PassRegs &A, const StageCtx<R> &X, R tq, R f, R &run,
                                          typename CT<R>::T (&a)[1 << Geo<R, NV>::RB],
                                          typename CT<R>::T (&l)[1 << Geo<R, NV>::RB], Acc<R> &acc,
                                          bool cot = false)
 {
+    const int pair = IS ? 0 : X.pair;
     if (IS && cot)
-        mix_regs_form<R, NV, ST, true, DUE, PHI>(A, cb, tq, f, run, a, l, acc);
+        mix_regs_form<R, NV, ST, true, DUE, PHI>(A, X.cb, tq, f, run, 0, X.psign, a, l, acc);
     else
-        mix_regs_form<R, NV, ST, false, DUE, PHI>(A, cb, tq, f, run, a, l, acc);
+        mix_regs_form<R, NV, ST, false, DUE, PHI>(A, X.cb, tq, f, run, pair, X.psign, a, l, acc);
+}
+
+// The shared-memory base of a stage's registers with the top register bit:
+// in the last stage of a pair pass the mirrored thread's, else the thread's own.
+template <typename G, int ST>
+__device__ __forceinline__ uint32_t top_base(uint32_t base, int pair)
+{
+    if constexpr (ST == G::NST - 1)
+        return pair ? base ^ stage_base<G, ST>((1u << (G::T - G::RB)) - 1u) : base;
+    return base;
 }
 
 // One register stage of a pass over the tile(s) in sv0 (and sv1 for NV = 2).
@@ -939,8 +1053,9 @@ __device__ __forceinline__ void run_stage(const PassRegs &A, StageCtx<R> &X,
     constexpr int RB = G::RB, NR = 1 << RB, NTB = G::T - RB;
     constexpr bool LAST = (ST == G::NST - 1);
 
+    const int pair = IS ? 0 : X.pair;
     const uint32_t base = stage_base<G, ST>((uint32_t)X.tid);
-    const uint32_t sb = G::swz(base);
+    const uint32_t sb = G::swz(base), sb2 = G::swz(top_base<G, ST>(base, pair));
 
     // the stage a pass starts with: stage 0 of a low pass, or stage 1 of a
     // complex64 high pass (the generating pass of a forward sweep may be one)
@@ -948,7 +1063,12 @@ __device__ __forceinline__ void run_stage(const PassRegs &A, StageCtx<R> &X,
     if (MAY_START && X.first && !A.load) {  // |+>^n in the twisted frame: 2^(-n/2) i^|x|
         // the four values amp * i^((c0 + j) & 3) once, then a compile-time
         // choice by the register index's own bit count
-        const int c0 = (__popcll(X.fixed) + __popc(base)) & 3;
+        // (of the stored index: a pair pass's mirrored tile has the other
+        // fixed bits, and its tile bit T - 1 is no index bit)
+        int c0 = __popcll(X.fixed) + __popc(base);
+        if (ST == 1 && pair && (base >> (G::T - 1)))
+            c0 = (X.s - X.cb) - __popcll(X.fixed) + __popc(base) - 1;
+        c0 &= 3;
         const R amp = X.amp0;
         C zc[4];
 #pragma unroll
@@ -960,10 +1080,10 @@ __device__ __forceinline__ void run_stage(const PassRegs &A, StageCtx<R> &X,
         for (int m = 0; m < NR; m++)
             a[m] = zc[__popc(m) & 3];
     } else {
-        load_regs<R, NV, ST>(X.sv0, sb, a);
+        load_regs<R, NV, ST>(X.sv0, sb, sb2, a);
         if constexpr (NV == 2)  // lambda exists unless this pass forms it
             if (!(OPS && X.first && A.pre_lambda) && !(OPS && (A.post & POST_LAMBDA)))
-                load_regs<R, NV, ST>(X.sv1, sb, l);
+                load_regs<R, NV, ST>(X.sv1, sb, sb2, l);
     }
 
     // cut-function constants: function 0 is C (cost), 1 the observable O
@@ -975,7 +1095,8 @@ __device__ __forceinline__ void run_stage(const PassRegs &A, StageCtx<R> &X,
             ising_vals<G, R, ST>(X.tv + 16 * e, X.ptv + e * (RB + 1) * G::NTHR + X.tid, X.qv + 32 * e, X.qz[e], X.tid,
                                  v);
         else
-            cut_real<G, R, ST>(e ? tc1 : tc0, e ? pt1 : pt0, X.qr + 32 * e, X.qrf + 32 * e, X.qz[e], X.tid, v);
+            cut_real<G, R, ST>(e ? tc1 : tc0, e ? pt1 : pt0, X.qr + 32 * e, X.qrf + 32 * e, X.qz[e], X.tid, pair,
+                                v);
     };
     // the cost layer's phase factors of the thread's states (this pass's table)
     auto phases = [&](C (&P)[NR]) {
@@ -983,7 +1104,7 @@ __device__ __forceinline__ void run_stage(const PassRegs &A, StageCtx<R> &X,
             ising_phases<G, C, ST>(X.tp, X.ptp + X.tid, X.qp, X.qz[0], X.tid, P);
         } else {
             int cv[NR];
-            cut_int<G, ST>(tc0, pt0, X.qr, X.qz[0], X.tid, cv);
+            cut_int<G, ST>(tc0, pt0, X.qr, X.qz[0], X.tid, pair, cv);
 #pragma unroll
             for (int m = 0; m < NR; m++)
                 P[m] = X.tab[cv[m]];
@@ -1008,9 +1129,9 @@ __device__ __forceinline__ void run_stage(const PassRegs &A, StageCtx<R> &X,
     }
 
     if (NV == 2 && OPS && (A.post & POST_LAMBDA))  // phi alone (lambda is formed below)
-        mix_regs<R, NV, ST, IS, DUE, true>(A, X.cb, X.tq, X.f, X.run, a, l, acc0, X.cot);
+        mix_regs<R, NV, ST, IS, DUE, true>(A, X, X.tq, X.f, X.run, a, l, acc0, X.cot);
     else
-        mix_regs<R, NV, ST, IS, DUE>(A, X.cb, X.tq, X.f, X.run, a, l, acc0, X.cot);
+        mix_regs<R, NV, ST, IS, DUE>(A, X, X.tq, X.f, X.run, a, l, acc0, X.cot);
 
     if (OPS && LAST && (A.post & POST_RESCALE)) {  // the stored state is the exact one
 #pragma unroll
@@ -1076,12 +1197,12 @@ __device__ __forceinline__ void run_stage(const PassRegs &A, StageCtx<R> &X,
         }
     }
     if constexpr (FUSE && LAST)
-        mix_regs<R, NV, ST, IS, DUE>(A, X.cb, X.tq2, X.f2, X.run2, a, l, acc2, X.cot2);
+        mix_regs<R, NV, ST, IS, DUE>(A, X, X.tq2, X.f2, X.run2, a, l, acc2, X.cot2);
     if (!LAST || A.write) {
-        store_regs<R, NV, ST>(X.sv0, sb, a);
+        store_regs<R, NV, ST>(X.sv0, sb, sb2, a);
         if constexpr (NV == 2)
             if (LAST || !(OPS && (A.post & POST_LAMBDA)))  // lambda exists from the last stage on
-                store_regs<R, NV, ST>(X.sv1, sb, l);
+                store_regs<R, NV, ST>(X.sv1, sb, sb2, l);
     }
 }
 
@@ -1094,14 +1215,15 @@ __device__ __forceinline__ void mix_stage(const PassRegs &A, StageCtx<R> &X,
     using G = Geo<R, NV>;
     const uint32_t base = stage_base<G, ST>((uint32_t)X.tid);
     const uint32_t sb = G::swz(base);
-    load_regs<R, NV, ST>(X.sv0, sb, a);
+    static_assert(ST != G::NST - 1, "a fused pass comes back to its first stage");
+    load_regs<R, NV, ST>(X.sv0, sb, sb, a);
     if constexpr (NV == 2)
-        load_regs<R, NV, ST>(X.sv1, sb, l);
-    mix_regs<R, NV, ST, IS, DUE>(A, X.cb, X.tq2, X.f2, X.run2, a, l, acc2, X.cot2);
+        load_regs<R, NV, ST>(X.sv1, sb, sb, l);
+    mix_regs<R, NV, ST, IS, DUE>(A, X, X.tq2, X.f2, X.run2, a, l, acc2, X.cot2);
     if (!(turn_keeps_phi<R> && NV == 2 && (A.post & POST_LAMBDA)))  // the turnaround keeps the loaded phi
-        store_regs<R, NV, ST>(X.sv0, sb, a);
+        store_regs<R, NV, ST>(X.sv0, sb, sb, a);
     if constexpr (NV == 2)
-        store_regs<R, NV, ST>(X.sv1, sb, l);
+        store_regs<R, NV, ST>(X.sv1, sb, sb, l);
 }
 
 // Which owned bits of stage st a pass with this shape transforms: 0 every
@@ -1277,6 +1399,21 @@ constexpr int FW_TURN = flag_word(1, 0, 0, 1, POST_REDUCE | POST_RESCALE | POST_
 // the register stages. Per stage buffer s two mbarriers hand the buffer over:
 // full[s] (producer -> compute: tile loaded, or buffer free in a generating
 // pass) and done[s] (compute -> producer: results in shared memory).
+//
+// A MaxCut state does not change when all bits flip (the cut function and the
+// mixer commute with X^n and |+>^n is its eigenvector): psi(x) = psi(~x). Its
+// passes keep the half with vertex n - 1 on side 0, 2^(n-1) amplitudes, and
+// every sum over the state is twice the half's (the host's slot scales). All
+// bits but one are then ordinary index bits; the rotation of vertex n - 1
+// joins y with ~y. The pass whose tiles span that vertex (A.pair, a high pass
+// whose top tile bit it is) takes the tile with fixed bits f and the mirrored
+// tile ~f, half a tile each, as the two values of that bit: the mirrored
+// tile's other bits run backwards, which only the last stage (that bit is its
+// top register bit) and cut values notice. Ising plans keep the whole state.
+// The passes are bound by memory or by issue, both proportional to the
+// amplitudes, so half of them is half the time: n = 30, p = 2 complex64
+// gradient 47.6 -> 24.7 ms, n = 24, p = 3 complex128 gradient 21.8 -> 11.3 ms,
+// 4096 energies at n = 20 18.4 -> 10.5 ms.
 // MODE 0: mixer only; 1: with cut-function work on one graph; 2: the same
 // with point b of the batch being its own graph (A.pt[b]); 3: as 1, and the
 // pass is fused (A.fuse): after the last stage's operations the mixer of
@@ -1327,7 +1464,12 @@ __global__ void __maxnreg__((Geo<R, NV>::MAXREG))
     // tile = 2^cb contiguous amplitudes x 2^(T-cb) rows along qubits s..
     const int cb = A.cb, hb = G::T - A.cb;
     const int midbits = A.s - cb;
-    const unsigned tiles_per_hi = (unsigned)A.tiles >> midbits;  // 2^(n - s - hb)
+    const int pair = IS ? 0 : A.pair;
+    // stored index: high bits | mid bits | row qubits | mid bits; a pair pass
+    // has no bits above its rows and half the mid values (the other half are
+    // the mirrored tiles)
+    const unsigned tiles_per_hi = pair ? 1u : (unsigned)A.tiles >> midbits;
+    const unsigned midmask = (1u << midbits) - 1u;
     const bool reduce = A.slot_idx[0] >= 0 || A.slot_idx[1] >= 0 || A.slot_idx[2] >= 0;
 
     if (tid == 0) {
@@ -1406,24 +1548,27 @@ __global__ void __maxnreg__((Geo<R, NV>::MAXREG))
             const int st = est[e];
             if (st < 0)
                 continue;
+            const int tl = st == 1 ? logical_tid<G, 1>(tid, pair) : tid;
             int q = 0;
             for (int j = 0; j < NTB; j++)
                 for (int j2 = 0; j2 < j; j2++)
-                    if (((tid >> j) & 1) && ((tid >> j2) & 1))
+                    if (((tl >> j) & 1) && ((tl >> j2) & 1))
                         q -= 2 * wgt(e, gq(G::thr(st, j)), gq(G::thr(st, j2)));
             ptc[(e * (RB + 1)) * NTHR + tid] = q;
             for (int kk = 0; kk < RB; kk++) {
                 int dk = 0;
                 for (int j = 0; j < NTB; j++)
-                    if ((tid >> j) & 1)
+                    if ((tl >> j) & 1)
                         dk -= 2 * wgt(e, gq(G::reg(st, kk)), gq(G::thr(st, j)));
                 ptc[(e * (RB + 1) + 1 + kk) * NTHR + tid] = dk;
             }
             if (tid < (1 << RB)) {
+                // the state of register tid: flipped in the mirrored half of the last stage
+                const int rm = pair && st == G::NST - 1 && (tid >> (RB - 1)) ? tid ^ ((1 << (RB - 1)) - 1) : tid;
                 int qq = 0;
                 for (int kk = 0; kk < RB; kk++)
                     for (int k2 = 0; k2 < kk; k2++)
-                        if (((tid >> kk) & 1) && ((tid >> k2) & 1))
+                        if (((rm >> kk) & 1) && ((rm >> k2) & 1))
                             qq -= 2 * wgt(e, gq(G::reg(st, kk)), gq(G::reg(st, k2)));
                 qr[qs][e][tid] = qq;
                 qrf[qs][e][tid] = (float)qq;
@@ -1495,7 +1640,7 @@ __global__ void __maxnreg__((Geo<R, NV>::MAXREG))
         const unsigned g = cta_tile(blockIdx.x, k, grid, (unsigned)A.chunk);
         b = g >> tiles_log2;
         t = g & ((unsigned)A.tiles - 1u);
-        mid = t & ((1u << midbits) - 1u);
+        mid = t & midmask;
         const unsigned hi = t >> midbits;
         c4 = (int)(hi + b * tiles_per_hi);
     };
@@ -1630,6 +1775,12 @@ __global__ void __maxnreg__((Geo<R, NV>::MAXREG))
                 tma_load_5d(buf, &map0, &full[s], 0, c1, c2, 0, c4);
                 if (A.nvec_io == 2)
                     tma_load_5d(buf + TB, &map1, &full[s], 0, c1, c2, 0, c4);
+                if (pair) {  // the mirrored tile (boxes of half a tile; rows are wide here)
+                    const int cm = (int)(~mid & midmask);
+                    tma_load_5d(buf + TB / 2, &map0, &full[s], 0, 0, cm, 0, c4);
+                    if (A.nvec_io == 2)
+                        tma_load_5d(buf + TB + TB / 2, &map1, &full[s], 0, 0, cm, 0, c4);
+                }
             } else {
                 mbar_arrive(&full[s]);  // generating pass: the buffer is free
             }
@@ -1651,6 +1802,13 @@ __global__ void __maxnreg__((Geo<R, NV>::MAXREG))
                         tma_store_5d(&map0, buf, 0, c1, c2, 0, c4);
                     if (NV == 2)
                         tma_store_5d(&map1, buf + TB, 0, c1, c2, 0, c4);
+                    if (pair) {
+                        const int cm = (int)(~mid & midmask);
+                        if (!(turn_keeps_phi<R> && NV == 2 && (A.post & POST_LAMBDA)))
+                            tma_store_5d(&map0, buf + TB / 2, 0, 0, cm, 0, c4);
+                        if (NV == 2)
+                            tma_store_5d(&map1, buf + TB + TB / 2, 0, 0, cm, 0, c4);
+                    }
                     asm volatile("cp.async.bulk.commit_group;" ::: "memory");
                     if (k + NS < niter)  // the buffer is reloaded: its store must have read it
                         asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
@@ -1707,6 +1865,9 @@ __global__ void __maxnreg__((Geo<R, NV>::MAXREG))
             X.tid = tid;
             X.amp0 = (R)A.amp0;
             X.first = true;
+            X.pair = pair ? ((A.n - 1) & 1 ? 1 : 2) : 0;
+            // bit count parity of this thread's last-stage bits, and of i^(1-m)
+            const int ppar = __popc(stage_base<G, G::NST - 1>((uint32_t)tid)) + ((A.n - 1) >> 1);
 
             // A point change costs no extra barrier. The phase table has two
             // slots (the one being replaced was last read before the previous
@@ -1836,6 +1997,8 @@ __global__ void __maxnreg__((Geo<R, NV>::MAXREG))
                 X.tv = &tvs[IS ? s : 0][0][0];
                 X.tp = &tps[IS ? s : 0][0];
                 X.fixed = ((uint64_t)mid << cb) | ((uint64_t)(t >> midbits) << (A.s + hb));
+                if (!IS)
+                    X.psign = ((ppar + __popc(mid)) & 1) ? (R)-1 : (R)1;
 
                 // No barrier between tiles unless a point starts: a warp may begin
                 // this tile while others still store the previous one. The first
