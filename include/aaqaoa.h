@@ -434,6 +434,9 @@ int aaqaoa_inject_fault(aaqaoa_plan *plan, int kind);
  *   high pass fewer (n = 30: 14 + 8 + 8 instead of 8 + 8 + 7 + 7). A batch of
  *   B points runs that pass once per point.
  *   INVALID_ARG if an (L, K) does not tile n with rows of >= 128 bytes.
+ *   MaxCut energies and gradients of up to 20 qubits run as one whole-circuit
+ *   launch where that is faster; a plan set here (any non-zero entry), like
+ *   layer fusion switched off, makes them run the tiled passes.
  *   Rebuilds the workspace's tensor maps; the stored state becomes invalid.
  * aaqaoa_autotune: times each candidate (the fewest and one more high pass,
  *   each with the full and the two-stage low pass, and for the complex64
@@ -466,7 +469,8 @@ int aaqaoa_set_layer_fusion(aaqaoa_plan *plan, int enable);
 int aaqaoa_get_layer_fusion(aaqaoa_plan *plan, int *enable);
 
 /*
- * aaqaoa_get_schedule -- the tiled passes one sweep launches, in order, as
+ * aaqaoa_get_schedule -- the tiled passes of one sweep, in order (for calls that
+ * run the passes, see aaqaoa_set_pass_plan), as
  * 5 ints each (host, row-major [cap][5]): the pass's first qubit s, its
  * qubit count, the layer l whose mixer it applies there, the second layer of
  * a fused pass or -1, and the number of layer l's qubits mixed by earlier

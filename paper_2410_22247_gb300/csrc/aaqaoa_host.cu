@@ -97,7 +97,7 @@ struct Pass {
 };
 
 struct Layout {
-    size_t ctrl, out, params, cs, tab, partials, zz, samp, ising, phi, lam, total;
+    size_t ctrl, fns, out, params, cs, tab, partials, zz, samp, ising, phi, lam, total;
     size_t partial_count;
 };
 
@@ -162,11 +162,13 @@ struct aaqaoa_plan {
     double state_bytes() const { return (double)((size_t)1 << n) * (double)amp(); }
     double sym() const { return half() ? 2.0 : 1.0; }  // what a sum over the stored amplitudes counts
     int tiles() const { return small() ? 1 : 1 << (bits() - T()); }
+    bool forced = false;  // the caller set the pass plan (aaqaoa_set_pass_plan)
     bool fuse = true;  // fuse layer boundaries into one pass where the plan allows
     int *err_shared = nullptr;  // set when the plan is part of a multi-graph batch
     const GraphFns *pt_dev = nullptr;  // set for a group of same-n graphs: point b is graph b
     int *d_err() const { return err_shared ? err_shared : reinterpret_cast<int *>(ws + L.ctrl); }
     unsigned *d_counter_pass() const { return reinterpret_cast<unsigned *>(ws + L.ctrl + 8); }
+    unsigned *d_team_bar() const { return reinterpret_cast<unsigned *>(ws + L.ctrl + 256); }
     unsigned *d_counter_agg() const { return reinterpret_cast<unsigned *>(ws + L.ctrl + 16); }
     double *d_out() const { return reinterpret_cast<double *>(ws + L.out); }
     double *d_params() const { return reinterpret_cast<double *>(ws + L.params); }
@@ -232,13 +234,17 @@ int pass_flags(const PassArgs &a)
     return ((a.pre_phase || a.pre_lambda || a.post) ? 1 : 0) | (a.fuse ? 2 : 0) | ((a.post & POST_LAMBDA) ? 8 : 0);
 }
 
+constexpr size_t CTRL_BYTES = 256 + 4 * CIRCUIT_MAX_POINTS;
+
 Layout layout(const aaqaoa_plan *pl, int batch, bool grad)
 {
     Layout L{};
     size_t off = 0;
     const size_t B = (size_t)batch;
-    L.ctrl = off;
-    off += 256;
+    L.ctrl = off;  // error flag, counters | team counters of the whole-circuit kernel
+    off += CTRL_BYTES;
+    L.fns = off;  // the plan's cut functions
+    off = align256(off + sizeof(GraphFns));
     L.out = off;
     off = align256(off + B * pl->out_stride() * sizeof(double));
     L.params = off;
@@ -848,12 +854,77 @@ int enqueue_aggregate(aaqaoa_plan *pl, int obs, int agg)
     return AAQAOA_OK;
 }
 
+// Whether a call runs as one whole-circuit launch (aaqaoa_circuit.cu): MaxCut
+// plans whose state fits its CTAs; a forced pass plan or fusion setting, a
+// pending test fault and a stored state beyond one CTA need the passes.
+bool use_circuit(const aaqaoa_plan *pl, int B, bool grad, bool state, CircuitPlan *q)
+{
+    if (pl->ising || pl->pt_dev || !circuit_plan(pl->c128, grad, pl->n, pl->p, pl->tab_len(), B, q))
+        return false;
+    if (pl->small())
+        return true;
+    if (pl->forced || !pl->fuse || pl->inject || state)
+        return false;
+    return q->cluster || ((size_t)B * (grad ? 1 + 2 * pl->p : 1) << q->c) <= pl->L.partial_count;
+}
+
+// the plan's and the shape's part of the arguments
+CircuitArgs circuit_args(const aaqaoa_plan *pl, int B, const CircuitPlan &q)
+{
+    CircuitArgs a;
+    memset(&a, 0, sizeof a);
+    a.n = pl->n;
+    a.p = pl->p;
+    a.tab_len = pl->tab_len();
+    a.B = B;
+    a.c = q.c;
+    a.Tl = q.Tl;
+    a.a = q.a;
+    a.km = q.km;
+    a.resident = q.resident;
+    a.amp0 = std::pow(2.0, -0.5 * pl->n);
+    return a;
+}
+
+int enqueue_circuit(aaqaoa_plan *pl, int B, const double *d_gamma, const double *d_beta, int obs, bool grad, bool state,
+                    const CircuitPlan &q)
+{
+    (void)cudaGetLastError();
+    CircuitArgs a = circuit_args(pl, B, q);
+    a.gamma = d_gamma;
+    a.beta = d_beta;
+    a.out = pl->d_out();
+    a.out_stride = pl->out_stride();
+    a.state = state ? pl->d_phi() : nullptr;
+    a.phi = pl->d_phi();
+    a.lam = pl->d_lam();
+    a.partials = pl->d_partials();
+    a.bar = pl->d_team_bar();
+    a.err = pl->d_err();
+    a.fns = reinterpret_cast<const GraphFns *>(pl->ws + pl->L.fns);
+    a.obs = obs;
+    ProfScope ps_(pl, PK_SMALL, state ? (double)B * pl->state_bytes() : 0.0);
+    CKL(launch_circuit(pl->c128, grad, a, q, pl->stream), "whole-circuit kernel");
+    pl->launches++;
+    return AAQAOA_OK;
+}
+
 int enqueue_expect(aaqaoa_plan *pl, int B, const double *d_gamma, const double *d_beta, int obs, int agg)
 {
+    const bool materialise = agg != AAQAOA_AGG_FUSED;
+    CircuitPlan q;
+    if (use_circuit(pl, B, false, materialise, &q)) {
+        if (!pl->small())
+            pl->state_valid = false;  // the exchange buffers are the stored state's
+        int r = enqueue_circuit(pl, B, d_gamma, d_beta, obs, false, materialise, q);
+        if (r || !materialise)
+            return r;
+        pl->state_valid = true;
+        return enqueue_aggregate(pl, obs, agg);
+    }
     int r = enqueue_params(pl, B, d_gamma, d_beta);
     if (r)
         return r;
-    const bool materialise = agg != AAQAOA_AGG_FUSED;
     if (pl->small()) {
         SmallArgs s = small_args(pl, obs, SMALL_ENERGY, materialise ? 1 : 0);
         ProfScope ps_(pl, PK_SMALL, materialise ? (double)B * (double)((size_t)1 << pl->n) * (double)pl->amp() : 0.0);
@@ -872,9 +943,35 @@ int enqueue_expect(aaqaoa_plan *pl, int B, const double *d_gamma, const double *
     return AAQAOA_OK;
 }
 
+// the final state in phi: the whole one for small plans, else the passes'
+// stored form; parameters at d_params()
+int enqueue_state(aaqaoa_plan *pl)
+{
+    const double *dg = pl->d_params(), *db = dg + pl->p;
+    CircuitPlan q;
+    if (pl->small() && use_circuit(pl, 1, false, true, &q))
+        return enqueue_circuit(pl, 1, dg, db, AAQAOA_OBS_FULL, false, true, q);
+    int r = enqueue_params(pl, 1, dg, db);
+    if (r)
+        return r;
+    if (pl->small()) {
+        SmallArgs s = small_args(pl, AAQAOA_OBS_FULL, SMALL_ENERGY, 1);
+        CKL(launch_small(pl->c128, s, 1, pl->stream), "whole-circuit kernel");
+        pl->launches++;
+        return AAQAOA_OK;
+    }
+    return enqueue_forward(pl, 1, AAQAOA_OBS_FULL, FWD_STATE);
+}
+
 // energy and gradient of B points (rows of d_out)
 int enqueue_grad(aaqaoa_plan *pl, const double *d_gamma, const double *d_beta, int obs, int B = 1)
 {
+    CircuitPlan q;
+    if (use_circuit(pl, B, true, false, &q)) {
+        if (!pl->small())
+            pl->state_valid = false;
+        return enqueue_circuit(pl, B, d_gamma, d_beta, obs, true, false, q);
+    }
     int r = enqueue_params(pl, B, d_gamma, d_beta);
     if (r)
         return r;
@@ -902,7 +999,7 @@ int fetch_out(aaqaoa_plan *pl, int B, std::vector<double> &rows)
     CK(cudaMemcpyAsync(rows.data(), pl->d_out(), nout * sizeof(double), cudaMemcpyDeviceToHost, pl->stream));
     CK(cudaStreamSynchronize(pl->stream));
     if (err) {
-        cudaMemsetAsync(pl->ws + pl->L.ctrl, 0, 256, pl->stream);
+        cudaMemsetAsync(pl->ws + pl->L.ctrl, 0, CTRL_BYTES, pl->stream);
         cudaStreamSynchronize(pl->stream);
         return fail(AAQAOA_ERR_TIMEOUT, "a bounded device wait expired (TMA tile never arrived)");
     }
@@ -1292,7 +1389,9 @@ int aaqaoa_set_workspace(aaqaoa_plan *pl, void *device_ptr, size_t bytes, int ba
     int r = build_maps(pl);
     if (r)
         return r;
-    CK(cudaMemsetAsync(pl->ws + L.ctrl, 0, 256, pl->stream));
+    CK(cudaMemsetAsync(pl->ws + L.ctrl, 0, CTRL_BYTES, pl->stream));
+    const GraphFns fns{pl->cost, {pl->obs[0], pl->obs[1]}};
+    CK(cudaMemcpyAsync(pl->ws + L.fns, &fns, sizeof fns, cudaMemcpyHostToDevice, pl->stream));
     if (pl->ising)
         CK(cudaMemcpyAsync(pl->ws + L.ising, pl->ifn.data(), pl->ifn.size() * sizeof(IsingFn), cudaMemcpyHostToDevice,
                            pl->stream));
@@ -1347,7 +1446,10 @@ int aaqaoa_set_pass_plan(aaqaoa_plan *pl, int fwd_low, int fwd_high, int bwd_low
     if (fwd_low < 0 || fwd_high < 0 || bwd_low < 0 || bwd_high < 0)
         return fail(AAQAOA_ERR_INVALID_ARG, "negative pass-plan entry");
     const int plan4[4] = {fwd_low, fwd_high, bwd_low, bwd_high};
-    return set_layers(pl, plan4);
+    const int r = set_layers(pl, plan4);
+    if (!r)
+        pl->forced = fwd_low || fwd_high || bwd_low || bwd_high;
+    return r;
 }
 
 int aaqaoa_set_layer_fusion(aaqaoa_plan *pl, int enable)
@@ -1708,15 +1810,9 @@ int aaqaoa_statevector(aaqaoa_plan *pl, const double *gamma, const double *beta,
     pl->launches = 0;
     if ((r = upload_params(pl, 1, gamma, beta)))
         return r;
-    if ((r = enqueue_params(pl, 1, pl->d_params(), pl->d_params() + pl->p)))
+    if ((r = enqueue_state(pl)))
         return r;
-    if (pl->small()) {
-        SmallArgs s = small_args(pl, AAQAOA_OBS_FULL, SMALL_ENERGY, 1);
-        CKL(launch_small(pl->c128, s, 1, pl->stream), "whole-circuit kernel");
-        pl->launches++;
-    } else {
-        if ((r = enqueue_forward(pl, 1, AAQAOA_OBS_FULL, FWD_STATE)))
-            return r;
+    if (!pl->small()) {
         // the passes store the twisted, shifted-angle state: map it back
         CKL(launch_untwist(pl->c128, pl->d_phi(), pl->n, pl->bits(), pl->d_cs(), pl->p, pl->ising ? 1 : 0, pl->stream),
             "statevector export");
@@ -1741,15 +1837,8 @@ int aaqaoa_edge_zz(aaqaoa_plan *pl, const double *gamma, const double *beta, dou
     pl->launches = 0;
     if ((r = upload_params(pl, 1, gamma, beta)))
         return r;
-    if ((r = enqueue_params(pl, 1, pl->d_params(), pl->d_params() + pl->p)))
+    if ((r = enqueue_state(pl)))
         return r;
-    if (pl->small()) {
-        SmallArgs s = small_args(pl, AAQAOA_OBS_FULL, SMALL_ENERGY, 1);
-        CKL(launch_small(pl->c128, s, 1, pl->stream), "whole-circuit kernel");
-        pl->launches++;
-    } else if ((r = enqueue_forward(pl, 1, AAQAOA_OBS_FULL, FWD_STATE))) {
-        return r;
-    }
     pl->state_valid = true;
     const int grid = pl->n < 10 ? 1 : agg_grid(pl->c128);
     for (int t0 = 0; t0 < pl->m; t0 += 64) {
@@ -1847,15 +1936,8 @@ int aaqaoa_sample(aaqaoa_plan *pl, const double *gamma, const double *beta, int 
     pl->launches = 0;
     if ((r = upload_params(pl, 1, gamma, beta)))
         return r;
-    if ((r = enqueue_params(pl, 1, pl->d_params(), pl->d_params() + pl->p)))
+    if ((r = enqueue_state(pl)))
         return r;
-    if (pl->small()) {
-        SmallArgs s = small_args(pl, AAQAOA_OBS_FULL, SMALL_ENERGY, 1);
-        CKL(launch_small(pl->c128, s, 1, pl->stream), "whole-circuit kernel");
-        pl->launches++;
-    } else if ((r = enqueue_forward(pl, 1, AAQAOA_OBS_FULL, FWD_STATE))) {
-        return r;
-    }
     pl->state_valid = true;
     CK(cudaMemcpyAsync(pl->d_samp_u(), u, (size_t)K * sizeof(double), cudaMemcpyHostToDevice, pl->stream));
     CKL(launch_sample(pl->c128, pl->d_phi(), pl->n, pl->bits(), pl->d_samp_sums(), pl->d_samp_total(), K, pl->d_samp_u(),
@@ -2097,6 +2179,24 @@ extern "C" int aaqaoa_expect_static(aaqaoa_plan *pl, const double *gamma, const 
     CK(cudaMemsetAsync(d_out, 0, (size_t)pl->out_stride() * sizeof(double), st));
     CK(cudaMemcpyAsync(d_par, gamma, (size_t)p * sizeof(double), cudaMemcpyHostToDevice, st));
     CK(cudaMemcpyAsync(d_par + p, beta, (size_t)p * sizeof(double), cudaMemcpyHostToDevice, st));
+    CircuitPlan q;
+    if (pl->small() && use_circuit(pl, 1, false, false, &q)) {
+        GraphFns *d_fns = reinterpret_cast<GraphFns *>(d_phi);  // no state is stored
+        const GraphFns fns{pl->cost, {pl->obs[0], pl->obs[1]}};
+        CK(cudaMemcpyAsync(d_fns, &fns, sizeof fns, cudaMemcpyHostToDevice, st));
+        CircuitArgs a = circuit_args(pl, 1, q);  // a small plan's CTAs need no exchange buffers
+        a.gamma = d_par;
+        a.beta = d_par + p;
+        a.out = d_out;
+        a.out_stride = pl->out_stride();
+        a.err = d_err;
+        a.fns = d_fns;
+        a.obs = observable;
+        CKL(launch_circuit(pl->c128, false, a, q, st), "whole-circuit kernel");
+        CK(cudaMemcpyAsync(energy, d_out, sizeof(double), cudaMemcpyDeviceToHost, st));
+        CK(cudaStreamSynchronize(st));
+        return AAQAOA_OK;
+    }
     CKL(launch_params(pl->c128, 1, p, pl->tab_len(), pl->n, d_par, d_par + p, d_tab, d_cs, st), "parameter tables");
 
     if (pl->small()) {

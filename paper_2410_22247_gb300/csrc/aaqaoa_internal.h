@@ -135,6 +135,33 @@ struct SmallArgs {
     const double *gam;     // [B][p]
 };
 
+// Whole MaxCut circuit in one launch (aaqaoa_circuit.cu).
+struct CircuitArgs {
+    int n, p, tab_len, B;
+    int c, Tl, a, km;    // CTAs per point 2^c, local bits, low bits of the high layout, bits per stage
+    int resident;        // the phase tables of all layers fit shared memory
+    double amp0;         // 2^(-n/2)
+    const double *gamma, *beta;  // [B][p]
+    double *out;         // [B][out_stride]
+    int out_stride;
+    void *state;         // also store psi_p, [B][2^n] (or null; not with exchange buffers)
+    void *phi, *lam;     // c > 0: exchange buffers, 2^n amplitudes per point (two states' halves)
+    double *partials;    // c > 0: [B][rows][2^c]
+    unsigned *bar;       // c > 0: one arrival counter per point, zero between launches
+    int *err;
+    const GraphFns *fns; // the graph's cut functions (device memory)
+    int obs;
+};
+// the kernel's shape for a call, from circuit_plan (false: the call does not fit it)
+struct CircuitPlan {
+    int c, Tl, a, km, nt, teams, resident;
+    int cluster;         // the 2^c CTAs are a cluster; else they exchange through global memory
+    size_t smem;
+};
+constexpr int CIRCUIT_MAX_POINTS = 64;  // points of one launch when c > 0 (arrival counters)
+bool circuit_plan(bool c128, bool grad, int n, int p, int tab_len, int B, CircuitPlan *q);
+int launch_circuit(bool c128, bool grad, const CircuitArgs &a, const CircuitPlan &q, cudaStream_t st);
+
 // Device descriptor of one small graph in an uneven batch (whole circuit in
 // one CTA): cost masks, and the masks and weights of both observables
 // (index 0 = H_C, 1 = H_red).

@@ -905,12 +905,12 @@ __host__ __device__ constexpr int first_owned(int st)
 // count of r (compile time) from X.psign (register 0, per thread and tile).
 // The pair's term of dE/dbeta likewise: g [Re(conj l_b a) - Re(conj l_a b)],
 // or sigma [Im(conj l_b a) + Im(conj l_a b)] with g = i sigma.
-template <typename R, int NV, bool PHI>
-__device__ __forceinline__ R mix_mirror(int pair, R t, typename CT<R>::T (&a)[1 << Geo<R, NV>::RB],
-                                        typename CT<R>::T (&l)[1 << Geo<R, NV>::RB])
+template <typename R, int NV, int RB, bool PHI>
+__device__ __forceinline__ R mix_mirror(int pair, R t, typename CT<R>::T (&a)[1 << RB],
+                                        typename CT<R>::T (&l)[1 << RB])
 {
     using C = typename CT<R>::T;
-    constexpr int H = 1 << (Geo<R, NV>::RB - 1);
+    constexpr int H = 1 << (RB - 1);
     if (pair == 1) {
         C ipp[2], ipn[2];
         ipp[0] = ipp[1] = ipn[0] = ipn[1] = mkc<C>((R)0, (R)0);
@@ -974,7 +974,7 @@ __device__ __forceinline__ void mix_regs_form(const PassRegs &A, int cb, R tq, R
         if (!due)
             continue;
         if (!COT && ST == G::NST - 1 && k == RB - 1 && pair) {  // vertex n - 1 of a half state
-            const R q = psign * mix_mirror<R, NV, PHI>(pair, psign * tq, a, l);
+            const R q = psign * mix_mirror<R, NV, RB, PHI>(pair, psign * tq, a, l);
             if constexpr (NV == 2 && !PHI)
                 gb = fma(q, sc * sc, gb);
             sc *= f;

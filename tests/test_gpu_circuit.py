@@ -1,0 +1,99 @@
+"""Whole circuits in one launch, and the flip-symmetric half of the passes, at
+the sizes where their shapes change: one CTA up to a team of 128, odd and even
+numbers of stored index bits, the first and last sizes of a register stage,
+more points than CTAs at once, phase tables that do not fit, pair passes over
+one qubit and over the most. Oracle: the plain FP64 statevector code;
+tolerances as in test_gpu_parity (complex128 1e-10, complex64 1e-5, gradients
+on the energy's scale).
+"""
+import numpy as np
+import pytest
+
+from oracle import oracle as O
+from paper_2410_22247_gb300 import workloads as W
+from paper_2410_22247_gb300 import orbits as ORB
+
+pytestmark = pytest.mark.gpu
+
+TOL = {"c64": 1e-5, "c128": 1e-10}
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _cuda():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+
+
+def _plan(n, e, p, prec, **kw):
+    from paper_2410_22247_gb300.api import Plan
+    return Plan(n, e, p, orbits=ORB.edge_orbits(n, e, weights=kw.get("weights")), precision=prec, **kw)
+
+
+def _check(got, ref, prec):
+    E, dg, db = got
+    Er, dgr, dbr = ref
+    scale = max(abs(Er), 1.0)
+    assert abs(E - Er) <= TOL[prec] * scale
+    assert np.max(np.abs(np.concatenate([dg - dgr, db - dbr]))) <= TOL[prec] * scale
+
+
+@pytest.mark.parametrize("prec", ["c64", "c128"])
+@pytest.mark.parametrize("n", [4, 5, 6, 8, 9, 11, 12, 13, 14, 15, 16, 17, 18, 19, 20])
+def test_one_launch_matches_oracle(n, prec):
+    n, e = W.prufer_tree(n, 300 + n)
+    g, b = W.random_angles(2, 40 + n)  # both rotation forms occur over the sizes
+    pl = _plan(n, e, 2, prec)
+    _check(pl.grad(g, b, "red"), O.energy_grad(n, e, g, b), prec)
+    if n >= 5:
+        assert pl.launch_count() == 1
+    if n <= 13:
+        assert np.max(np.abs(pl.statevector(g, b) - O.qaoa_state(n, e, g, b))) <= TOL[prec]
+    assert abs(pl.expect(g, b, "red") - O.energy(n, e, g, b)) <= TOL[prec] * max(n / 2, 1)
+
+
+@pytest.mark.parametrize("n,B,prec", [(9, 700, "c64"), (13, 3, "c64"), (13, 320, "c128"), (14, 40, "c64"),
+                                      (15, 5, "c128"), (16, 20, "c64"), (18, 3, "c64")])
+def test_points_share_a_launch(n, B, prec):
+    n, e = W.circulant_graph(n, (1, 3))
+    a = [W.random_angles(2, 900 + k) for k in range(B)]
+    gs, bs = np.array([x[0] for x in a]), np.array([x[1] for x in a])
+    pl = _plan(n, e, 2, prec, batch=B)
+    E, dg, db = pl.grad_batch(gs, bs, "red")
+    assert pl.launch_count() == 1
+    assert np.array_equal(pl.grad_batch(gs, bs, "red")[0], E)
+    for k in {0, 1, B // 2, B - 1}:
+        _check((E[k], dg[k], db[k]), O.energy_grad(n, e, gs[k], bs[k]), prec)
+
+
+@pytest.mark.parametrize("prec", ["c64", "c128"])
+def test_tables_larger_than_shared_memory(prec):
+    n, e = W.star_graph(12)
+    w = [51] * 11  # 562 table entries per layer, two tables, 24 layers
+    g, b = W.random_angles(24, 5)
+    pl = _plan(n, e, 24, prec, weights=w)
+    got = pl.grad(g, b, "red")
+    assert pl.launch_count() == 1
+    # 24 layers with cut values up to 561: errors on the scale of the norm
+    # bounds, max O for the energy and 2 max O max C for a gradient component
+    ref = O.energy_grad_w(n, e, w, g, b)
+    assert abs(got[0] - ref[0]) <= TOL[prec] * 561
+    assert np.max(np.abs(np.concatenate([got[1] - ref[1], got[2] - ref[2]]))) <= TOL[prec] * 2 * 561 ** 2
+
+
+@pytest.mark.parametrize("n,plan,prec", [(14, (13, 1, 12, 1), "c64"), (14, (9, 1, 8, 1), "c64"),
+                                         (15, (13, 2, 12, 2), "c64"), (18, (9, 1, 12, 1), "c64"),
+                                         (13, (12, 1, 11, 1), "c128"), (14, (8, 1, 7, 1), "c128"),
+                                         (17, (8, 1, 11, 1), "c128")])
+def test_pair_passes_match_oracle(n, plan, prec):
+    n, e = W.prufer_tree(n, 70 + n)
+    pl = _plan(n, e, 2, prec)
+    pl.set_pass_plan(*plan)
+    for seed in (3, 4):
+        g, b = W.random_angles(2, seed)
+        _check(pl.grad(g, b, "red"), O.energy_grad(n, e, g, b), prec)
+        assert pl.launch_count() > 1
+        psi = O.qaoa_state(n, e, g, b)
+        assert np.max(np.abs(pl.statevector(g, b) - psi)) <= TOL[prec]
+    pl.set_pass_plan()
+    _check(pl.grad(g, b, "red"), O.energy_grad(n, e, g, b), prec)
