@@ -55,12 +55,13 @@ _PROTOS = [
     ("aaqaoa_workspace_bytes", ctypes.c_int, [_vp, ctypes.c_int, ctypes.c_int, ctypes.POINTER(ctypes.c_size_t)]),
     ("aaqaoa_set_workspace", ctypes.c_int, [_vp, _vp, ctypes.c_size_t, ctypes.c_int, ctypes.c_int]),
     ("aaqaoa_set_stream", ctypes.c_int, [_vp, _vp]),
-    ("aaqaoa_expect", ctypes.c_int, [_vp, _f64p, _f64p, ctypes.c_int, ctypes.c_int, _f64p]),
-    ("aaqaoa_grad", ctypes.c_int, [_vp, _f64p, _f64p, ctypes.c_int, _f64p, _f64p, _f64p]),
-    ("aaqaoa_expect_batch", ctypes.c_int, [_vp, ctypes.c_int, _f64p, _f64p, ctypes.c_int, _f64p]),
+    # (the calls of an optimiser loop also take addresses: a typed pointer costs as much as the call)
+    ("aaqaoa_expect", ctypes.c_int, [_vp, _vp, _vp, ctypes.c_int, ctypes.c_int, _vp]),
+    ("aaqaoa_grad", ctypes.c_int, [_vp, _vp, _vp, ctypes.c_int, _vp, _vp, _vp]),
+    ("aaqaoa_expect_batch", ctypes.c_int, [_vp, ctypes.c_int, _vp, _vp, ctypes.c_int, _vp]),
     ("aaqaoa_expect_device", ctypes.c_int, [_vp, ctypes.c_int, _vp, _vp, ctypes.c_int, _vp]),
     ("aaqaoa_grad_device", ctypes.c_int, [_vp, _vp, _vp, ctypes.c_int, _vp]),
-    ("aaqaoa_grad_batch", ctypes.c_int, [_vp, ctypes.c_int, _f64p, _f64p, ctypes.c_int, _f64p, _f64p, _f64p]),
+    ("aaqaoa_grad_batch", ctypes.c_int, [_vp, ctypes.c_int, _vp, _vp, ctypes.c_int, _vp, _vp, _vp]),
     ("aaqaoa_grad_batch_device", ctypes.c_int, [_vp, ctypes.c_int, _vp, _vp, ctypes.c_int, _vp]),
     ("aaqaoa_sync", ctypes.c_int, [_vp]),
     ("aaqaoa_edge_zz", ctypes.c_int, [_vp, _f64p, _f64p, _f64p]),

@@ -25,6 +25,11 @@ def _f64(a):
     return np.ascontiguousarray(np.asarray(a, dtype=np.float64).reshape(-1))
 
 
+def _addr(a):
+    """The address of a contiguous array's data, or None when it is empty."""
+    return a.ctypes.data if a.size else None
+
+
 def _ptr(a, t):
     return a.ctypes.data_as(ctypes.POINTER(t)) if a is not None and a.size else None
 
@@ -109,8 +114,8 @@ class Plan:
     def expect(self, gamma, beta, observable="full", agg="fused") -> float:
         g, b = _f64(gamma), _f64(beta)
         out = ctypes.c_double()
-        N.check(N.aaqaoa_expect(self.handle, _ptr(g, ctypes.c_double), _ptr(b, ctypes.c_double),
-                                OBSERVABLES[observable], AGG_MODES[agg], ctypes.byref(out)), "aaqaoa_expect")
+        N.check(N.aaqaoa_expect(self.handle, _addr(g), _addr(b), OBSERVABLES[observable], AGG_MODES[agg],
+                                ctypes.byref(out)), "aaqaoa_expect")
         return out.value
 
     def grad(self, gamma, beta, observable="full"):
@@ -118,9 +123,8 @@ class Plan:
         E = ctypes.c_double()
         dg = np.zeros(self.p)
         db = np.zeros(self.p)
-        N.check(N.aaqaoa_grad(self.handle, _ptr(g, ctypes.c_double), _ptr(b, ctypes.c_double),
-                              OBSERVABLES[observable], ctypes.byref(E), _ptr(dg, ctypes.c_double),
-                              _ptr(db, ctypes.c_double)), "aaqaoa_grad")
+        N.check(N.aaqaoa_grad(self.handle, _addr(g), _addr(b), OBSERVABLES[observable], ctypes.byref(E), _addr(dg),
+                              _addr(db)), "aaqaoa_grad")
         return E.value, dg, db
 
     def _batch_points(self, g, b):
@@ -134,8 +138,8 @@ class Plan:
         b = _f64(betas)
         B = self._batch_points(g, b)
         out = np.zeros(B)
-        N.check(N.aaqaoa_expect_batch(self.handle, B, _ptr(g, ctypes.c_double), _ptr(b, ctypes.c_double),
-                                      OBSERVABLES[observable], _ptr(out, ctypes.c_double)), "aaqaoa_expect_batch")
+        N.check(N.aaqaoa_expect_batch(self.handle, B, _addr(g), _addr(b), OBSERVABLES[observable], _addr(out)),
+                "aaqaoa_expect_batch")
         return out
 
     def grad_batch(self, gammas, betas, observable="full"):
@@ -147,9 +151,8 @@ class Plan:
         E = np.zeros(B)
         dg = np.zeros(B * self.p)
         db = np.zeros(B * self.p)
-        N.check(N.aaqaoa_grad_batch(self.handle, B, _ptr(g, ctypes.c_double), _ptr(b, ctypes.c_double),
-                                    OBSERVABLES[observable], _ptr(E, ctypes.c_double), _ptr(dg, ctypes.c_double),
-                                    _ptr(db, ctypes.c_double)), "aaqaoa_grad_batch")
+        N.check(N.aaqaoa_grad_batch(self.handle, B, _addr(g), _addr(b), OBSERVABLES[observable], _addr(E), _addr(dg),
+                                    _addr(db)), "aaqaoa_grad_batch")
         return E, dg.reshape(B, self.p), db.reshape(B, self.p)
 
     def edge_zz(self, gamma, beta):
@@ -410,13 +413,15 @@ def _autograd_function():
             b = beta.detach().to(dtype=torch.float64).contiguous()
             out = torch.empty(1 + 2 * plan.p, dtype=torch.float64, device=g.device)
             plan.grad_device(g, b, out, observable)
-            ctx.save_for_backward(out[1:1 + plan.p].clone(), out[1 + plan.p:].clone())
+            ctx.save_for_backward(out)
+            ctx.p = plan.p
             return out[0].clone()
 
         @staticmethod
         def backward(ctx, grad_out):
-            dg, db = ctx.saved_tensors
-            return grad_out * dg, grad_out * db, None, None
+            (out,) = ctx.saved_tensors
+            d = grad_out * out[1:]  # both gradients in one product
+            return d[:ctx.p], d[ctx.p:], None, None
 
     return AAQAOAFunction
 

@@ -339,7 +339,7 @@ __global__ void __launch_bounds__(512) k_circuit(const __grid_constant__ Circuit
         __syncthreads();
 
     for (unsigned b = team; b < (unsigned)A.B; b += teams) {
-        const double *gam = A.gamma + (size_t)b * p, *bet = A.beta + (size_t)b * p;
+        const double *gam = A.gamma ? A.gamma + (size_t)b * p : A.ang, *bet = A.gamma ? A.beta + (size_t)b * p : A.ang + p;
         // ------------------------------------------------ angles, tables
         // Warps take layers, lanes table entries; the first entry of a lane is
         // computed beside the mixer's angles (the last warps), its scale

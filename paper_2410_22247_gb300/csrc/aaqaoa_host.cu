@@ -162,6 +162,7 @@ struct aaqaoa_plan {
     double state_bytes() const { return (double)((size_t)1 << n) * (double)amp(); }
     double sym() const { return half() ? 2.0 : 1.0; }  // what a sum over the stored amplitudes counts
     int tiles() const { return small() ? 1 : 1 << (bits() - T()); }
+    double *slot = nullptr;  // pinned result row of one-point host calls (HostSlots)
     bool forced = false;  // the caller set the pass plan (aaqaoa_set_pass_plan)
     bool fuse = true;  // fuse layer boundaries into one pass where the plan allows
     int *err_shared = nullptr;  // set when the plan is part of a multi-graph batch
@@ -241,11 +242,11 @@ Layout layout(const aaqaoa_plan *pl, int batch, bool grad)
     Layout L{};
     size_t off = 0;
     const size_t B = (size_t)batch;
-    L.ctrl = off;  // error flag, counters | team counters of the whole-circuit kernel
-    off += CTRL_BYTES;
     L.fns = off;  // the plan's cut functions
     off = align256(off + sizeof(GraphFns));
-    L.out = off;
+    L.ctrl = off;  // right behind: error flag, counters | team counters of the whole-circuit kernel
+    off += CTRL_BYTES;
+    L.out = off;  // right behind: one copy fetches the error flag and the rows
     off = align256(off + B * pl->out_stride() * sizeof(double));
     L.params = off;
     off = align256(off + 2 * B * pl->p * sizeof(double));
@@ -886,15 +887,22 @@ CircuitArgs circuit_args(const aaqaoa_plan *pl, int B, const CircuitPlan &q)
     return a;
 }
 
+// out: rows of `stride` doubles, or null for the workspace's. Host angles of one
+// point (h_angles: gamma, then beta) go by value.
 int enqueue_circuit(aaqaoa_plan *pl, int B, const double *d_gamma, const double *d_beta, int obs, bool grad, bool state,
-                    const CircuitPlan &q)
+                    const CircuitPlan &q, double *out = nullptr, int stride = 0, const double *h_gamma = nullptr,
+                    const double *h_beta = nullptr)
 {
     (void)cudaGetLastError();
     CircuitArgs a = circuit_args(pl, B, q);
     a.gamma = d_gamma;
     a.beta = d_beta;
-    a.out = pl->d_out();
-    a.out_stride = pl->out_stride();
+    if (h_gamma) {
+        memcpy(a.ang, h_gamma, pl->p * sizeof(double));
+        memcpy(a.ang + pl->p, h_beta, pl->p * sizeof(double));
+    }
+    a.out = out ? out : pl->d_out();
+    a.out_stride = out ? stride : pl->out_stride();
     a.state = state ? pl->d_phi() : nullptr;
     a.phi = pl->d_phi();
     a.lam = pl->d_lam();
@@ -906,6 +914,97 @@ int enqueue_circuit(aaqaoa_plan *pl, int B, const double *d_gamma, const double 
     ProfScope ps_(pl, PK_SMALL, state ? (double)B * pl->state_bytes() : 0.0);
     CKL(launch_circuit(pl->c128, grad, a, q, pl->stream), "whole-circuit kernel");
     pl->launches++;
+    return AAQAOA_OK;
+}
+
+// Pinned, device-visible result rows for one-point host calls: a plan that makes
+// such calls holds one until it is destroyed. One block per process (128 KB, made
+// by the first such call); without a free row a call copies its results back.
+class HostSlots {
+  public:
+    static constexpr int COUNT = 64, ROW = 256;  // doubles per row: 1 + 2 * 64 results and spare
+    static double *take()
+    {
+        std::lock_guard<std::mutex> lock(mutex());
+        State &s = state();
+        if (!s.tried) {
+            s.tried = true;
+            void *p = nullptr;
+            if (cudaHostAlloc(&p, sizeof(double) * COUNT * ROW, cudaHostAllocPortable | cudaHostAllocMapped) ==
+                cudaSuccess)
+                s.base = static_cast<double *>(p);
+            else
+                (void)cudaGetLastError();
+        }
+        if (!s.base || !~s.used)
+            return nullptr;
+        for (int i = 0; i < COUNT; i++)
+            if (!((s.used >> i) & 1ull)) {
+                s.used |= 1ull << i;
+                return s.base + (size_t)i * ROW;
+            }
+        return nullptr;
+    }
+    static void give(double *p)
+    {
+        if (!p)
+            return;
+        std::lock_guard<std::mutex> lock(mutex());
+        state().used &= ~(1ull << ((p - state().base) / ROW));
+    }
+
+  private:
+    struct State {
+        bool tried = false;
+        double *base = nullptr;
+        unsigned long long used = 0;
+    };
+    static State &state()
+    {
+        static State s;
+        return s;
+    }
+    static std::mutex &mutex()
+    {
+        static std::mutex m;
+        return m;
+    }
+};
+
+int fetch_out(aaqaoa_plan *pl, int B, std::vector<double> &rows);
+
+// A one-point host call as one launch and one wait: angles by value, results
+// written to the plan's pinned row (a copy either way was 20 us of a 55 us
+// gradient at n = 10). Returns 1 when the call does not fit this form, else its code.
+int circuit_host(aaqaoa_plan *pl, const double *gamma, const double *beta, int obs, bool grad, std::vector<double> &rows)
+{
+    CircuitPlan q;
+    if (!gamma || !beta || pl->p > 16 || !use_circuit(pl, 1, grad, false, &q))
+        return 1;
+    if (!pl->slot && !(pl->slot = HostSlots::take()))
+        return 1;
+    void *d_row = nullptr;
+    if (cudaHostGetDevicePointer(&d_row, pl->slot, 0) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return 1;
+    }
+    const unsigned long long unset = 0x7ff8aa90a0000001ull;  // no result has these bits
+    unsigned long long first = unset;
+    memcpy(pl->slot, &unset, sizeof unset);
+    if (!pl->small())
+        pl->state_valid = false;  // the exchange buffers are the stored state's
+    int r = enqueue_circuit(pl, 1, nullptr, nullptr, obs, grad, false, q, static_cast<double *>(d_row),
+                            pl->out_stride(), gamma, beta);
+    if (r)
+        return r;
+    CK(cudaStreamSynchronize(pl->stream));
+    memcpy(&first, pl->slot, sizeof first);
+    if (first == unset) {  // the launch gave up: its error flag says why
+        if ((r = fetch_out(pl, 1, rows)))
+            return r;
+        return fail(AAQAOA_ERR_CUDA, "the whole-circuit kernel left no result");
+    }
+    rows.assign(pl->slot, pl->slot + (grad ? pl->out_stride() : 1));
     return AAQAOA_OK;
 }
 
@@ -989,15 +1088,28 @@ int enqueue_grad(aaqaoa_plan *pl, const double *d_gamma, const double *d_beta, i
     return enqueue_backward(pl, B, obs);
 }
 
+// Whether the whole-circuit kernel may write a device call's results itself: a
+// row may be written while another point's angles are still read.
+bool direct_out(const aaqaoa_plan *pl, int B, const double *d_gamma, const double *d_beta, const double *d_out,
+                int stride)
+{
+    const size_t in = (size_t)B * pl->p, out = (size_t)B * stride;
+    const uintptr_t o = (uintptr_t)d_out, g = (uintptr_t)d_gamma, b = (uintptr_t)d_beta;
+    auto apart = [&](uintptr_t x) { return x + in * sizeof(double) <= o || o + out * sizeof(double) <= x; };
+    return !(o & 7) && apart(g) && apart(b);
+}
+
 // copy [err | pad | out rows] back and check the device error flag
 int fetch_out(aaqaoa_plan *pl, int B, std::vector<double> &rows)
 {
-    const size_t nout = (size_t)B * pl->out_stride();
-    rows.resize(nout);
-    int err = 0;
-    CK(cudaMemcpyAsync(&err, pl->d_err(), sizeof(int), cudaMemcpyDeviceToHost, pl->stream));
-    CK(cudaMemcpyAsync(rows.data(), pl->d_out(), nout * sizeof(double), cudaMemcpyDeviceToHost, pl->stream));
+    const size_t nout = (size_t)B * pl->out_stride(), nctrl = CTRL_BYTES / sizeof(double);
+    rows.resize(nctrl + nout);  // control words and rows lie side by side
+    CK(cudaMemcpyAsync(rows.data(), pl->ws + pl->L.ctrl, (nctrl + nout) * sizeof(double), cudaMemcpyDeviceToHost,
+                       pl->stream));
     CK(cudaStreamSynchronize(pl->stream));
+    int err = 0;
+    memcpy(&err, rows.data(), sizeof err);
+    rows.erase(rows.begin(), rows.begin() + nctrl);
     if (err) {
         cudaMemsetAsync(pl->ws + pl->L.ctrl, 0, CTRL_BYTES, pl->stream);
         cudaStreamSynchronize(pl->stream);
@@ -1010,10 +1122,16 @@ int upload_params(aaqaoa_plan *pl, int B, const double *gamma, const double *bet
 {
     if (!gamma || !beta)
         return fail(AAQAOA_ERR_INVALID_ARG, "gamma/beta is NULL");
-    const size_t bytes = (size_t)B * pl->p * sizeof(double);
-    double *dg = pl->d_params(), *db = pl->d_params() + (size_t)B * pl->p;
-    CK(cudaMemcpyAsync(dg, gamma, bytes, cudaMemcpyHostToDevice, pl->stream));
-    CK(cudaMemcpyAsync(db, beta, bytes, cudaMemcpyHostToDevice, pl->stream));
+    const size_t count = (size_t)B * pl->p, bytes = count * sizeof(double);
+    double both[1024];
+    if (2 * count <= sizeof both / sizeof both[0]) {  // one copy (pageable memory: staged before the call returns)
+        memcpy(both, gamma, bytes);
+        memcpy(both + count, beta, bytes);
+        CK(cudaMemcpyAsync(pl->d_params(), both, 2 * bytes, cudaMemcpyHostToDevice, pl->stream));
+        return AAQAOA_OK;
+    }
+    CK(cudaMemcpyAsync(pl->d_params(), gamma, bytes, cudaMemcpyHostToDevice, pl->stream));
+    CK(cudaMemcpyAsync(pl->d_params() + count, beta, bytes, cudaMemcpyHostToDevice, pl->stream));
     return AAQAOA_OK;
 }
 
@@ -1389,9 +1507,15 @@ int aaqaoa_set_workspace(aaqaoa_plan *pl, void *device_ptr, size_t bytes, int ba
     int r = build_maps(pl);
     if (r)
         return r;
-    CK(cudaMemsetAsync(pl->ws + L.ctrl, 0, CTRL_BYTES, pl->stream));
-    const GraphFns fns{pl->cost, {pl->obs[0], pl->obs[1]}};
-    CK(cudaMemcpyAsync(pl->ws + L.fns, &fns, sizeof fns, cudaMemcpyHostToDevice, pl->stream));
+    struct {
+        GraphFns fns;
+        unsigned char pad[256 - sizeof(GraphFns) % 256], ctrl[CTRL_BYTES];
+    } head{};  // the cut functions and zeroed control words, one copy
+    static_assert(sizeof(GraphFns) % 256 && sizeof head.fns + sizeof head.pad + CTRL_BYTES == sizeof head);
+    if (L.fns + sizeof head != L.out)
+        return fail(AAQAOA_ERR_CUDA, "workspace layout");
+    head.fns = GraphFns{pl->cost, {pl->obs[0], pl->obs[1]}};
+    CK(cudaMemcpyAsync(pl->ws + L.fns, &head, sizeof head, cudaMemcpyHostToDevice, pl->stream));
     if (pl->ising)
         CK(cudaMemcpyAsync(pl->ws + L.ising, pl->ifn.data(), pl->ifn.size() * sizeof(IsingFn), cudaMemcpyHostToDevice,
                            pl->stream));
@@ -1644,11 +1768,17 @@ int aaqaoa_expect(aaqaoa_plan *pl, const double *gamma, const double *beta, int 
     if (!energy)
         return fail(AAQAOA_ERR_INVALID_ARG, "energy is NULL");
     pl->launches = 0;
+    std::vector<double> rows;
+    r = agg_mode == AAQAOA_AGG_FUSED ? circuit_host(pl, gamma, beta, observable, false, rows) : 1;
+    if (r <= 0) {
+        if (!r)
+            *energy = rows[0];
+        return r;
+    }
     if ((r = upload_params(pl, 1, gamma, beta)))
         return r;
     if ((r = enqueue_expect(pl, 1, pl->d_params(), pl->d_params() + pl->p, observable, agg_mode)))
         return r;
-    std::vector<double> rows;
     if ((r = fetch_out(pl, 1, rows)))
         return r;
     *energy = rows[0];
@@ -1665,12 +1795,15 @@ int aaqaoa_grad(aaqaoa_plan *pl, const double *gamma, const double *beta, int ob
     if (!energy || !dgamma || !dbeta)
         return fail(AAQAOA_ERR_INVALID_ARG, "output pointer is NULL");
     pl->launches = 0;
-    if ((r = upload_params(pl, 1, gamma, beta)))
-        return r;
-    if ((r = enqueue_grad(pl, pl->d_params(), pl->d_params() + pl->p, observable)))
-        return r;
     std::vector<double> rows;
-    if ((r = fetch_out(pl, 1, rows)))
+    if ((r = circuit_host(pl, gamma, beta, observable, true, rows)) > 0) {
+        if ((r = upload_params(pl, 1, gamma, beta)))
+            return r;
+        if ((r = enqueue_grad(pl, pl->d_params(), pl->d_params() + pl->p, observable)))
+            return r;
+        r = fetch_out(pl, 1, rows);
+    }
+    if (r)
         return r;
     *energy = rows[0];
     for (int l = 0; l < pl->p; l++) {
@@ -1752,6 +1885,12 @@ int aaqaoa_grad_batch_device(aaqaoa_plan *pl, int B, const double *d_gamma, cons
     if (!d_gamma || !d_beta || !d_out)
         return fail(AAQAOA_ERR_INVALID_ARG, "device pointer is NULL");
     pl->launches = 0;
+    CircuitPlan q;
+    if (use_circuit(pl, B, true, false, &q) && direct_out(pl, B, d_gamma, d_beta, d_out, pl->out_stride())) {
+        if (!pl->small())
+            pl->state_valid = false;
+        return enqueue_circuit(pl, B, d_gamma, d_beta, observable, true, false, q, d_out, pl->out_stride());
+    }
     if ((r = enqueue_grad(pl, d_gamma, d_beta, observable, B)))
         return r;
     CK(cudaMemcpyAsync(d_out, pl->d_out(), (size_t)B * pl->out_stride() * sizeof(double), cudaMemcpyDeviceToDevice,
@@ -1769,6 +1908,12 @@ int aaqaoa_expect_device(aaqaoa_plan *pl, int B, const double *d_gamma, const do
     if (!d_gamma || !d_beta || !d_energy)
         return fail(AAQAOA_ERR_INVALID_ARG, "device pointer is NULL");
     pl->launches = 0;
+    CircuitPlan q;
+    if (use_circuit(pl, B, false, false, &q) && direct_out(pl, B, d_gamma, d_beta, d_energy, 1)) {
+        if (!pl->small())
+            pl->state_valid = false;
+        return enqueue_circuit(pl, B, d_gamma, d_beta, observable, false, false, q, d_energy, 1);
+    }
     if ((r = enqueue_expect(pl, B, d_gamma, d_beta, observable, AAQAOA_AGG_FUSED)))
         return r;
     CK(cudaMemcpy2DAsync(d_energy, sizeof(double), pl->d_out(), pl->out_stride() * sizeof(double), sizeof(double),
@@ -1785,6 +1930,12 @@ int aaqaoa_grad_device(aaqaoa_plan *pl, const double *d_gamma, const double *d_b
     if (!d_gamma || !d_beta || !d_out)
         return fail(AAQAOA_ERR_INVALID_ARG, "device pointer is NULL");
     pl->launches = 0;
+    CircuitPlan q;
+    if (use_circuit(pl, 1, true, false, &q) && direct_out(pl, 1, d_gamma, d_beta, d_out, pl->out_stride())) {
+        if (!pl->small())
+            pl->state_valid = false;
+        return enqueue_circuit(pl, 1, d_gamma, d_beta, observable, true, false, q, d_out, pl->out_stride());
+    }
     if ((r = enqueue_grad(pl, d_gamma, d_beta, observable)))
         return r;
     CK(cudaMemcpyAsync(d_out, pl->d_out(), pl->out_stride() * sizeof(double), cudaMemcpyDeviceToDevice, pl->stream));
@@ -2085,6 +2236,7 @@ void aaqaoa_destroy(aaqaoa_plan *pl)
     }
     for (auto e : pl->prof_pool)
         cudaEventDestroy(e);
+    HostSlots::give(pl->slot);
     delete pl;
 }
 

@@ -141,7 +141,8 @@ struct CircuitArgs {
     int c, Tl, a, km;    // CTAs per point 2^c, local bits, low bits of the high layout, bits per stage
     int resident;        // the phase tables of all layers fit shared memory
     double amp0;         // 2^(-n/2)
-    const double *gamma, *beta;  // [B][p]
+    const double *gamma, *beta;  // [B][p], or null: ang
+    double ang[32];      // one point's angles by value, gamma then beta (p <= 16)
     double *out;         // [B][out_stride]
     int out_stride;
     void *state;         // also store psi_p, [B][2^n] (or null; not with exchange buffers)
