@@ -741,13 +741,12 @@ template <> struct AggLayout<double> {
 };
 
 template <int NTHR>
-__device__ void agg_finish(const AggArgs &A, int nslots, double (*vals), double (*red)[32])
+__device__ void agg_finish(const AggArgs &A, double val, double (*red)[32])
 {
-    // vals[t]: this block's partial of slot t (already block-reduced, valid in thread 0)
+    // val: this block's partial (already block-reduced, valid in thread 0)
     __shared__ unsigned s_last;
     if (threadIdx.x == 0) {
-        for (int t = 0; t < nslots; t++)
-            A.partials[(size_t)t * gridDim.x + blockIdx.x] = vals[t];
+        A.partials[blockIdx.x] = val;
         __threadfence();
         s_last = (atomicAdd(A.counter, 1u) == gridDim.x - 1u) ? 1u : 0u;
     }
@@ -755,24 +754,14 @@ __device__ void agg_finish(const AggArgs &A, int nslots, double (*vals), double 
     if (!s_last)
         return;
     __threadfence();
-    for (int t = 0; t < nslots; t++) {
-        double a = 0.0, dummy = 0.0;
-        for (int i = threadIdx.x; i < (int)gridDim.x; i += NTHR)
-            a += __ldcg(A.partials + (size_t)t * gridDim.x + i);
-        block_sum2<NTHR>(a, dummy, red);
-        if (threadIdx.x == 0) {
-            a *= A.scale;
-            if (A.num_terms == 0) {
-                *A.out_energy += a;
-            } else {
-                if (A.out_terms)
-                    A.out_terms[t] = a;
-                *A.out_energy += A.term_w[t] * 0.5 * (1.0 - a);
-            }
-        }
-    }
-    if (threadIdx.x == 0)
+    double a = 0.0, dummy = 0.0;
+    for (int i = threadIdx.x; i < (int)gridDim.x; i += NTHR)
+        a += __ldcg(A.partials + i);
+    block_sum2<NTHR>(a, dummy, red);
+    if (threadIdx.x == 0) {
+        *A.out_energy += a * A.scale;
         *A.counter = 0u;
+    }
 }
 
 // E += sum_x |psi_x|^2 O(x) over a stored state (one read). A flip-symmetric
@@ -812,64 +801,145 @@ __global__ void __launch_bounds__(256) k_agg_fused(const __grid_constant__ AggAr
     }
     double dummy = 0.0;
     block_sum2<256>(acc, dummy, red);
-    double v[1] = {acc};
-    agg_finish<256>(A, 1, v, red);
+    agg_finish<256>(A, acc, red);
 }
 
 // Per-term <Z_u Z_v> over a stored state, all terms of the launch in one read.
 // Per lane: p_m = |psi_m|^2 for its 32 amplitudes, Walsh-Hadamard transformed
-// over the 5 register bits, F[mask] = sum_m p_m (-1)^{popcount(m & mask)};
-// a term whose endpoints fall on register bits `mask` (and on lane/chunk bits
-// elsewhere) contributes sign(x0) * F[mask].
+// over the 5 register bits, F[mask] = sum_m p_m (-1)^{popcount(m & mask)}. A
+// term with both ends on register bits adds F of the two; otherwise it needs
+// F[0] or F[one register bit] with the signs of its other ends on lane bits
+// and chunk bits. Those six values are transformed over the lanes too (a
+// butterfly of shuffles: lane L holds the sum with the signs of lane mask L),
+// so that a chunk costs one FP64 addition per term and warp, each term owned
+// by a lane, instead of one per term and lane: 42 terms at n = 28 took 2.3 ms
+// of selects and FP64 additions against 0.16 ms of memory time, and take 0.4.
+// One term reads the state at 5.4-6.0 TB/s (n = 28, 30). The lanes'
+// sums carry their rounding errors along (float pairs, TwoSum), as the FP64
+// sums over lanes did.
+template <typename R> struct LaneSum;
+template <> struct LaneSum<float> {
+    float hi, lo;
+    __device__ __forceinline__ static LaneSum make(float v) { return {v, 0.f}; }
+    __device__ __forceinline__ LaneSum step(int o, bool neg) const  // butterfly with lane ^ o
+    {
+        const float a = neg ? -hi : hi, la = neg ? -lo : lo;
+        const float b = __shfl_xor_sync(0xffffffffu, hi, o), lb = __shfl_xor_sync(0xffffffffu, lo, o);
+        const float t = __fadd_rn(a, b), z = __fsub_rn(t, a);
+        const float e = __fadd_rn(__fsub_rn(a, __fsub_rn(t, z)), __fsub_rn(b, z));
+        return {t, __fadd_rn(__fadd_rn(la, lb), e)};
+    }
+    // sums of chunks: the rounded parts in FP64, the rounding errors (2^-24 of
+    // them) in float
+    __device__ __forceinline__ void add_to(double &a, float &b, bool neg) const
+    {
+        a += (double)(neg ? -hi : hi);
+        b += neg ? -lo : lo;
+    }
+};
+template <> struct LaneSum<double> {
+    double v;
+    __device__ __forceinline__ static LaneSum make(double v) { return {v}; }
+    __device__ __forceinline__ LaneSum step(int o, bool neg) const
+    {
+        return {(neg ? -v : v) + __shfl_xor_sync(0xffffffffu, v, o)};
+    }
+    __device__ __forceinline__ void add_to(double &a, float &, bool neg) const { a += neg ? -v : v; }
+};
+
 template <typename R>
-__global__ void __launch_bounds__(256) k_agg_terms(const __grid_constant__ AggArgs A)
+__global__ void __launch_bounds__(256, std::is_same<R, float>::value ? 2 : 1) k_agg_terms(const __grid_constant__ AggArgs A)
 {
     using C = typename CT<R>::T;
     using L = AggLayout<R>;
-    extern __shared__ double acc_s[];  // [num_terms][256]
-    __shared__ double red[2][32];
-    const int lane = threadIdx.x & 31, T = A.num_terms;
-    for (int t = 0; t < T; t++)
-        acc_s[t * 256 + threadIdx.x] = 0.0;
+    using LS = LaneSum<R>;
+    constexpr int PAIRS = 10;  // pairs of register bits, (k2, k) with k2 < k at k (k - 1) / 2 + k2
+    __shared__ LS vals[8][6 * 32];
+    __shared__ double wsum[64][8], tsum[64];
+    __shared__ unsigned s_last;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, T = A.num_terms;
     const C *st = reinterpret_cast<const C *>(A.state);
+    for (int i = threadIdx.x; i < 64 * 8; i += 256)
+        wsum[i / 8][i % 8] = 0.0;
+    __syncthreads();
     if (A.bits < 10) {
         const int N = 1 << A.bits;
         if (blockIdx.x == 0)
-            for (int x = threadIdx.x; x < N; x += 256) {
-                const double pr = (double)(st[x].x * st[x].x + st[x].y * st[x].y);
-                for (int t = 0; t < T; t++)
-                    acc_s[t * 256 + threadIdx.x] += (((x >> A.term_u[t]) ^ (x >> A.term_v[t])) & 1) ? -pr : pr;
+            for (int t = warp; t < T; t += 8) {
+                double a = 0.0;
+                for (int x = lane; x < N; x += 32) {
+                    const double pr = (double)(st[x].x * st[x].x + st[x].y * st[x].y);
+                    a += (((x >> A.term_u[t]) ^ (x >> A.term_v[t])) & 1) ? -pr : pr;
+                }
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1)
+                    a += __shfl_xor_sync(0xffffffffu, a, o);
+                if (lane == 0)
+                    wsum[t][0] = a;
             }
     } else {
-        // register-bit masks of each term's endpoints
-        uint32_t tmask[64];
-        uint64_t tfix[64];
-        for (int t = 0; t < T; t++) {
-            uint32_t m = 0;
-            uint64_t f = 0;
-            const int ends[2] = {A.term_u[t], A.term_v[t]};
-            for (int e = 0; e < 2; e++) {
+        // the ends of a term: register mask, lane mask, chunk mask
+        const uint64_t lanes = L::lane_bits(31);
+        auto ends = [&](int t, uint32_t &rm, uint32_t &lm, uint64_t &cm) {
+            rm = lm = 0;
+            cm = 0;
+            const int e[2] = {A.term_u[t], A.term_v[t]};
+            for (int q = 0; q < 2; q++) {
                 int k = -1;
 #pragma unroll
                 for (int kk = 0; kk < 5; kk++)
-                    if (L::gp(kk) == ends[e])
+                    if (L::gp(kk) == e[q])
                         k = kk;
                 if (k >= 0)
-                    m ^= 1u << k;
+                    rm ^= 1u << k;
+                else if ((lanes >> e[q]) & 1ull)
+                    lm ^= (uint32_t)(1ull << e[q] >> (__ffsll((long long)lanes) - 1));
                 else
-                    f ^= 1ull << ends[e];
+                    cm ^= 1ull << e[q];
             }
-            tmask[t] = m;
-            tfix[t] = f;
+        };
+        // this lane's terms: which value of vals, which chunk bits; and the values any term needs
+        uint32_t need = 0, needp = 0;  // F[0] and F[1 << k]; pairs
+        int idx[2] = {-1, -1};
+        uint64_t cmask[2] = {0, 0};
+        for (int t = 0; t < T; t++) {
+            uint32_t rm, lm;
+            uint64_t cm;
+            ends(t, rm, lm, cm);
+            if (rm & (rm - 1)) {
+                const int k = 31 - __clz(rm), k2 = __ffs(rm) - 1;
+                needp |= 1u << (k * (k - 1) / 2 + k2);
+                continue;
+            }
+            const int j = rm ? __ffs(rm) : 0;
+            need |= 1u << j;
+            if ((t & 31) == lane) {
+                idx[t >> 5] = j * 32 + (int)lm;
+                cmask[t >> 5] = cm;
+            }
         }
+        double acc[2] = {0.0, 0.0}, pacc[PAIRS];
+        float accl[2] = {0.f, 0.f};
+#pragma unroll
+        for (int i = 0; i < PAIRS; i++)
+            pacc[i] = 0.0;
         const uint64_t warps = (uint64_t)gridDim.x * 8;
-        for (uint64_t ch = (uint64_t)blockIdx.x * 8 + (threadIdx.x >> 5); ch < A.chunks; ch += warps) {
-            C a[32];
+        // complex64: the next chunk's loads are in flight while this one is
+        // summed (128 registers, 16 warps an SM; one term at n = 28 251 -> 198 us)
+        constexpr bool AHEAD = std::is_same<R, float>::value;
+        C a[32];
+        uint64_t ch = (uint64_t)blockIdx.x * 8 + warp;
+        if (AHEAD && ch < A.chunks)
             L::load(st, ch << 10, lane, a);
+        for (; ch < A.chunks; ch += warps) {
+            if (!AHEAD)
+                L::load(st, ch << 10, lane, a);
             R F[32];
 #pragma unroll
             for (int m = 0; m < 32; m++)
                 F[m] = a[m].x * a[m].x + a[m].y * a[m].y;
+            if (AHEAD && ch + warps < A.chunks)
+                L::load(st, (ch + warps) << 10, lane, a);
 #pragma unroll
             for (int k = 0; k < 5; k++)
 #pragma unroll
@@ -879,24 +949,94 @@ __global__ void __launch_bounds__(256) k_agg_terms(const __grid_constant__ AggAr
                         F[m] = u + v;
                         F[m | (1 << k)] = u - v;
                     }
-            const uint64_t x0 = (ch << 10) | L::lane_bits(lane);
-            for (int t = 0; t < T; t++) {
-                R f = F[0];
+            __syncwarp();  // the warp's reads of the previous chunk's values
 #pragma unroll
-                for (int q = 1; q < 32; q++)
-                    f = (tmask[t] == (uint32_t)q) ? F[q] : f;
-                const R sgn = (__popcll(x0 & tfix[t]) & 1) ? (R)-1 : (R)1;
-                acc_s[t * 256 + threadIdx.x] += (double)(sgn * f);
+            for (int j = 0; j < 6; j++)
+                if ((need >> j) & 1) {
+                    LS v = LS::make(F[j ? 1 << (j - 1) : 0]);
+#pragma unroll
+                    for (int o = 1; o < 32; o <<= 1)
+                        v = v.step(o, lane & o);
+                    vals[warp][j * 32 + lane] = v;
+                }
+#pragma unroll
+            for (int k = 1; k < 5; k++)
+#pragma unroll
+                for (int k2 = 0; k2 < k; k2++)
+                    if ((needp >> (k * (k - 1) / 2 + k2)) & 1)
+                        pacc[k * (k - 1) / 2 + k2] += (double)F[(1 << k) | (1 << k2)];
+            __syncwarp();
+#pragma unroll
+            for (int q = 0; q < 2; q++)
+                if (idx[q] >= 0)
+                    vals[warp][idx[q]].add_to(acc[q], accl[q], __popcll((ch << 10) & cmask[q]) & 1);
+        }
+#pragma unroll
+        for (int q = 0; q < 2; q++)
+            if (idx[q] >= 0)
+                wsum[lane + 32 * q][warp] = acc[q] + (double)accl[q];
+#pragma unroll
+        for (int i = 0; i < PAIRS; i++)
+            if ((needp >> i) & 1) {
+                double v = pacc[i];
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1)
+                    v += __shfl_xor_sync(0xffffffffu, v, o);
+                pacc[i] = v;
             }
+        if (needp && lane == 0)
+            for (int t = 0; t < T; t++) {
+                uint32_t rm, lm;
+                uint64_t cm;
+                ends(t, rm, lm, cm);
+                if (rm & (rm - 1)) {
+                    const int k = 31 - __clz(rm), k2 = __ffs(rm) - 1;
+                    double v = 0.0;
+#pragma unroll
+                    for (int i = 0; i < PAIRS; i++)
+                        v = i == k * (k - 1) / 2 + k2 ? pacc[i] : v;
+                    wsum[t][warp] = v;
+                }
+            }
+    }
+    __syncthreads();
+    // per-CTA sums; the last CTA adds them, a warp per term, in a fixed order
+    if (threadIdx.x < T) {
+        double v = 0.0;
+        for (int w = 0; w < 8; w++)
+            v += wsum[threadIdx.x][w];
+        __stcg(A.partials + (size_t)threadIdx.x * gridDim.x + blockIdx.x, v);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        s_last = (atomicAdd(A.counter, 1u) == gridDim.x - 1u) ? 1u : 0u;
+        __threadfence();
+    }
+    __syncthreads();
+    if (!s_last)
+        return;
+    for (int t = warp; t < T; t += 8) {
+        double v = 0.0;
+        for (int i = lane; i < (int)gridDim.x; i += 32)
+            v += __ldcg(A.partials + (size_t)t * gridDim.x + i);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+            v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0) {
+            tsum[t] = v * A.scale;
+            if (A.out_terms)
+                A.out_terms[t] = v * A.scale;
         }
     }
-    double vals[64];
-    for (int t = 0; t < T; t++) {
-        double v = acc_s[t * 256 + threadIdx.x], dummy = 0.0;
-        block_sum2<256>(v, dummy, red);
-        vals[t] = v;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double e = 0.0;
+        for (int t = 0; t < T; t++)
+            e += A.term_w[t] * 0.5 * (1.0 - tsum[t]);
+        *A.out_energy += e;
+        *A.counter = 0u;
     }
-    agg_finish<256>(A, T, vals, red);
 }
 
 // ------------------------------------------------------------- launchers
@@ -1372,19 +1512,10 @@ int launch_agg_fused(bool c128, const AggArgs &a, cudaStream_t st, int grid)
 
 int launch_agg_terms(bool c128, const AggArgs &a, cudaStream_t st, int grid)
 {
-    const size_t smem = (size_t)a.num_terms * 256 * sizeof(double);
-    cudaError_t e;
-    if (c128) {
-        e = cudaFuncSetAttribute(k_agg_terms<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 256 * 8);
-        if (e != cudaSuccess)
-            return (int)e;
-        k_agg_terms<double><<<grid, 256, smem, st>>>(a);
-    } else {
-        e = cudaFuncSetAttribute(k_agg_terms<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 256 * 8);
-        if (e != cudaSuccess)
-            return (int)e;
-        k_agg_terms<float><<<grid, 256, smem, st>>>(a);
-    }
+    if (c128)
+        k_agg_terms<double><<<grid, 256, 0, st>>>(a);
+    else
+        k_agg_terms<float><<<grid, 256, 0, st>>>(a);
     return (int)cudaGetLastError();
 }
 
