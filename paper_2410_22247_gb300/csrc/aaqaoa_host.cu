@@ -128,8 +128,9 @@ struct aaqaoa_plan {
     bool ws_grad = false;
     Layout L{};
     std::vector<Pass> passes;      // forward passes (one-vector tile geometry)
+    std::vector<Pass> gpasses;     // forward passes of a gradient evaluation
     std::vector<Pass> bwd_passes;  // adjoint passes (two-vector tile geometry)
-    std::vector<CUtensorMap> map_phi;            // forward, per pass
+    std::vector<CUtensorMap> map_phi, map_gphi;  // forward, per pass
     std::vector<CUtensorMap> map_bphi, map_blam; // adjoint, per pass
     std::vector<std::array<CUtensorMap, 4>> map_bcl;  // cluster passes: load phi, lambda; store phi, lambda
     int launches = 0;
@@ -388,9 +389,35 @@ void default_layer(int n, int T, int cbmin, int hbmax, int L2, int *L, int *K, b
     *L = (L2 < T && layer_passes(n, T, cbmin, hbmax, L2, L2, *K, v, false, big_last)) ? L2 : T;
 }
 
+// Default plan of a gradient evaluation with two high passes per layer: equal
+// high groups (8 qubits, or 7) for both sweeps, so that the forward's last group
+// is the adjoint's and a turnaround pass joins them (5 S of traffic become 2 S).
+// The low passes take what is left: the forward's the bits of two register
+// stages where its groups then still end alike, the adjoint's a whole tile where
+// its larger last group does. Against the separate defaults (complex64, p = 2,
+// ms): n = 23 0.319 -> 0.311, 24 0.501 -> 0.475, 25 0.874 -> 0.801, 26 1.521 ->
+// 1.413, 27 2.84 -> 2.64, 28 5.56 -> 5.11; complex128 n = 24 7.49 -> 7.39. With
+// three high passes the equal split costs more passes' stages than it saves
+// (n = 29 12.9 -> 13.9, n = 30 has a turnaround without it).
+bool turn_layers(const aaqaoa_plan *pl, std::vector<Pass> &g, std::vector<Pass> &b)
+{
+    int T1, T2, CB1, CB2, HB1, HB2;
+    pass_geometry(pl->c128, 1, &T1, &CB1, &HB1);
+    pass_geometry(pl->c128, 2, &T2, &CB2, &HB2);
+    const int n = pl->n, L1 = low_two_stage_bits(pl->c128, 1), L2 = low_two_stage_bits(pl->c128, 2);
+    const int r = std::min(2 * HB2, (n - L2) & ~1), L = n - r;
+    if (r < 14 || L > T2)
+        return false;
+    const int Lb = (n - T2 + 1) / 2 == r / 2 ? T2 : L;
+    const int Lf = (n - L1) / 2 == r / 2 && (n - L1 + 1) / 2 <= HB1 ? L1 : L;
+    return layer_passes(n, T1, CB1, HB1, L1, Lf, 2, g, false, false, pl->half()) &&
+           layer_passes(n, T2, CB2, HB2, L2, Lb, 2, b, false, true, pl->half());
+}
+
 void build_passes(aaqaoa_plan *pl)
 {
     pl->passes.clear();
+    pl->gpasses.clear();
     pl->bwd_passes.clear();
     if (pl->small())
         return;
@@ -400,6 +427,13 @@ void build_passes(aaqaoa_plan *pl)
         const int L2 = low_two_stage_bits(pl->c128, nv);
         default_layer(pl->n, T, CB, HB, L2, &L, &K, nv == 2);
         layer_passes(pl->n, T, CB, HB, L2, L, K, nv == 1 ? pl->passes : pl->bwd_passes, false, nv == 2, pl->half());
+    }
+    std::vector<Pass> g, b;
+    if (turn_layers(pl, g, b)) {
+        pl->gpasses = g;
+        pl->bwd_passes = b;
+    } else {
+        pl->gpasses = pl->passes;
     }
 }
 
@@ -556,17 +590,17 @@ Turn turnaround(const aaqaoa_plan *pl)
     Turn t;
     // the adjoint's first layer keeps a high pass after the turnaround's group
     // (its last stage carries dE/dgamma and the inverse phase)
-    if (!plan_fuses(pl) || pl->small() || pl->passes.size() < 3 || pl->bwd_passes.size() < 3)
+    if (!plan_fuses(pl) || pl->small() || pl->gpasses.size() < 3 || pl->bwd_passes.size() < 3)
         return t;
     for (size_t kb = 0; kb < pl->bwd_passes.size(); kb++) {
         const Pass &b = pl->bwd_passes[kb];
         if (b.is_low || b.cluster)
             continue;
-        for (size_t kf = 0; kf < pl->passes.size(); kf++) {
-            const Pass &f = pl->passes[kf];
+        for (size_t kf = 0; kf < pl->gpasses.size(); kf++) {
+            const Pass &f = pl->gpasses[kf];
             if (f.is_low || f.s != b.s || f.qubits != b.qubits)
                 continue;
-            if (layer_schedule(pl->p, pl->passes, true, false, !pl->c128, (int)kf).empty())
+            if (layer_schedule(pl->p, pl->gpasses, true, false, !pl->c128, (int)kf).empty())
                 continue;
             t.kf = (int)kf;
             t.kb = (int)kb;
@@ -582,7 +616,7 @@ enum FwdMode { FWD_ENERGY, FWD_GRAD, FWD_STATE };
 // over B points. The workspace pointers are the plan's (base_args).
 PassArgs forward_args(const aaqaoa_plan *pl, int obs, int B, const Step &sp, size_t i, size_t n, FwdMode mode)
 {
-    const Pass &ps = pl->passes[sp.k];
+    const Pass &ps = (mode == FWD_GRAD ? pl->gpasses : pl->passes)[sp.k];
     PassArgs a = base_args(pl, obs);
     a.B = B;
     a.s = ps.s;
@@ -627,7 +661,8 @@ int enqueue_forward(aaqaoa_plan *pl, int B, int obs, FwdMode mode)
     const int grid = pass_grid(total);
     const int chunk = B > 1 ? (int)((total + grid - 1) / grid) : 0;
     const Turn tn = mode == FWD_GRAD ? turnaround(pl) : Turn{};
-    std::vector<Step> sched = layer_schedule(pl->p, pl->passes, plan_fuses(pl), false, !pl->c128, tn.kf);
+    std::vector<Step> sched = layer_schedule(pl->p, mode == FWD_GRAD ? pl->gpasses : pl->passes, plan_fuses(pl), false,
+                                             !pl->c128, tn.kf);
     if (tn.kf >= 0)
         sched.pop_back();
     for (size_t i = 0; i < sched.size(); i++) {
@@ -640,7 +675,8 @@ int enqueue_forward(aaqaoa_plan *pl, int B, int obs, FwdMode mode)
         }
         const double S = (double)B * pl->state_bytes();
         ProfScope ps_(pl, PK_FWD, S * ((a.load ? 1 : 0) + (a.write ? 1 : 0)), pass_flags(a));
-        CKL(launch_pass(pl->c128, 1, pl->map_phi[sp.k], pl->map_phi[sp.k], a, grid, pl->stream), "forward pass");
+        const CUtensorMap &map = (mode == FWD_GRAD ? pl->map_gphi : pl->map_phi)[sp.k];
+        CKL(launch_pass(pl->c128, 1, map, map, a, grid, pl->stream), "forward pass");
         pl->launches++;
     }
     return AAQAOA_OK;
@@ -1449,6 +1485,7 @@ int aaqaoa_workspace_bytes(const aaqaoa_plan *plan, int batch, int with_grad, si
 int build_maps(aaqaoa_plan *pl)
 {
     pl->map_phi.assign(pl->passes.size(), CUtensorMap{});
+    pl->map_gphi.assign(pl->gpasses.size(), CUtensorMap{});
     pl->map_bphi.assign(pl->bwd_passes.size(), CUtensorMap{});
     pl->map_blam.assign(pl->bwd_passes.size(), CUtensorMap{});
     pl->map_bcl.assign(pl->bwd_passes.size(), std::array<CUtensorMap, 4>{});
@@ -1459,6 +1496,13 @@ int build_maps(aaqaoa_plan *pl)
     for (size_t k = 0; k < pl->passes.size(); k++) {
         Pass &ps = pl->passes[k];
         int r = make_map(&pl->map_phi[k], pl->d_phi(), pl->bits(), ps.s, ps.cb, T - ps.pair, CB, pl->amp(), pl->cap,
+                         &ps.wide);
+        if (r)
+            return r;
+    }
+    for (size_t k = 0; k < pl->gpasses.size() && pl->ws_grad; k++) {
+        Pass &ps = pl->gpasses[k];
+        int r = make_map(&pl->map_gphi[k], pl->d_phi(), pl->bits(), ps.s, ps.cb, T - ps.pair, CB, pl->amp(), pl->cap,
                          &ps.wide);
         if (r)
             return r;
@@ -1531,6 +1575,11 @@ static int set_layers(aaqaoa_plan *pl, const int plan4[4])
 {
     if (pl->small())
         return AAQAOA_OK;
+    if (!plan4[0] && !plan4[1] && !plan4[2] && !plan4[3]) {
+        build_passes(pl);
+        pl->state_valid = false;
+        return build_maps(pl);
+    }
     std::vector<Pass> v[2];
     for (int nv = 1; nv <= 2; nv++) {
         int T, CB, HB, L, K;
@@ -1545,7 +1594,7 @@ static int set_layers(aaqaoa_plan *pl, const int plan4[4])
             return fail(AAQAOA_ERR_INVALID_ARG, "%s plan: low pass of %d qubits + %d high passes does not tile n=%d",
                         nv == 1 ? "forward" : "adjoint", L, K, pl->n);
     }
-    pl->passes = v[0];
+    pl->passes = pl->gpasses = v[0];
     pl->bwd_passes = v[1];
     pl->state_valid = false;
     return build_maps(pl);
@@ -1601,7 +1650,7 @@ int aaqaoa_get_schedule(aaqaoa_plan *pl, int adjoint, int32_t *steps, int cap, i
     if (!pl || !count || cap < 0 || (cap > 0 && !steps) || adjoint < 0 || adjoint > 2)
         return fail(AAQAOA_ERR_INVALID_ARG, "plan/count is NULL, cap < 0, steps is NULL or adjoint not 0/1/2");
     const bool bwd = adjoint == 1;
-    const std::vector<Pass> &passes = bwd ? pl->bwd_passes : pl->passes;
+    const std::vector<Pass> &passes = bwd ? pl->bwd_passes : adjoint ? pl->gpasses : pl->passes;
     const Turn tn = adjoint ? turnaround(pl) : Turn{};  // gradient evaluations only
     std::vector<Step> sched = bwd ? layer_schedule(pl->p, passes, plan_fuses(pl), true, false, -1, tn.kb)
                                   : layer_schedule(pl->p, passes, plan_fuses(pl), false, !pl->c128, tn.kf);
@@ -1735,6 +1784,22 @@ int aaqaoa_autotune(aaqaoa_plan *pl, int *plan4)
             }
             if ((r = set_layers(pl, best.data())))
                 return r;
+            if (pl->ws_grad) {  // the default may give the two sweeps of a gradient matching groups
+                auto both = [&]() {
+                    const int q = enqueue_forward(pl, 1, AAQAOA_OBS_FULL, FWD_GRAD);
+                    return q ? q : enqueue_backward(pl, 1, AAQAOA_OBS_FULL);
+                };
+                time_ms(pl->stream, both, 1);
+                const float tuned = time_ms(pl->stream, both, 2);
+                const std::array<int, 4> dflt{0, 0, 0, 0};
+                if ((r = set_layers(pl, dflt.data())))
+                    return r;
+                time_ms(pl->stream, both, 1);
+                if (time_ms(pl->stream, both, 2) <= tuned)
+                    best = dflt;
+                else if ((r = set_layers(pl, best.data())))
+                    return r;
+            }
             std::vector<double> rows;
             if ((r = fetch_out(pl, 1, rows)))  // a device timeout during tuning surfaces here
                 return r;
