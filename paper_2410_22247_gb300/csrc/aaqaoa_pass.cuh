@@ -1226,8 +1226,8 @@ __device__ __forceinline__ void mix_stage(const PassRegs &A, StageCtx<R> &X,
         store_regs<R, NV, ST>(X.sv1, sb, sb, l);
 }
 
-// Which owned bits of stage st a pass with this shape transforms: 0 every
-// owned bit, 1 all but the first, -1 another set. A high pass transforms the
+// Which owned bits of stage st a pass with this shape transforms: d >= 0 all but
+// the first d (up to 3), -1 another set. A high pass transforms the
 // tile bits from cb up, a low pass those below cb plus the high bits in hmask.
 template <typename G>
 __host__ __device__ inline int due_form(int st, int is_low, int hmask, int cb)
@@ -1241,7 +1241,10 @@ __host__ __device__ inline int due_form(int st, int is_low, int hmask, int cb)
         if (bit >= cb ? ((hmask >> (bit - cb)) & 1) : is_low)
             due |= 1u << k;
     }
-    return due == own ? 0 : due == (own & (own - 1u)) ? 1 : -1;
+    for (int d = 0; d < 4 && own; d++, own &= own - 1u)
+        if (due == own)
+            return d;
+    return -1;
 }
 
 // A register stage in the compiled form of its due pattern d (complex64: the
@@ -1258,6 +1261,13 @@ __device__ __forceinline__ void run_stage_due(int d, const PassRegs &A, StageCtx
             return run_stage<R, NV, ST, OPS, FUSE, IS, 0>(A, X, a, l, acc0, acc1, acc2);
         if (d == 1)
             return run_stage<R, NV, ST, OPS, FUSE, IS, 1>(A, X, a, l, acc0, acc1, acc2);
+        // one-vector high passes of 7 and 6 qubits (n = 20, 28; n = 19)
+        if constexpr (NV == 1 && ST == 1 && !IS) {
+            if (d == 2)
+                return run_stage<R, NV, ST, OPS, FUSE, IS, 2>(A, X, a, l, acc0, acc1, acc2);
+            if (d == 3)
+                return run_stage<R, NV, ST, OPS, FUSE, IS, 3>(A, X, a, l, acc0, acc1, acc2);
+        }
     }
     run_stage<R, NV, ST, OPS, FUSE, IS, -1>(A, X, a, l, acc0, acc1, acc2);
 }
