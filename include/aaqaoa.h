@@ -424,7 +424,9 @@ int aaqaoa_inject_fault(aaqaoa_plan *plan, int kind);
  * passes and {L, K} of the two-vector adjoint passes (all 0 for plans small
  * enough for the whole-circuit kernel).
  *
- * aaqaoa_get_pass_plan: plan4 (host, 4 ints) receives the current plan.
+ * aaqaoa_get_pass_plan: plan4 (host, 4 ints) receives the current plan. (Without
+ *   a plan set here, the forward sweep of a gradient may use other groups than
+ *   an energy's, chosen to end on the adjoint's last: aaqaoa_get_schedule.)
  * aaqaoa_set_pass_plan: 0 keeps the default for that entry (the fewest high
  *   passes; a two-register-stage low pass when they can take the rest).
  *   For complex64 plans the adjoint's low pass may span 14 qubits (bwd_low =

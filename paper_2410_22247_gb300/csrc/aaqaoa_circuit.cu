@@ -204,47 +204,6 @@ __device__ __noinline__ int4 circ_cuts(const uint32_t *nbr, const int *w, int K,
     return make_int4(base, base + d0, base + d1, base + d0 + d1 - 2 * w01);
 }
 
-// cos x, sin x in FP64 for the phase tables, by reduction to |r| <= pi/4 (x -
-// k pi/2 with pi/2 in two parts, fused) and the Taylor series there: the
-// library's function costs 3 us at the head of a launch. float: a relative
-// error below 1e-10, rounded once to the table's precision; double: 1e-16.
-template <typename R>
-__device__ __noinline__ double2 phase_sincos(double x)  // (cos, sin)
-{
-    const double k = rint(x * 0.63661977236758134308);
-    if (!(fabs(k) < 1e9)) {
-        double sn, cn;
-        sincos(x, &sn, &cn);
-        return make_double2(cn, sn);
-    }
-    double r = fma(k, -1.5707963267948965580, x);
-    r = fma(k, -6.1232339957367660359e-17, r);
-    const double s = r * r;
-    double ps, pc;
-    if constexpr (std::is_same<R, float>::value) {
-        ps = fma(s, -1.0 / 39916800.0, 1.0 / 362880.0);
-        pc = fma(s, 1.0 / 479001600.0, -1.0 / 3628800.0);
-    } else {
-        ps = fma(s, -1.0 / 1307674368000.0, 1.0 / 6227020800.0);
-        pc = fma(s, 1.0 / 20922789888000.0, -1.0 / 87178291200.0);
-        ps = fma(ps, s, -1.0 / 39916800.0);
-        pc = fma(pc, s, 1.0 / 479001600.0);
-        ps = fma(ps, s, 1.0 / 362880.0);
-        pc = fma(pc, s, -1.0 / 3628800.0);
-    }
-    ps = fma(ps, s, -1.0 / 5040.0);
-    pc = fma(pc, s, 1.0 / 40320.0);
-    ps = fma(ps, s, 1.0 / 120.0);
-    pc = fma(pc, s, -1.0 / 720.0);
-    ps = fma(ps, s, -1.0 / 6.0);
-    pc = fma(pc, s, 1.0 / 24.0);
-    pc = fma(pc, s, -0.5);
-    const double sr = fma(r * s, ps, r), cr = fma(s, pc, 1.0);
-    const int q = (int)(long long)k & 3;
-    const double a = (q & 1) ? cr : sr, b = (q & 1) ? sr : cr;
-    return make_double2(((q + 1) & 2) ? -b : b, (q & 2) ? -a : a);
-}
-
 // cluster (distributed shared memory) helpers
 __device__ __forceinline__ void circ_cluster_sync()
 {
@@ -350,16 +309,9 @@ __global__ void __launch_bounds__(512) k_circuit(const __grid_constant__ Circuit
         for (int l = nt - 1 - tid; l < p; l += nt) {
             const double2 z = phase_sincos<double>(bet[l]);
             const bool sh = fabs(z.y) > fabs(z.x);  // rotate by beta - pi/2 (see rot)
-            const double u = sh ? -z.x : z.y, v = sh ? z.y : z.x;
-            double t;
-            if constexpr (std::is_same<R, float>::value)
-                t = (double)((float)u / (float)v);
-            else
-                t = u / v;
-            // the factor that a butterfly with the rounded t drops,
-            // 1 / sqrt(1 + t^2) with v's sign: v (1 - u (t v - u)) to first
-            // order in the rounding, t v - u
-            const double f = v - v * (u * fma(t, v, -u)), fi = sh ? -f : f;
+            double t, f;
+            mix_ratio<R>(sh ? -z.x : z.y, sh ? z.y : z.x, t, f);
+            const double fi = sh ? -f : f;
             double fn = 1.0, q = f;
             for (int k = n; k; k >>= 1) {
                 if (k & 1)

@@ -174,7 +174,7 @@ struct aaqaoa_plan {
     unsigned *d_counter_agg() const { return reinterpret_cast<unsigned *>(ws + L.ctrl + 16); }
     double *d_out() const { return reinterpret_cast<double *>(ws + L.out); }
     double *d_params() const { return reinterpret_cast<double *>(ws + L.params); }
-    double2 *d_cs() const { return reinterpret_cast<double2 *>(ws + L.cs); }
+    MixRow *d_cs() const { return reinterpret_cast<MixRow *>(ws + L.cs); }
     void *d_tab() const { return ws + L.tab; }
     double *d_partials() const { return reinterpret_cast<double *>(ws + L.partials); }
     double *d_zz() const { return reinterpret_cast<double *>(ws + L.zz); }
@@ -252,7 +252,7 @@ Layout layout(const aaqaoa_plan *pl, int batch, bool grad)
     L.params = off;
     off = align256(off + 2 * B * pl->p * sizeof(double));
     L.cs = off;
-    off = align256(off + B * pl->p * sizeof(double2));
+    off = align256(off + B * pl->p * sizeof(MixRow));
     L.tab = off;  // three tables: exact, forward-scaled, inverse layer
     off = align256(off + 3 * B * pl->p * pl->tab_len() * pl->amp());
     const size_t pass_partials = pl->small() ? 0 : 3 * B * (size_t)device_sms();
@@ -389,29 +389,29 @@ void default_layer(int n, int T, int cbmin, int hbmax, int L2, int *L, int *K, b
     *L = (L2 < T && layer_passes(n, T, cbmin, hbmax, L2, L2, *K, v, false, big_last)) ? L2 : T;
 }
 
-// Default plan of a gradient evaluation with two high passes per layer: equal
-// high groups (8 qubits, or 7) for both sweeps, so that the forward's last group
-// is the adjoint's and a turnaround pass joins them (5 S of traffic become 2 S).
-// The low passes take what is left: the forward's the bits of two register
-// stages where its groups then still end alike, the adjoint's a whole tile where
-// its larger last group does. Against the separate defaults (complex64, p = 2,
-// ms): n = 23 0.319 -> 0.311, 24 0.501 -> 0.475, 25 0.874 -> 0.801, 26 1.521 ->
-// 1.413, 27 2.84 -> 2.64, 28 5.56 -> 5.11; complex128 n = 24 7.49 -> 7.39. With
-// three high passes the equal split costs more passes' stages than it saves
-// (n = 29 12.9 -> 13.9, n = 30 has a turnaround without it).
-bool turn_layers(const aaqaoa_plan *pl, std::vector<Pass> &g, std::vector<Pass> &b)
+// The forward passes of a gradient evaluation. With two high passes per adjoint
+// layer they are chosen to end on the adjoint's last group, so that a turnaround
+// pass joins the sweeps (5 S of traffic become 2 S): two high groups, the last one
+// with the adjoint's q qubits, the low pass n - 2q or one fewer (one fewer where
+// that spares it the third register stage, or fills it less: 11 qubits beat 12).
+// Energies keep the plan that is best for them. Complex64, p = 2, ms, against the
+// energy's plan: n = 22 0.224 -> 0.220, 24 0.501 -> 0.475, 26 1.521 -> 1.413, 27
+// 2.84 -> 2.64, 28 5.56 -> 5.11. With three high passes an equal split costs more
+// in its passes than it saves (n = 29 12.9 -> 13.9; n = 30 turns without it).
+void gradient_passes(aaqaoa_plan *pl)
 {
-    int T1, T2, CB1, CB2, HB1, HB2;
-    pass_geometry(pl->c128, 1, &T1, &CB1, &HB1);
-    pass_geometry(pl->c128, 2, &T2, &CB2, &HB2);
-    const int n = pl->n, L1 = low_two_stage_bits(pl->c128, 1), L2 = low_two_stage_bits(pl->c128, 2);
-    const int r = std::min(2 * HB2, (n - L2) & ~1), L = n - r;
-    if (r < 14 || L > T2)
-        return false;
-    const int Lb = (n - T2 + 1) / 2 == r / 2 ? T2 : L;
-    const int Lf = (n - L1) / 2 == r / 2 && (n - L1 + 1) / 2 <= HB1 ? L1 : L;
-    return layer_passes(n, T1, CB1, HB1, L1, Lf, 2, g, false, false, pl->half()) &&
-           layer_passes(n, T2, CB2, HB2, L2, Lb, 2, b, false, true, pl->half());
+    pl->gpasses = pl->passes;
+    if (pl->bwd_passes.size() != 3 || pl->bwd_passes[0].cluster || pl->n < (pl->c128 ? 21 : 22))
+        return;
+    int T, CB, HB;
+    pass_geometry(pl->c128, 1, &T, &CB, &HB);
+    const int L1 = low_two_stage_bits(pl->c128, 1), q = pl->bwd_passes[2].qubits;
+    int L = pl->n - 2 * q;
+    if (L - 1 == L1 || L == T - 1)
+        L--;
+    std::vector<Pass> g;
+    if (L <= T && layer_passes(pl->n, T, CB, HB, L1, L, 2, g, false, false, pl->half()))
+        pl->gpasses = g;
 }
 
 void build_passes(aaqaoa_plan *pl)
@@ -428,13 +428,7 @@ void build_passes(aaqaoa_plan *pl)
         default_layer(pl->n, T, CB, HB, L2, &L, &K, nv == 2);
         layer_passes(pl->n, T, CB, HB, L2, L, K, nv == 1 ? pl->passes : pl->bwd_passes, false, nv == 2, pl->half());
     }
-    std::vector<Pass> g, b;
-    if (turn_layers(pl, g, b)) {
-        pl->gpasses = g;
-        pl->bwd_passes = b;
-    } else {
-        pl->gpasses = pl->passes;
-    }
+    gradient_passes(pl);
 }
 
 // table `kind` (0 exact, 1 forward-scaled, 2 inverse) of a call with B points
@@ -841,15 +835,17 @@ int check_ready(aaqaoa_plan *pl, int obs, bool grad, int B)
 }
 
 // parameters already in device memory (point-major B x p)
-int enqueue_params(aaqaoa_plan *pl, int B, const double *d_gamma, const double *d_beta)
+// grad: the adjoint's tables too
+int enqueue_params(aaqaoa_plan *pl, int B, const double *d_gamma, const double *d_beta, bool grad)
 {
     (void)cudaGetLastError();  // a stale error of an unrelated earlier call must not be reported here
     pl->cur_gamma = d_gamma;
     ProfScope ps_(pl, PK_PARAMS, 0.0);
-    CKL(launch_params(pl->c128, B, pl->p, pl->tab_len(), pl->n, d_gamma, d_beta, pl->d_tab(), pl->d_cs(), pl->stream),
+    CKL(launch_params(pl->c128, B, pl->p, pl->tab_len(), pl->n, d_gamma, d_beta, pl->d_tab(), pl->d_cs(),
+                      pl->small() ? 1 : grad ? 6 : 2, pl->ising, pl->d_out(), (long long)B * pl->out_stride(),
+                      pl->stream),
         "parameter tables");
     pl->launches++;
-    CK(cudaMemsetAsync(pl->d_out(), 0, (size_t)B * pl->out_stride() * sizeof(double), pl->stream));
     return AAQAOA_OK;
 }
 
@@ -1057,7 +1053,7 @@ int enqueue_expect(aaqaoa_plan *pl, int B, const double *d_gamma, const double *
         pl->state_valid = true;
         return enqueue_aggregate(pl, obs, agg);
     }
-    int r = enqueue_params(pl, B, d_gamma, d_beta);
+    int r = enqueue_params(pl, B, d_gamma, d_beta, false);
     if (r)
         return r;
     if (pl->small()) {
@@ -1086,7 +1082,7 @@ int enqueue_state(aaqaoa_plan *pl)
     CircuitPlan q;
     if (pl->small() && use_circuit(pl, 1, false, true, &q))
         return enqueue_circuit(pl, 1, dg, db, AAQAOA_OBS_FULL, false, true, q);
-    int r = enqueue_params(pl, 1, dg, db);
+    int r = enqueue_params(pl, 1, dg, db, false);
     if (r)
         return r;
     if (pl->small()) {
@@ -1107,7 +1103,7 @@ int enqueue_grad(aaqaoa_plan *pl, const double *d_gamma, const double *d_beta, i
             pl->state_valid = false;
         return enqueue_circuit(pl, B, d_gamma, d_beta, obs, true, false, q);
     }
-    int r = enqueue_params(pl, B, d_gamma, d_beta);
+    int r = enqueue_params(pl, B, d_gamma, d_beta, true);
     if (r)
         return r;
     if (pl->small()) {
@@ -1571,15 +1567,10 @@ int aaqaoa_set_workspace(aaqaoa_plan *pl, void *device_ptr, size_t bytes, int ba
 // A layer's qubits per pass (the low pass's qubit count L and the number K of
 // high passes) for the forward (nv = 1) and the two-vector adjoint (nv = 2)
 // passes. 0 selects the default of build_passes().
-static int set_layers(aaqaoa_plan *pl, const int plan4[4])
+static int set_layers(aaqaoa_plan *pl, const int plan4[4], bool forced = false)
 {
     if (pl->small())
         return AAQAOA_OK;
-    if (!plan4[0] && !plan4[1] && !plan4[2] && !plan4[3]) {
-        build_passes(pl);
-        pl->state_valid = false;
-        return build_maps(pl);
-    }
     std::vector<Pass> v[2];
     for (int nv = 1; nv <= 2; nv++) {
         int T, CB, HB, L, K;
@@ -1596,6 +1587,8 @@ static int set_layers(aaqaoa_plan *pl, const int plan4[4])
     }
     pl->passes = pl->gpasses = v[0];
     pl->bwd_passes = v[1];
+    if (!forced)
+        gradient_passes(pl);
     pl->state_valid = false;
     return build_maps(pl);
 }
@@ -1619,9 +1612,10 @@ int aaqaoa_set_pass_plan(aaqaoa_plan *pl, int fwd_low, int fwd_high, int bwd_low
     if (fwd_low < 0 || fwd_high < 0 || bwd_low < 0 || bwd_high < 0)
         return fail(AAQAOA_ERR_INVALID_ARG, "negative pass-plan entry");
     const int plan4[4] = {fwd_low, fwd_high, bwd_low, bwd_high};
-    const int r = set_layers(pl, plan4);
+    const bool forced = fwd_low || fwd_high || bwd_low || bwd_high;
+    const int r = set_layers(pl, plan4, forced);
     if (!r)
-        pl->forced = fwd_low || fwd_high || bwd_low || bwd_high;
+        pl->forced = forced;
     return r;
 }
 
@@ -1746,16 +1740,15 @@ int aaqaoa_autotune(aaqaoa_plan *pl, int *plan4)
                 b[l] = 0.2 + 0.05 * l;
             }
             if ((r = upload_params(pl, 1, g.data(), b.data())) ||
-                (r = enqueue_params(pl, 1, pl->d_params(), pl->d_params() + pl->p)))
+                (r = enqueue_params(pl, 1, pl->d_params(), pl->d_params() + pl->p, pl->ws_grad)))
                 return r;
-            const FwdMode fm = pl->ws_grad ? FWD_GRAD : FWD_ENERGY;
             std::array<int, 4> best{0, 0, 0, 0};
             float best_ms = 1e30f;
             for (auto &c : layer_candidates(pl, 1)) {
                 const int cand[4] = {c[0], c[1], 0, 0};
                 if ((r = set_layers(pl, cand)))
                     return r;
-                auto run = [&]() { return enqueue_forward(pl, 1, AAQAOA_OBS_FULL, fm); };
+                auto run = [&]() { return enqueue_forward(pl, 1, AAQAOA_OBS_FULL, FWD_ENERGY); };
                 time_ms(pl->stream, run, 1);
                 const float ms = time_ms(pl->stream, run, 2);
                 if (ms < best_ms) {
@@ -1770,9 +1763,10 @@ int aaqaoa_autotune(aaqaoa_plan *pl, int *plan4)
                     const int cand[4] = {best[0], best[1], c[0], c[1]};
                     if ((r = set_layers(pl, cand)))
                         return r;
-                    if ((r = enqueue_forward(pl, 1, AAQAOA_OBS_FULL, FWD_GRAD)))
-                        return r;
-                    auto run = [&]() { return enqueue_backward(pl, 1, AAQAOA_OBS_FULL); };
+                    auto run = [&]() {  // both sweeps: the forward's groups follow the adjoint's
+                        const int q = enqueue_forward(pl, 1, AAQAOA_OBS_FULL, FWD_GRAD);
+                        return q ? q : enqueue_backward(pl, 1, AAQAOA_OBS_FULL);
+                    };
                     time_ms(pl->stream, run, 1);
                     const float ms = time_ms(pl->stream, run, 2);
                     if (ms < best_ms) {
@@ -1784,22 +1778,6 @@ int aaqaoa_autotune(aaqaoa_plan *pl, int *plan4)
             }
             if ((r = set_layers(pl, best.data())))
                 return r;
-            if (pl->ws_grad) {  // the default may give the two sweeps of a gradient matching groups
-                auto both = [&]() {
-                    const int q = enqueue_forward(pl, 1, AAQAOA_OBS_FULL, FWD_GRAD);
-                    return q ? q : enqueue_backward(pl, 1, AAQAOA_OBS_FULL);
-                };
-                time_ms(pl->stream, both, 1);
-                const float tuned = time_ms(pl->stream, both, 2);
-                const std::array<int, 4> dflt{0, 0, 0, 0};
-                if ((r = set_layers(pl, dflt.data())))
-                    return r;
-                time_ms(pl->stream, both, 1);
-                if (time_ms(pl->stream, both, 2) <= tuned)
-                    best = dflt;
-                else if ((r = set_layers(pl, best.data())))
-                    return r;
-            }
             std::vector<double> rows;
             if ((r = fetch_out(pl, 1, rows)))  // a device timeout during tuning surfaces here
                 return r;
@@ -2377,10 +2355,10 @@ extern "C" int aaqaoa_expect_static(aaqaoa_plan *pl, const double *gamma, const 
     off = align256(off + (size_t)pl->out_stride() * sizeof(double));
     double *d_par = reinterpret_cast<double *>(base + off);
     off = align256(off + 2 * (size_t)p * sizeof(double));
-    double2 *d_cs = reinterpret_cast<double2 *>(base + off);
-    off = align256(off + (size_t)p * sizeof(double2));
-    void *d_tab = base + off;  // exact, forward-scaled and inverse tables
-    off = align256(off + 3 * (size_t)p * pl->tab_len() * pl->amp());
+    MixRow *d_cs = reinterpret_cast<MixRow *>(base + off);
+    off = align256(off + (size_t)p * sizeof(MixRow));
+    void *d_tab = base + off;  // exact and forward-scaled tables
+    off = align256(off + 2 * (size_t)p * pl->tab_len() * pl->amp());
     double *d_part = reinterpret_cast<double *>(base + off);
     off = align256(off + 3 * (size_t)device_sms() * sizeof(double));
     if (off > STATIC_FIXED_BYTES)
@@ -2414,7 +2392,9 @@ extern "C" int aaqaoa_expect_static(aaqaoa_plan *pl, const double *gamma, const 
         CK(cudaStreamSynchronize(st));
         return AAQAOA_OK;
     }
-    CKL(launch_params(pl->c128, 1, p, pl->tab_len(), pl->n, d_par, d_par + p, d_tab, d_cs, st), "parameter tables");
+    CKL(launch_params(pl->c128, 1, p, pl->tab_len(), pl->n, d_par, d_par + p, d_tab, d_cs, pl->small() ? 1 : 2, false,
+                      d_out, pl->out_stride(), st),
+        "parameter tables");
 
     if (pl->small()) {
         SmallArgs s;

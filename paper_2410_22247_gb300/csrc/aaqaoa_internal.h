@@ -48,6 +48,14 @@ struct GraphFns {
     CutFn obs[2];
 };
 
+// One mixer layer of one parameter point, from k_params: cos and sin of beta, the
+// rotation's ratio t and dropped factor f (see rot; Ising plans: the cot form when
+// |sin| > |cos|), and f's powers. Of the inverse layer: -t, and -f when |sin| > |cos|.
+struct MixRow {
+    double c, s, t, f;
+    double pw[MAXN + 2];
+};
+
 // Operations of one tiled pass over the statevector(s).
 enum PostOp : int {
     POST_REDUCE = 1,      // acc0 += |phi|^2 O(x)                 (energy)
@@ -93,7 +101,7 @@ struct PassArgs {
     double sign2;     // the second layer of a fused pass: the same, or 0 for sign_s
     double amp0;      // 2^(-n/2) for the generated |+>^n
     const void *tab;  // this pass's phase tables [B][p][tab_len]: forward-scaled or inverse
-    const double2 *cs;  // [B][p] (cos beta_l, sin beta_l)
+    const MixRow *cs;   // [B][p]
     double *partials; // [3][B][grid]
     unsigned *counter;  // last-block counter (zero between launches)
     double *out;      // [B][out_stride]
@@ -124,7 +132,7 @@ struct SmallArgs {
     int write_state;   // also store psi_p to `state`
     double amp0;
     const void *tab;
-    const double2 *cs;
+    const MixRow *cs;
     double *out;       // [B][out_stride]
     int out_stride;
     void *state;       // [B][2^n] (optional)
@@ -199,7 +207,8 @@ int low_two_stage_bits(bool c128, int nv);
 int device_sms();
 int pass_grid(long long total_tiles);
 int launch_params(bool c128, int B, int p, int tab_len, int n, const double *d_gamma, const double *d_beta,
-                  void *d_tab, double2 *d_cs, cudaStream_t st);
+                  void *d_tab, MixRow *d_cs, int kinds, bool ising, double *d_out, long long out_count,
+                  cudaStream_t st);
 int launch_pass(bool c128, int nv_kernel, const CUtensorMap &m0, const CUtensorMap &m1, const PassArgs &a,
                 int grid, cudaStream_t st);
 // the pass instantiations, one unit each: complex64 cut-function plans
@@ -224,7 +233,7 @@ int launch_agg_fused(bool c128, const AggArgs &a, cudaStream_t st, int grid);
 int launch_agg_terms(bool c128, const AggArgs &a, cudaStream_t st, int grid);
 int agg_grid(bool c128);
 size_t small_multi_smem_bytes(bool c128, int max_n, int max_tab);
-int launch_untwist(bool c128, void *psi, int n, int bits, const double2 *cs, int p, int noshift, cudaStream_t st);
+int launch_untwist(bool c128, void *psi, int n, int bits, const MixRow *cs, int p, int noshift, cudaStream_t st);
 int launch_maxcut(const CostFn &cost, int n, unsigned long long *d_key, cudaStream_t st);
 size_t sample_chunk_count(int n);
 int launch_sample(bool c128, const void *psi, int n, int bits, double *d_sums, double *d_total, int K, const double *d_u,

@@ -282,21 +282,14 @@ __global__ void __maxnreg__((Geo<float, 2>::MAXREG))
         X.amp0 = (R)A.amp0;
         X.cot = X.cot2 = false;
         {
-            const double2 csd = A.cs[A.layer];
-            const double cbv = csd.x, sbv = A.sign_s * csd.y;
-            const bool shifted = fabs(sbv) > fabs(cbv);
-            X.tq = shifted ? (R)(-cbv / sbv) : (R)(sbv / cbv);
-            const double f = shifted ? sbv : cbv;
-            double fj = 1.0, fn = 1.0;
-            for (int i = 0; i < A.n; i++) {
-                if (i < A.j0)
-                    fj *= f;
-                fn *= f;
-            }
-            X.f = (R)f;
+            const MixRow &mr = A.cs[A.layer];
+            const bool neg = A.sign_s < 0 && fabs(mr.s) > fabs(mr.c);
+            X.tq = (R)(A.sign_s * mr.t);
+            const double fn = neg && (A.n & 1) ? -mr.pw[A.n] : mr.pw[A.n];
+            X.f = (R)(neg ? -mr.f : mr.f);
             X.fn = (R)fn;
             X.fn2 = (R)(fn * fn);
-            X.scale0 = (R)fj;
+            X.scale0 = (R)(neg && (A.j0 & 1) ? -mr.pw[A.j0] : mr.pw[A.j0]);
         }
         const uint32_t sb2 = G::swz(stage_base<G, 2>((uint32_t)tid));
         constexpr uint32_t LOW2 = split_low<G, 2>();
@@ -431,65 +424,81 @@ __global__ void __maxnreg__((Geo<float, 2>::MAXREG))
 }
 
 // ------------------------------------------------------ parameter tables
-// The factor dropped by one tan/cot butterfly of the (inverse, sign = -1)
-// mixer: cos beta if |sin| <= |cos| else sign * sin beta. Mirrors the choice
-// the pass kernel makes from the same (cos, sin) pair.
-__device__ __forceinline__ double butterfly_factor(double cn, double sn, double sign)
-{
-    const double s = sign * sn;
-    return fabs(s) > fabs(cn) ? s : cn;
-}
-
-__device__ __forceinline__ double ipow(double f, int k)
-{
-    double r = 1.0;
-    for (int i = 0; i < k; i++)
-        r *= f;
-    return r;
-}
-
-// Three phase tables per (point, layer), each exp(-i ((gamma_l c) mod 2 pi))
-// for c = 0..tab_len-1 computed in FP64 and rounded once:
-//   tab[0]: exact, for the whole-circuit kernel;
+// Phase tables per (point, layer), each exp(-i ((gamma_l c) mod 2 pi)) for c =
+// 0..tab_len-1 computed in FP64 and rounded once (kinds: a bit per table):
+//   tab[0]: exact, for the whole-circuit kernel of Ising plans;
 //   tab[1]: times f_{l-1}^n, the factor the previous layer's n tan/cot
 //           butterflies left on the state (forward passes);
 //   tab[2]: conjugated and times f'_l^n for the inverse layer (adjoint).
-// cs[b][l] = (cos beta_l, sin beta_l) in FP64.
+// rows[b][l]: the mixer layers. out: the results' accumulators, zeroed.
+// A chain of FP64 operations at the head of every call, so few of them: a block
+// first gets f^n of the layers its entries need, once each, and an entry is one
+// sine and cosine (three of each per entry, with the library's range reduction
+// and n-step power chains, took 16-20 us).
 template <typename R>
-__global__ void k_params(int B, int p, int tab_len, int n, const double *__restrict__ gamma,
-                         const double *__restrict__ beta, typename CT<R>::T *__restrict__ tab,
-                         double2 *__restrict__ cs)
+__global__ void __launch_bounds__(256) k_params(int B, int p, int tab_len, int n, int kinds, int ising,
+                                                const double *__restrict__ gamma, const double *__restrict__ beta,
+                                                typename CT<R>::T *__restrict__ tab, MixRow *__restrict__ rows,
+                                                double *__restrict__ out, long long out_count)
 {
     using C = typename CT<R>::T;
-    const double TWO_PI = 6.283185307179586476925286766559;
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const long long N = (long long)B * p * tab_len;
+    __shared__ double s_fs[258], s_fb[258];
+    const long long i0 = (long long)blockIdx.x * 256, i = i0 + threadIdx.x, N = (long long)B * p * tab_len;
+    const long long BP = (long long)B * p;
+    auto rotation = [&](long long bl, double &c, double &s, double &t, double &f) -> bool {  // |sin| > |cos|
+        const double2 z = phase_sincos<double>(beta[bl]);
+        c = z.x;
+        s = z.y;
+        const bool sh = fabs(s) > fabs(c);
+        mix_ratio<R>(sh ? (ising ? c : -c) : s, sh ? s : c, t, f);
+        return sh;
+    };
+    // layers bl0 .. : the ones before (fs) and of (fb) this block's entries
+    const long long bl0 = i0 / tab_len, bl1 = i0 + 255 < N ? (i0 + 255) / tab_len : BP - 1;
+    for (long long bl = bl0 - 1 + threadIdx.x; bl <= bl1; bl += 256) {
+        if (bl < 0 || bl0 >= BP)
+            continue;
+        double c, s, t, f;
+        const bool sh = rotation(bl, c, s, t, f);
+        double fn = 1.0, q = f;
+        for (int k = n; k; k >>= 1) {
+            if (k & 1)
+                fn *= q;
+            q *= q;
+        }
+        if (bl < bl1)
+            s_fs[bl - bl0 + 1] = fn;  // for the next layer's entries
+        if (bl >= bl0)
+            s_fb[bl - bl0] = sh && (n & 1) ? -fn : fn;
+    }
+    __syncthreads();
     if (i < N) {
         const long long bl = i / tab_len;
-        const int c = (int)(i - bl * tab_len);
-        const int l = (int)(bl % p);
-        double ang = fmod(gamma[bl] * (double)c, TWO_PI);
-        if (ang < 0.0)
-            ang += TWO_PI;
-        double sn, cn;
-        sincos(ang, &sn, &cn);
-        double fs = 1.0;
-        if (l > 0) {
-            double bs, bc;
-            sincos(beta[bl - 1], &bs, &bc);
-            fs = ipow(butterfly_factor(bc, bs, 1.0), n);
-        }
-        double bs, bc;
-        sincos(beta[bl], &bs, &bc);
-        const double fb = ipow(butterfly_factor(bc, bs, -1.0), n);
-        tab[i] = mkc<C>((R)cn, (R)(-sn));
-        tab[N + i] = mkc<C>((R)(cn * fs), (R)(-sn * fs));
-        tab[2 * N + i] = mkc<C>((R)(cn * fb), (R)(sn * fb));
+        const double2 z = phase_sincos<R>(gamma[bl] * (double)(i - bl * tab_len));
+        const double fs = bl % p ? s_fs[bl - bl0] : 1.0, fb = s_fb[bl - bl0];
+        if (kinds & 1)
+            tab[i] = mkc<C>((R)z.x, (R)(-z.y));
+        if (kinds & 2)
+            tab[N + i] = mkc<C>((R)(z.x * fs), (R)(-z.y * fs));
+        if (kinds & 4)
+            tab[2 * N + i] = mkc<C>((R)(z.x * fb), (R)(z.y * fb));
     }
-    if (i < (long long)B * p) {
-        double sn, cn;
-        sincos(beta[i], &sn, &cn);
-        cs[i] = make_double2(cn, sn);
+    const long long step = (long long)gridDim.x * 256;
+    for (long long k = i; k < out_count; k += step)
+        out[k] = 0.0;
+    for (long long bl = step - 1 - i; bl < BP; bl += step) {  // (the last blocks: the first ones have tables)
+        MixRow &r = rows[bl];
+        double c, s, t, f;
+        rotation(bl, c, s, t, f);
+        r.c = c;
+        r.s = s;
+        r.t = t;
+        r.f = f;
+        double q = 1.0;
+        for (int k = 0; k <= n; k++) {
+            r.pw[k] = q;
+            q *= f;
+        }
     }
 }
 
@@ -552,8 +561,8 @@ __global__ void __launch_bounds__(256) k_small(const __grid_constant__ SmallArgs
             for (int i = tid; i < A.tab_len; i += NT)
                 tab[i] = src[i];
         }
-        const double2 cs = A.cs[(size_t)b * A.p + l];
-        const R c = (R)cs.x, s = (R)cs.y;
+        const MixRow &cs = A.cs[(size_t)b * A.p + l];
+        const R c = (R)cs.c, s = (R)cs.s;
         __syncthreads();
         if (ising) {  // exp(-i gamma_l C(x)), the angle in FP64
             const double gl = A.gam[(size_t)b * A.p + l];
@@ -591,8 +600,8 @@ __global__ void __launch_bounds__(256) k_small(const __grid_constant__ SmallArgs
         lam[x] = mkc<C>(phi[x].x * o, phi[x].y * o);
     }
     for (int l = A.p - 1; l >= 0; l--) {
-        const double2 cs = A.cs[(size_t)b * A.p + l];
-        const R c = (R)cs.x, s = (R)(-cs.y);
+        const MixRow &cs = A.cs[(size_t)b * A.p + l];
+        const R c = (R)cs.c, s = (R)(-cs.s);
         double gb = 0.0, gg = 0.0;
         for (int q = 0; q < n; q++) {
             __syncthreads();
@@ -1099,14 +1108,16 @@ int pass_grid(long long total_tiles)
 }
 
 int launch_params(bool c128, int B, int p, int tab_len, int n, const double *d_gamma, const double *d_beta,
-                  void *d_tab, double2 *d_cs, cudaStream_t st)
+                  void *d_tab, MixRow *d_cs, int kinds, bool ising, double *d_out, long long out_count, cudaStream_t st)
 {
     const long long total = (long long)B * p * (tab_len > 1 ? tab_len : 1);
     const int grid = (int)((total + 255) / 256);
     if (c128)
-        k_params<double><<<grid, 256, 0, st>>>(B, p, tab_len, n, d_gamma, d_beta, (double2 *)d_tab, d_cs);
+        k_params<double><<<grid, 256, 0, st>>>(B, p, tab_len, n, kinds, ising, d_gamma, d_beta, (double2 *)d_tab, d_cs,
+                                               d_out, out_count);
     else
-        k_params<float><<<grid, 256, 0, st>>>(B, p, tab_len, n, d_gamma, d_beta, (float2 *)d_tab, d_cs);
+        k_params<float><<<grid, 256, 0, st>>>(B, p, tab_len, n, kinds, ising, d_gamma, d_beta, (float2 *)d_tab, d_cs,
+                                              d_out, out_count);
     return (int)cudaGetLastError();
 }
 
@@ -1220,12 +1231,12 @@ int launch_small(bool c128, const SmallArgs &a, int B, cudaStream_t st)
 // place, and psi(~x) = psi(x) fills the buffer's other half. Ising plans keep
 // the whole state and never rotate by beta_l - pi/2 (noshift): K = 0.
 template <typename R>
-__global__ void k_untwist(typename CT<R>::T *psi, int n, int bits, const double2 *cs, int p, int noshift)
+__global__ void k_untwist(typename CT<R>::T *psi, int n, int bits, const MixRow *cs, int p, int noshift)
 {
     using C = typename CT<R>::T;
     int K = 0;
     for (int l = 0; l < p && !noshift; l++)
-        K += fabs(cs[l].y) > fabs(cs[l].x) ? 1 : 0;
+        K += fabs(cs[l].s) > fabs(cs[l].c) ? 1 : 0;
     const int ph = (4 - ((n * K) & 3)) & 3;  // (-i)^(nK) = i^ph
     auto turn = [](C v, int e) -> C {          // v * i^e
         e &= 3;
@@ -1458,7 +1469,7 @@ int launch_sample(bool c128, const void *psi, int n, int bits, double *d_sums, d
     return (int)cudaGetLastError();
 }
 
-int launch_untwist(bool c128, void *psi, int n, int bits, const double2 *cs, int p, int noshift, cudaStream_t st)
+int launch_untwist(bool c128, void *psi, int n, int bits, const MixRow *cs, int p, int noshift, cudaStream_t st)
 {
     const int grid = 4 * device_sms();
     if (c128)

@@ -167,6 +167,62 @@ __device__ __forceinline__ void dot_acc(C &acc, const C &u, const C &v)
     }
 }
 
+// cos x, sin x in FP64 for the phase tables, by reduction to |r| <= pi/4 (x -
+// k pi/2 with pi/2 in two parts, fused) and the Taylor series there: the
+// library's function costs 3 us at the head of a launch. float: a relative
+// error below 1e-10, rounded once to the table's precision; double: 1e-16.
+template <typename R>
+__device__ __noinline__ double2 phase_sincos(double x)  // (cos, sin)
+{
+    const double k = rint(x * 0.63661977236758134308);
+    if (!(fabs(k) < 1e9)) {
+        double sn, cn;
+        sincos(x, &sn, &cn);
+        return make_double2(cn, sn);
+    }
+    double r = fma(k, -1.5707963267948965580, x);
+    r = fma(k, -6.1232339957367660359e-17, r);
+    const double s = r * r;
+    double ps, pc;
+    if constexpr (std::is_same<R, float>::value) {
+        ps = fma(s, -1.0 / 39916800.0, 1.0 / 362880.0);
+        pc = fma(s, 1.0 / 479001600.0, -1.0 / 3628800.0);
+    } else {
+        ps = fma(s, -1.0 / 1307674368000.0, 1.0 / 6227020800.0);
+        pc = fma(s, 1.0 / 20922789888000.0, -1.0 / 87178291200.0);
+        ps = fma(ps, s, -1.0 / 39916800.0);
+        pc = fma(pc, s, 1.0 / 479001600.0);
+        ps = fma(ps, s, 1.0 / 362880.0);
+        pc = fma(pc, s, -1.0 / 3628800.0);
+    }
+    ps = fma(ps, s, -1.0 / 5040.0);
+    pc = fma(pc, s, 1.0 / 40320.0);
+    ps = fma(ps, s, 1.0 / 120.0);
+    pc = fma(pc, s, -1.0 / 720.0);
+    ps = fma(ps, s, -1.0 / 6.0);
+    pc = fma(pc, s, 1.0 / 24.0);
+    pc = fma(pc, s, -0.5);
+    const double sr = fma(r * s, ps, r), cr = fma(s, pc, 1.0);
+    const int q = (int)(long long)k & 3;
+    const double a = (q & 1) ? cr : sr, b = (q & 1) ? sr : cr;
+    return make_double2(((q + 1) & 2) ? -b : b, (q & 2) ? -a : a);
+}
+
+// The rotation of one mixer layer from (cos, sin) of its angle: u / v = t, the
+// ratio the butterflies use (rounded to the amplitude type), and f, the factor one
+// butterfly with that t drops: 1 / sqrt(1 + t^2) with v's sign, to first order in
+// the rounding error t v - u. f and t belong together: with f = cos beta the norm
+// drifts by the rounding of t in every butterfly.
+template <typename R>
+__device__ __forceinline__ void mix_ratio(double u, double v, double &t, double &f)
+{
+    if constexpr (std::is_same<R, float>::value)
+        t = (double)((float)u / (float)v);
+    else
+        t = u / v;
+    f = v - v * (u * fma(t, v, -u));
+}
+
 // Im(conj(l) f)
 template <typename C>
 __device__ __forceinline__ auto im_conj_mul(C l, C f) -> decltype(l.x) { return l.x * f.y - l.y * f.x; }
@@ -672,9 +728,8 @@ struct StageCtx {
     R amp0;        // 2^(-n/2), the amplitude of the generated |+>^n
     // turnaround pass (POST_LAMBDA, turn_keeps_phi): phi is not stored back,
     // the stored lambda carries kap = f^(2 j0 - n) instead (see run_stage),
-    // and the pass's dE/dbeta sums are multiplied by 1/kap once per point
+    // and the pass's dE/dbeta sums are divided by kap once per point
     R kap;
-    double ikap;
     R tq2, f2;     // fused pass: rotation of the second layer
     R run2;        // its f^j (the second layer starts on exact vectors: j = 0)
     bool cot, cot2;  // Ising plans: the layer (second layer) uses the cot form
@@ -1901,10 +1956,10 @@ __global__ void __maxnreg__((Geo<R, NV>::MAXREG))
             // that stash comes after a barrier thread 0 only reaches when done.
             const int lane = tid & 31, warp = tid >> 5;
             int pend_b = -1, tslot = 1, par = 1;
+            double kapd = 1.0, pend_kap = 1.0;  // turnaround: the factor of this point's stored lambda
             auto stash = [&](int b) {
                 double s0 = acc0.get(), s1 = acc1.get(), s2 = acc2.get();
-                if (turn_keeps_phi<R> && NV == 2 && (P.post & POST_LAMBDA))  // lambda carried kap
-                    s2 *= X.ikap;
+                pend_kap = kapd;
     #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) {
                     s0 += __shfl_xor_sync(0xffffffffu, s0, o);
@@ -1933,8 +1988,9 @@ __global__ void __maxnreg__((Geo<R, NV>::MAXREG))
                     }
                     A.partials[((size_t)0 * A.B + pend_b) * grid + blockIdx.x] = s0;
                     A.partials[((size_t)1 * A.B + pend_b) * grid + blockIdx.x] = s1;
-                    if (FUSE)
-                        A.partials[((size_t)2 * A.B + pend_b) * grid + blockIdx.x] = s2;
+                    if (FUSE)  // (lambda carried kap)
+                        A.partials[((size_t)2 * A.B + pend_b) * grid + blockIdx.x] =
+                            turn_keeps_phi<R> && NV == 2 && (P.post & POST_LAMBDA) ? s2 / pend_kap : s2;
                 }
                 pend_b = -1;
             };
@@ -1984,33 +2040,35 @@ __global__ void __maxnreg__((Geo<R, NV>::MAXREG))
                         for (int i = tid; i < A.tab_len; i += NTHR)
                             dst[i] = src[i];
                     }
-                    const double2 csd = A.cs[(size_t)b * A.p + A.layer];
-                    const double cbv = csd.x, sbv = A.sign_s * csd.y;
-                    const bool shifted = fabs(sbv) > fabs(cbv);  // rotate by beta - pi/2 (Ising: cot form)
+                    // the layer's rotation and the powers of its factor, ready in the
+                    // row (building them here, in FP64 on every thread, was 6 us per
+                    // launch and per point of a batch)
+                    const MixRow &mr = A.cs[(size_t)b * A.p + A.layer];
+                    const bool shifted = fabs(mr.s) > fabs(mr.c);  // rotate by beta - pi/2 (Ising: cot form)
+                    const bool neg = A.sign_s < 0 && shifted;      // the inverse's factor is -f
                     X.cot = IS && shifted;
-                    X.tq = shifted ? (R)((IS ? cbv : -cbv) / sbv) : (R)(sbv / cbv);
-                    const double f = shifted ? sbv : cbv;
-                    double fj = 1.0, fn = 1.0;
-                    for (int i = 0; i < A.n; i++) {
-                        if (i < A.j0)
-                            fj *= f;
-                        fn *= f;
-                    }
-                    X.f = (R)f;
+                    X.tq = (R)(A.sign_s * mr.t);
+                    const double fn = neg && (A.n & 1) ? -mr.pw[A.n] : mr.pw[A.n];
+                    X.f = (R)(neg ? -mr.f : mr.f);
                     X.fn = (R)fn;
                     X.fn2 = (R)(fn * fn);
-                    X.scale0 = (R)fj;
+                    X.scale0 = (R)(neg && (A.j0 & 1) ? -mr.pw[A.j0] : mr.pw[A.j0]);
                     if constexpr (turn_keeps_phi<R> && NV == 2) {
-                        X.kap = (R)(fj * fj / fn);  // f^(2 j0 - n), j0 = n - q
-                        X.ikap = fn / (fj * fj);
+                        if (A.post & POST_LAMBDA) {  // f^(2 j0 - n), j0 = n - q (a forward layer: no sign)
+                            const int e = 2 * A.j0 - A.n;
+                            kapd = e >= 0 ? mr.pw[e] : 1.0 / mr.pw[-e];
+                            if (X.cot && ((A.n - A.j0) & 1))  // a cot butterfly and its inverse: -(1 + t^2)
+                                kapd = -kapd;
+                            X.kap = (R)kapd;
+                        }
                     }
                     if constexpr (FUSE) {  // the second layer's rotation
-                        const double2 cs2 = A.cs[(size_t)b * A.p + A.layer2];
-                        const double c2 = cs2.x, s2 = (A.sign2 != 0.0 ? A.sign2 : A.sign_s) * cs2.y;
-                        const bool sh2 = fabs(s2) > fabs(c2);
+                        const MixRow &m2 = A.cs[(size_t)b * A.p + A.layer2];
+                        const double sg2 = A.sign2 != 0.0 ? A.sign2 : A.sign_s;
+                        const bool sh2 = fabs(m2.s) > fabs(m2.c);
                         X.cot2 = IS && sh2;
-                        X.tq2 = sh2 ? (R)((IS ? c2 : -c2) / s2) : (R)(s2 / c2);
-                        X.f2 = (R)(sh2 ? s2 : c2);
+                        X.tq2 = (R)(sg2 * m2.t);
+                        X.f2 = (R)(sg2 < 0 && sh2 ? -m2.f : m2.f);
                     }
                     cur_b = (int)b;
                 }

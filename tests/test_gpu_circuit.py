@@ -97,3 +97,23 @@ def test_pair_passes_match_oracle(n, plan, prec):
         assert np.max(np.abs(pl.statevector(g, b) - psi)) <= TOL[prec]
     pl.set_pass_plan()
     _check(pl.grad(g, b, "red"), O.energy_grad(n, e, g, b), prec)
+
+
+@pytest.mark.parametrize("plan", [(9, 2, 10, 2), (12, 2, 12, 2), (8, 2, 8, 2)])
+def test_ising_turnaround_over_odd_and_even_groups(plan):
+    """The turnaround's group has 5, 4 and 6 qubits; in the last layer of the
+    second angles |sin beta| > |cos beta| (the cot form, whose butterfly and
+    inverse change the sign once per qubit)."""
+    n, e = W.prufer_tree(20, 8)
+    w, h = W.ising_couplings(n, e, 9)
+    from paper_2410_22247_gb300.api import Plan
+    pl = Plan(n, e, 2, precision="c64", with_grad=True, couplings=w, fields=h)
+    pl.set_pass_plan(*plan)
+    adj = pl.schedule(True)
+    assert adj[0][2] == adj[0][3], "no turnaround"
+    scale = float(np.sum(np.abs(w)) + np.sum(np.abs(h)))
+    for beta in ([0.4, 0.3], [0.4, 1.2]):
+        E, dg, db = pl.grad([0.5, 0.8], beta, "full")
+        Er, dgr, dbr = O.ising_energy_grad(n, O.ising(e, w, h), np.array([0.5, 0.8]), np.array(beta))
+        assert abs(E - Er) <= 1e-5 * scale
+        assert np.max(np.abs(np.concatenate([dg - dgr, db - dbr]))) <= 1e-5 * scale
