@@ -1316,28 +1316,36 @@ int launch_maxcut(const CostFn &cost, int n, unsigned long long *d_key, cudaStre
 // if rounding leaves none). Of a flip-symmetric state the half with the top
 // bit clear is stored (bits = n - 1): psi(x) = psi(~x), and chunk c of the
 // other half holds the amplitudes of chunk nchunks - 1 - c backwards.
-constexpr int SAMPLE_BITS = 12;
+// A chunk holds 2^SB amplitudes, SB from 7 to 12: small enough that drawing reads
+// little (every sample sums its chunk in FP64: with 2^12 at n = 20, 4096 samples
+// took ~250 us), and at most 2^14 chunks while SB allows, for the scan's one block.
+__host__ __device__ inline int sample_bits(int n)
+{
+    const int sb = n - 14 < 7 ? 7 : n - 14 > 12 ? 12 : n - 14;
+    return n < sb ? n : sb;
+}
 
 template <typename R>
 __global__ void __launch_bounds__(256) k_sample_chunks(const typename CT<R>::T *psi, int n, int bits, double *sums)
 {
-    __shared__ double red[2][32];
-    const int cb = n < SAMPLE_BITS ? n : SAMPLE_BITS;
+    const int cb = sample_bits(n), lane = threadIdx.x & 31;
     const uint64_t all = 1ull << (n - cb), nchunks = bits < n ? all / 2 : all, len = 1ull << cb;
-    for (uint64_t c = blockIdx.x; c < nchunks; c += gridDim.x) {
+    const uint64_t warps = (uint64_t)gridDim.x * 8;
+    for (uint64_t c = (uint64_t)blockIdx.x * 8 + (threadIdx.x >> 5); c < nchunks; c += warps) {
         double s = 0.0;
-        for (uint64_t i = threadIdx.x; i < len; i += blockDim.x) {
+#pragma unroll 4
+        for (uint64_t i = lane; i < len; i += 32) {
             const typename CT<R>::T a = psi[c * len + i];
             s += (double)a.x * (double)a.x + (double)a.y * (double)a.y;
         }
-        double z = 0.0;
-        block_sum2<256>(s, z, red);
-        if (threadIdx.x == 0) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+            s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lane == 0) {
             sums[c] = s;
             if (bits < n)
                 sums[all - 1 - c] = s;
         }
-        __syncthreads();
     }
 }
 
@@ -1380,7 +1388,7 @@ __global__ void __launch_bounds__(256) k_sample_draw(const typename CT<R>::T *ps
     const int lane = threadIdx.x & 31;
     const int warp = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     const int nwarps = (int)((gridDim.x * blockDim.x) >> 5);
-    const int cb = n < SAMPLE_BITS ? n : SAMPLE_BITS;
+    const int cb = sample_bits(n);
     const uint64_t nchunks = 1ull << (n - cb), len = 1ull << cb, N = 1ull << n;
     const uint64_t per = len >= 32 ? len / 32 : 1;  // amplitudes per lane
     auto mass = [&](uint64_t x) {
@@ -1389,13 +1397,12 @@ __global__ void __launch_bounds__(256) k_sample_draw(const typename CT<R>::T *ps
     };
     for (int k = warp; k < K; k += nwarps) {
         const double t = u[k] * *total;
-        uint64_t lo = 0, hi = nchunks;  // last chunk with prefix <= t
-        while (hi - lo > 1) {
-            const uint64_t mid = lo + (hi - lo) / 2;
-            if (prefix[mid] <= t)
-                lo = mid;
-            else
-                hi = mid;
+        uint64_t lo = 0;  // last chunk with prefix <= t (prefix[0] = 0): the lanes probe 32 points a step
+        for (uint64_t width = nchunks; width > 1;) {
+            const uint64_t stepw = width >= 32 ? width / 32 : 1;
+            const bool in = (uint64_t)lane * stepw < width && prefix[lo + (uint64_t)lane * stepw] <= t;
+            lo += (uint64_t)(31 - __clz(__ballot_sync(0xffffffffu, in || lane == 0))) * stepw;
+            width = stepw;
         }
         const uint64_t c = lo;
         const double rem = t - prefix[c];
@@ -1448,14 +1455,15 @@ __global__ void __launch_bounds__(256) k_sample_draw(const typename CT<R>::T *ps
     }
 }
 
-size_t sample_chunk_count(int n) { return (size_t)1 << (n < SAMPLE_BITS ? 0 : n - SAMPLE_BITS); }
+size_t sample_chunk_count(int n) { return (size_t)1 << (n - sample_bits(n)); }
 
 int launch_sample(bool c128, const void *psi, int n, int bits, double *d_sums, double *d_total, int K, const double *d_u,
                   unsigned long long *d_x, int *d_cut, const CostFn &cost, cudaStream_t st)
 {
     const uint64_t nchunks = sample_chunk_count(n);
     const uint64_t own = bits < n && nchunks > 1 ? nchunks / 2 : nchunks;
-    const int g1 = (int)(own < (uint64_t)(8 * device_sms()) ? own : (uint64_t)(8 * device_sms()));
+    const uint64_t need = (own + 7) / 8;
+    const int g1 = (int)(need < (uint64_t)(8 * device_sms()) ? need : (uint64_t)(8 * device_sms()));
     const int g3 = (K + 7) / 8 < 4 * device_sms() ? (K + 7) / 8 : 4 * device_sms();
     if (c128)
         k_sample_chunks<double><<<g1, 256, 0, st>>>((const double2 *)psi, n, bits, d_sums);
