@@ -1449,6 +1449,7 @@ __host__ __device__ constexpr int flag_word(int load, int pre_phase, int pre_lam
     return (load ? 1 : 0) | (pre_phase ? 2 : 0) | (pre_lambda ? 4 : 0) | (write ? 8 : 0) | (post << 4);
 }
 constexpr int FW_FWD_FIRST = flag_word(0, 1, 0, 1, 0);                          // |+> generated, first phase
+constexpr int FW_FWD_PHASE = flag_word(1, 1, 0, 1, 0);                          // an unfused layer starts
 constexpr int FW_FWD_LAST = flag_word(1, 0, 0, 1, POST_REDUCE | POST_RESCALE);  // energy, state kept
 constexpr int FW_FWD_ENERGY = flag_word(1, 0, 0, 0, POST_REDUCE);               // energy only
 constexpr int FW_FWD_FUSED = flag_word(1, 0, 0, 1, POST_PHASE);
@@ -2153,11 +2154,13 @@ __global__ void __maxnreg__((Geo<R, NV>::MAXREG))
                 compiled = true;
             }
         };
-        // cut-function modes 1 and 3 and their Ising counterparts 4 and 5
+        // cut-function modes 1 (2: a graph per point) and 3, their Ising counterparts 4 and 5
         constexpr bool F32 = std::is_same<R, float>::value;
-        if constexpr (F32 && (MODE == 1 || MODE == 4) && NV == 1) {
+        if constexpr (F32 && (MODE == 1 || MODE == 2 || MODE == 4) && NV == 1) {
             run_if(integral_constant<int, FW_FWD_FIRST>{});
-            run_if(integral_constant<int, FW_FWD_LAST>{});
+            run_if(integral_constant<int, FW_FWD_PHASE>{});
+            if constexpr (MODE != 2)
+                run_if(integral_constant<int, FW_FWD_LAST>{});
             run_if(integral_constant<int, FW_FWD_ENERGY>{});
         }
         if constexpr (F32 && (MODE == 3 || MODE == 5) && NV == 1)
