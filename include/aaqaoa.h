@@ -368,8 +368,10 @@ int aaqaoa_expect_static(aaqaoa_plan *plan, const double *gamma, const double *b
  * optional class of every edge, edge_orbit, NULL when not given).
  * aaqaoa_prepare_multi validates every graph (same rules and errors as
  * aaqaoa_prepare, the detail names the graph) and copies all host arrays.
- * Graphs that fit one CTA (n <= 13 for C64, n <= 12 for C128) are evaluated
- * together by one kernel launch; each larger graph runs the tiled passes.
+ * Graphs are evaluated in groups of equal n, each group by one whole-circuit
+ * launch or by the tiled passes; those of fewer than 5 vertices together by one
+ * launch. (aaqaoa_multi_info's small_graphs counts n <= 13 for C64, n <= 12 for
+ * C128.)
  * The first aaqaoa_expect_multi call for an observable times a few ways of
  * spreading the large graphs over parallel CUDA streams (autotune; cached per
  * device and batch shape for the process; AAQAOA_AUTOTUNE=0 in the

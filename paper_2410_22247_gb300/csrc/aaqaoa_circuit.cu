@@ -277,19 +277,6 @@ __global__ void __launch_bounds__(512) k_circuit(const __grid_constant__ Circuit
     X.off = 0;
     const unsigned team = blockIdx.x >> c, teams = gridDim.x >> c;
 
-    // cut functions of the plan (vertices of a circuit plan fit 32 bits): all
-    // classes, so that no load waits for their number
-    const CutFn &cost = A.fns->cost, &obs = A.fns->obs[A.obs];
-    const int Kc = cost.K, Ko = obs.K;
-    for (int i = tid; i < MAXK * CIRC_MAXN; i += nt) {
-        const int k = i / CIRC_MAXN, u = i % CIRC_MAXN;
-        s_cost[i] = u < n ? (uint32_t)cost.nbr[k][u] : 0u;
-        s_obs[i] = u < n ? (uint32_t)obs.nbr[k][u] : 0u;
-    }
-    if (tid < MAXK) {
-        s_cw[tid] = cost.w[tid];
-        s_ow[tid] = obs.w[tid];
-    }
     if (tid == 0)
         s_stop = 0;
     if (CL)
@@ -298,6 +285,24 @@ __global__ void __launch_bounds__(512) k_circuit(const __grid_constant__ Circuit
         __syncthreads();
 
     for (unsigned b = team; b < (unsigned)A.B; b += teams) {
+        // cut functions (vertices of a circuit plan fit 32 bits): all classes, so
+        // that no load waits for their number
+        const bool fresh = b == team || A.per_point;
+        const GraphFns &fns = A.fns[A.per_point ? b : 0];
+        const CutFn &cost = fns.cost, &obs = fns.obs[A.obs];
+        const int Kc = cost.K, Ko = obs.K;
+        if (fresh) {
+            for (int i = tid; i < MAXK * CIRC_MAXN; i += nt) {
+                const int k = i / CIRC_MAXN, u = i % CIRC_MAXN;
+                s_cost[i] = u < n ? (uint32_t)cost.nbr[k][u] : 0u;
+                s_obs[i] = u < n ? (uint32_t)obs.nbr[k][u] : 0u;
+            }
+            if (tid < MAXK) {
+                s_cw[tid] = cost.w[tid];
+                s_ow[tid] = obs.w[tid];
+            }
+            __syncthreads();
+        }
         const double *gam = A.gamma ? A.gamma + (size_t)b * p : A.ang, *bet = A.gamma ? A.beta + (size_t)b * p : A.ang + p;
         // ------------------------------------------------ angles, tables
         // Warps take layers, lanes table entries; the first entry of a lane is
@@ -321,7 +326,7 @@ __global__ void __launch_bounds__(512) k_circuit(const __grid_constant__ Circuit
             lay[l] = CircLayer{f, fi, fn, (sh && (n & 1)) ? -fn : fn, t};
         }
         // cut values of the tile's states in both layouts
-        if (b == team)
+        if (fresh)
             for (int h = 0; h < (c > 0 ? 2 : 1); h++)
                 for (uint32_t i = 4u * tid; i < NL; i += 4u * nt) {
                     const int4 v = circ_cuts(s_cost, s_cw, Kc, m, circ_index(X, h, i));
@@ -652,7 +657,7 @@ static bool circuit_shape(bool c128, bool grad, int n, int p, int tab_len, int B
 //   97 / 147, 343 / 345, n = 16, 16 points 206 / 152.
 bool circuit_plan(bool c128, bool grad, int n, int p, int tab_len, int B, CircuitPlan *q)
 {
-    if (n < 5 || n > 20 || p > CIRC_MAXP)
+    if (n < CIRCUIT_MIN_QUBITS || n > 20 || p > CIRC_MAXP)
         return false;
     const int m = n - 1;
     int c = c128 ? (m <= 8 ? 0 : m <= 12 ? m - 8 : m <= 14 ? 4 : m <= 15 ? 5 : m <= 17 ? 6 : 7)

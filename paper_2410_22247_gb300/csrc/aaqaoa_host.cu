@@ -892,7 +892,9 @@ int enqueue_aggregate(aaqaoa_plan *pl, int obs, int agg)
 // pending test fault and a stored state beyond one CTA need the passes.
 bool use_circuit(const aaqaoa_plan *pl, int B, bool grad, bool state, CircuitPlan *q)
 {
-    if (pl->ising || pl->pt_dev || !circuit_plan(pl->c128, grad, pl->n, pl->p, pl->tab_len(), B, q))
+    if (pl->ising || !circuit_plan(pl->c128, grad, pl->n, pl->p, pl->tab_len(), B, q))
+        return false;
+    if (pl->pt_dev && q->c && !q->cluster)  // parallel groups: no launches that need every SM at once
         return false;
     if (pl->small())
         return true;
@@ -941,7 +943,8 @@ int enqueue_circuit(aaqaoa_plan *pl, int B, const double *d_gamma, const double 
     a.partials = pl->d_partials();
     a.bar = pl->d_team_bar();
     a.err = pl->d_err();
-    a.fns = reinterpret_cast<const GraphFns *>(pl->ws + pl->L.fns);
+    a.fns = pl->pt_dev ? pl->pt_dev : reinterpret_cast<const GraphFns *>(pl->ws + pl->L.fns);
+    a.per_point = pl->pt_dev ? 1 : 0;
     a.obs = obs;
     ProfScope ps_(pl, PK_SMALL, state ? (double)B * pl->state_bytes() : 0.0);
     CKL(launch_circuit(pl->c128, grad, a, q, pl->stream), "whole-circuit kernel");
@@ -2450,7 +2453,7 @@ extern "C" int aaqaoa_expect_static(aaqaoa_plan *pl, const double *gamma, const 
 }
 
 // ============================================== uneven multi-graph batches
-// Graphs with n up to the tile size run together in one k_small_multi launch;
+// Graphs of a handful of vertices run together in one k_small_multi launch;
 // larger graphs each own a tiled sub-plan. One evaluation of the batch is
 // captured into a CUDA graph whose large-graph work is spread over `branches`
 // parallel streams; the branch count is chosen by timing (autotune) on the
@@ -2461,8 +2464,9 @@ struct aaqaoa_multi {
     cudaStream_t stream = nullptr;  // the caller's stream: uploads, graph launch, downloads
     cudaStream_t cap = nullptr;     // private stream the evaluation is captured on
     std::vector<aaqaoa_plan *> plans;  // one per graph (validation + host tables)
-    std::vector<int> small_idx, large_idx;
-    // Graphs too large for one CTA run in groups of equal n: one batched pass
+    std::vector<int> small_idx, large_idx;  // by kernel: k_small_multi (a handful of vertices); groups
+    int small_count = 0;                    // graphs that fit one CTA
+    // The others run in groups of equal n: one whole-circuit launch or batched pass
     // sequence per group, point b of the group being its b-th graph. Rows of
     // the parameter and energy arrays follow `order` (small graphs first,
     // then each group's members), so a group's rows are contiguous.
@@ -2682,7 +2686,8 @@ int aaqaoa_prepare_multi(int G, const aaqaoa_graph_desc *graphs, int p, unsigned
             return fail(r, "graph %d: %s", gi, why.c_str());
         }
         m->plans.push_back(pl);
-        if (pl->small()) {
+        m->small_count += pl->small() ? 1 : 0;
+        if (pl->small() && pl->n < CIRCUIT_MIN_QUBITS) {
             SmallGraph sg;
             memset(&sg, 0, sizeof sg);
             sg.gi = (int)m->small_idx.size();  // its row: small graphs come first
@@ -2850,7 +2855,7 @@ int aaqaoa_multi_info(const aaqaoa_multi *m, int *G, int *small_graphs, int *bra
     if (!m)
         return fail(AAQAOA_ERR_INVALID_ARG, "multi is NULL");
     if (G) *G = m->G;
-    if (small_graphs) *small_graphs = (int)m->small_idx.size();
+    if (small_graphs) *small_graphs = m->small_count;
     if (branches) *branches = std::max(m->branches[0], m->branches[1]);
     if (launches_per_call) *launches_per_call = m->launches;
     return AAQAOA_OK;

@@ -159,6 +159,7 @@ struct CircuitArgs {
     unsigned *bar;       // c > 0: one arrival counter per point, zero between launches
     int *err;
     const GraphFns *fns; // the graph's cut functions (device memory)
+    int per_point;       // point b is its own graph, fns[b]
     int obs;
 };
 // the kernel's shape for a call, from circuit_plan (false: the call does not fit it)
@@ -167,6 +168,7 @@ struct CircuitPlan {
     int cluster;         // the 2^c CTAs are a cluster; else they exchange through global memory
     size_t smem;
 };
+constexpr int CIRCUIT_MIN_QUBITS = 5;   // 16 stored amplitudes
 constexpr int CIRCUIT_MAX_POINTS = 64;  // points of one launch when c > 0 (arrival counters)
 bool circuit_plan(bool c128, bool grad, int n, int p, int tab_len, int B, CircuitPlan *q);
 int launch_circuit(bool c128, bool grad, const CircuitArgs &a, const CircuitPlan &q, cudaStream_t st);
