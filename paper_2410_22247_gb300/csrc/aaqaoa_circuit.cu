@@ -277,12 +277,16 @@ __global__ void __launch_bounds__(512) k_circuit(const __grid_constant__ Circuit
     X.off = 0;
     const unsigned team = blockIdx.x >> c, teams = gridDim.x >> c;
 
+    // (a team's wait gave up in an earlier launch whose error was not fetched yet:
+    // its counters are not at zero)
     if (tid == 0)
-        s_stop = 0;
+        s_stop = !CL && c && *reinterpret_cast<volatile int *>(A.err) ? 1 : 0;
     if (CL)
         circ_cluster_sync();  // every CTA of the cluster runs before its memory is written
     else
         __syncthreads();
+    if (!CL && s_stop)
+        return;
 
     for (unsigned b = team; b < (unsigned)A.B; b += teams) {
         // cut functions (vertices of a circuit plan fit 32 bits): all classes, so
@@ -657,7 +661,7 @@ static bool circuit_shape(bool c128, bool grad, int n, int p, int tab_len, int B
 //   97 / 147, 343 / 345, n = 16, 16 points 206 / 152.
 bool circuit_plan(bool c128, bool grad, int n, int p, int tab_len, int B, CircuitPlan *q)
 {
-    if (n < CIRCUIT_MIN_QUBITS || n > 20 || p > CIRC_MAXP)
+    if (n < CIRCUIT_MIN_QUBITS || n > CIRCUIT_MAX_QUBITS || p > CIRC_MAXP)
         return false;
     const int m = n - 1;
     int c = c128 ? (m <= 8 ? 0 : m <= 12 ? m - 8 : m <= 14 ? 4 : m <= 15 ? 5 : m <= 17 ? 6 : 7)

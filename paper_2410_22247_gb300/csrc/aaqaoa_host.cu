@@ -1501,6 +1501,15 @@ int build_maps(aaqaoa_plan *pl)
     }
     for (size_t k = 0; k < pl->gpasses.size() && pl->ws_grad; k++) {
         Pass &ps = pl->gpasses[k];
+        size_t same = 0;  // an energy pass with the same tiles has the map already
+        while (same < pl->passes.size() && (pl->passes[same].s != ps.s || pl->passes[same].cb != ps.cb ||
+                                            pl->passes[same].pair != ps.pair))
+            same++;
+        if (same < pl->passes.size()) {
+            pl->map_gphi[k] = pl->map_phi[same];
+            ps.wide = pl->passes[same].wide;
+            continue;
+        }
         int r = make_map(&pl->map_gphi[k], pl->d_phi(), pl->bits(), ps.s, ps.cb, T - ps.pair, CB, pl->amp(), pl->cap,
                          &ps.wide);
         if (r)
@@ -1558,7 +1567,10 @@ int aaqaoa_set_workspace(aaqaoa_plan *pl, void *device_ptr, size_t bytes, int ba
     if (L.fns + sizeof head != L.out)
         return fail(AAQAOA_ERR_CUDA, "workspace layout");
     head.fns = GraphFns{pl->cost, {pl->obs[0], pl->obs[1]}};
-    CK(cudaMemcpyAsync(pl->ws + L.fns, &head, sizeof head, cudaMemcpyHostToDevice, pl->stream));
+    if (!pl->ising && pl->n <= CIRCUIT_MAX_QUBITS)  // (only the whole-circuit kernel reads them there)
+        CK(cudaMemcpyAsync(pl->ws + L.fns, &head, sizeof head, cudaMemcpyHostToDevice, pl->stream));
+    else
+        CK(cudaMemsetAsync(pl->ws + L.ctrl, 0, CTRL_BYTES, pl->stream));
     if (pl->ising)
         CK(cudaMemcpyAsync(pl->ws + L.ising, pl->ifn.data(), pl->ifn.size() * sizeof(IsingFn), cudaMemcpyHostToDevice,
                            pl->stream));

@@ -169,6 +169,7 @@ struct CircuitPlan {
     size_t smem;
 };
 constexpr int CIRCUIT_MIN_QUBITS = 5;   // 16 stored amplitudes
+constexpr int CIRCUIT_MAX_QUBITS = 20;
 constexpr int CIRCUIT_MAX_POINTS = 64;  // points of one launch when c > 0 (arrival counters)
 bool circuit_plan(bool c128, bool grad, int n, int p, int tab_len, int B, CircuitPlan *q);
 int launch_circuit(bool c128, bool grad, const CircuitArgs &a, const CircuitPlan &q, cudaStream_t st);
