@@ -2466,8 +2466,8 @@ extern "C" int aaqaoa_expect_static(aaqaoa_plan *pl, const double *gamma, const 
 
 // ============================================== uneven multi-graph batches
 // Graphs of a handful of vertices run together in one k_small_multi launch;
-// larger graphs each own a tiled sub-plan. One evaluation of the batch is
-// captured into a CUDA graph whose large-graph work is spread over `branches`
+// the others run in groups of equal n, each a plan of its own. One evaluation of
+// the batch is captured into a CUDA graph whose groups are spread over `branches`
 // parallel streams; the branch count is chosen by timing (autotune) on the
 // first call for each observable and cached for the process.
 struct aaqaoa_multi {

@@ -639,7 +639,7 @@ __global__ void __launch_bounds__(256) k_small(const __grid_constant__ SmallArgs
 }
 
 // ------------------------------------- uneven batch of small graphs
-// One CTA per graph (n <= 13 for complex64, <= 12 for complex128), the whole
+// One CTA per graph (of fewer than 5 vertices; larger ones run in groups), the whole
 // p-layer circuit and the fused energy in shared memory. Each CTA reads its
 // graph's masks from a device descriptor and builds its own phase factors
 // exp(-i ((gamma_l c) mod 2 pi)) in FP64, so graphs of different n and |E|
