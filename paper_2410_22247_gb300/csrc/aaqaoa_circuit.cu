@@ -35,7 +35,7 @@ namespace aaq {
 namespace {
 
 constexpr int CIRC_MAXP = 64;
-constexpr int CIRC_MAXN = 32;  // row length of the neighbour masks (vertices fit 32 bits)
+constexpr int CIRC_MAXN = CIRCUIT_MASKS;  // row length of the neighbour masks
 
 __device__ __forceinline__ uint32_t cswz(uint32_t i) { return i ^ ((i >> 4) & 15u); }
 
@@ -289,21 +289,31 @@ __global__ void __launch_bounds__(512) k_circuit(const __grid_constant__ Circuit
         return;
 
     for (unsigned b = team; b < (unsigned)A.B; b += teams) {
-        // cut functions (vertices of a circuit plan fit 32 bits): all classes, so
-        // that no load waits for their number
-        const bool fresh = b == team || A.per_point;
-        const GraphFns &fns = A.fns[A.per_point ? b : 0];
-        const CutFn &cost = fns.cost, &obs = fns.obs[A.obs];
-        const int Kc = cost.K, Ko = obs.K;
+        // cut functions. A graph per point reads all classes, so that no load waits
+        // for their number; one graph's are launch constants, only those in use (a
+        // constant read by lane-dependent index costs one access per lane).
+        const bool fresh = b == team || A.fns;
+        const GraphFns *const pt = A.fns ? A.fns + b : nullptr;
+        const int Kc = pt ? pt->cost.K : A.fn[0].K, Ko = pt ? pt->obs[A.obs].K : A.fn[1].K;
         if (fresh) {
-            for (int i = tid; i < MAXK * CIRC_MAXN; i += nt) {
-                const int k = i / CIRC_MAXN, u = i % CIRC_MAXN;
-                s_cost[i] = u < n ? (uint32_t)cost.nbr[k][u] : 0u;
-                s_obs[i] = u < n ? (uint32_t)obs.nbr[k][u] : 0u;
-            }
-            if (tid < MAXK) {
-                s_cw[tid] = cost.w[tid];
-                s_ow[tid] = obs.w[tid];
+            if (pt) {
+                const CutFn &cost = pt->cost, &obs = pt->obs[A.obs];
+                for (int i = tid; i < MAXK * CIRC_MAXN; i += nt) {
+                    const int k = i / CIRC_MAXN, u = i % CIRC_MAXN;
+                    s_cost[i] = u < n ? (uint32_t)cost.nbr[k][u] : 0u;
+                    s_obs[i] = u < n ? (uint32_t)obs.nbr[k][u] : 0u;
+                }
+                if (tid < MAXK) {
+                    s_cw[tid] = cost.w[tid];
+                    s_ow[tid] = obs.w[tid];
+                }
+            } else {
+                for (int i = tid; i < (Kc + Ko) * CIRC_MAXN; i += nt) {
+                    const int e = i >= Kc * CIRC_MAXN, j = e ? i - Kc * CIRC_MAXN : i;
+                    (e ? s_obs : s_cost)[j] = A.fn[e].nbr[j / CIRC_MAXN][j % CIRC_MAXN];
+                }
+                for (int k = tid; k < 2 * MAXK; k += nt)
+                    (k < MAXK ? s_cw : s_ow)[k % MAXK] = A.fn[k / MAXK].w[k % MAXK];
             }
             __syncthreads();
         }

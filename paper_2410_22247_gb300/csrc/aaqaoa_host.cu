@@ -97,7 +97,7 @@ struct Pass {
 };
 
 struct Layout {
-    size_t ctrl, fns, out, params, cs, tab, partials, zz, samp, ising, phi, lam, total;
+    size_t ctrl, out, params, cs, tab, partials, zz, samp, ising, phi, lam, total;
     size_t partial_count;
 };
 
@@ -243,9 +243,7 @@ Layout layout(const aaqaoa_plan *pl, int batch, bool grad)
     Layout L{};
     size_t off = 0;
     const size_t B = (size_t)batch;
-    L.fns = off;  // the plan's cut functions
-    off = align256(off + sizeof(GraphFns));
-    L.ctrl = off;  // right behind: error flag, counters | team counters of the whole-circuit kernel
+    L.ctrl = off;  // error flag, counters | team counters of the whole-circuit kernel
     off += CTRL_BYTES;
     L.out = off;  // right behind: one copy fetches the error flag and the rows
     off = align256(off + B * pl->out_stride() * sizeof(double));
@@ -903,8 +901,21 @@ bool use_circuit(const aaqaoa_plan *pl, int B, bool grad, bool state, CircuitPla
     return q->cluster || ((size_t)B * (grad ? 1 + 2 * pl->p : 1) << q->c) <= pl->L.partial_count;
 }
 
+// a cut function by value
+CircuitFn circuit_fn(const CutFn &f, int n)
+{
+    CircuitFn c{};
+    c.K = f.K;
+    for (int k = 0; k < f.K; k++) {
+        c.w[k] = f.w[k];
+        for (int u = 0; u < n; u++)
+            c.nbr[k][u] = (uint32_t)f.nbr[k][u];
+    }
+    return c;
+}
+
 // the plan's and the shape's part of the arguments
-CircuitArgs circuit_args(const aaqaoa_plan *pl, int B, const CircuitPlan &q)
+CircuitArgs circuit_args(const aaqaoa_plan *pl, int B, const CircuitPlan &q, int obs)
 {
     CircuitArgs a;
     memset(&a, 0, sizeof a);
@@ -918,6 +929,10 @@ CircuitArgs circuit_args(const aaqaoa_plan *pl, int B, const CircuitPlan &q)
     a.km = q.km;
     a.resident = q.resident;
     a.amp0 = std::pow(2.0, -0.5 * pl->n);
+    if (!pl->pt_dev) {
+        a.fn[0] = circuit_fn(pl->cost, pl->n);
+        a.fn[1] = circuit_fn(pl->obs[obs], pl->n);
+    }
     return a;
 }
 
@@ -928,7 +943,7 @@ int enqueue_circuit(aaqaoa_plan *pl, int B, const double *d_gamma, const double 
                     const double *h_beta = nullptr)
 {
     (void)cudaGetLastError();
-    CircuitArgs a = circuit_args(pl, B, q);
+    CircuitArgs a = circuit_args(pl, B, q, obs);
     a.gamma = d_gamma;
     a.beta = d_beta;
     if (h_gamma) {
@@ -943,8 +958,7 @@ int enqueue_circuit(aaqaoa_plan *pl, int B, const double *d_gamma, const double 
     a.partials = pl->d_partials();
     a.bar = pl->d_team_bar();
     a.err = pl->d_err();
-    a.fns = pl->pt_dev ? pl->pt_dev : reinterpret_cast<const GraphFns *>(pl->ws + pl->L.fns);
-    a.per_point = pl->pt_dev ? 1 : 0;
+    a.fns = pl->pt_dev;
     a.obs = obs;
     ProfScope ps_(pl, PK_SMALL, state ? (double)B * pl->state_bytes() : 0.0);
     CKL(launch_circuit(pl->c128, grad, a, q, pl->stream), "whole-circuit kernel");
@@ -1559,18 +1573,7 @@ int aaqaoa_set_workspace(aaqaoa_plan *pl, void *device_ptr, size_t bytes, int ba
     int r = build_maps(pl);
     if (r)
         return r;
-    struct {
-        GraphFns fns;
-        unsigned char pad[256 - sizeof(GraphFns) % 256], ctrl[CTRL_BYTES];
-    } head{};  // the cut functions and zeroed control words, one copy
-    static_assert(sizeof(GraphFns) % 256 && sizeof head.fns + sizeof head.pad + CTRL_BYTES == sizeof head);
-    if (L.fns + sizeof head != L.out)
-        return fail(AAQAOA_ERR_CUDA, "workspace layout");
-    head.fns = GraphFns{pl->cost, {pl->obs[0], pl->obs[1]}};
-    if (!pl->ising && pl->n <= CIRCUIT_MAX_QUBITS)  // (only the whole-circuit kernel reads them there)
-        CK(cudaMemcpyAsync(pl->ws + L.fns, &head, sizeof head, cudaMemcpyHostToDevice, pl->stream));
-    else
-        CK(cudaMemsetAsync(pl->ws + L.ctrl, 0, CTRL_BYTES, pl->stream));
+    CK(cudaMemsetAsync(pl->ws + L.ctrl, 0, CTRL_BYTES, pl->stream));
     if (pl->ising)
         CK(cudaMemcpyAsync(pl->ws + L.ising, pl->ifn.data(), pl->ifn.size() * sizeof(IsingFn), cudaMemcpyHostToDevice,
                            pl->stream));
@@ -2391,17 +2394,12 @@ extern "C" int aaqaoa_expect_static(aaqaoa_plan *pl, const double *gamma, const 
     CK(cudaMemcpyAsync(d_par + p, beta, (size_t)p * sizeof(double), cudaMemcpyHostToDevice, st));
     CircuitPlan q;
     if (pl->small() && use_circuit(pl, 1, false, false, &q)) {
-        GraphFns *d_fns = reinterpret_cast<GraphFns *>(d_phi);  // no state is stored
-        const GraphFns fns{pl->cost, {pl->obs[0], pl->obs[1]}};
-        CK(cudaMemcpyAsync(d_fns, &fns, sizeof fns, cudaMemcpyHostToDevice, st));
-        CircuitArgs a = circuit_args(pl, 1, q);  // a small plan's CTAs need no exchange buffers
+        CircuitArgs a = circuit_args(pl, 1, q, observable);  // a small plan's CTAs need no exchange buffers
         a.gamma = d_par;
         a.beta = d_par + p;
         a.out = d_out;
         a.out_stride = pl->out_stride();
         a.err = d_err;
-        a.fns = d_fns;
-        a.obs = observable;
         CKL(launch_circuit(pl->c128, false, a, q, st), "whole-circuit kernel");
         CK(cudaMemcpyAsync(energy, d_out, sizeof(double), cudaMemcpyDeviceToHost, st));
         CK(cudaStreamSynchronize(st));

@@ -143,6 +143,15 @@ struct SmallArgs {
     const double *gam;     // [B][p]
 };
 
+// A cut function as the whole-circuit kernel takes it: by value, so that nothing of
+// a plan has to stay in its workspace from one call to the next (vertices fit 32 bits).
+constexpr int CIRCUIT_MASKS = 32;  // neighbour masks per class
+struct CircuitFn {
+    int K;
+    int w[MAXK];
+    uint32_t nbr[MAXK][CIRCUIT_MASKS];
+};
+
 // Whole MaxCut circuit in one launch (aaqaoa_circuit.cu).
 struct CircuitArgs {
     int n, p, tab_len, B;
@@ -158,10 +167,11 @@ struct CircuitArgs {
     double *partials;    // c > 0: [B][rows][2^c]
     unsigned *bar;       // c > 0: one arrival counter per point, zero between launches
     int *err;
-    const GraphFns *fns; // the graph's cut functions (device memory)
-    int per_point;       // point b is its own graph, fns[b]
-    int obs;
+    CircuitFn fn[2];     // the cost and the observable, or
+    const GraphFns *fns; // per point (device memory): point b is its own graph, fns[b]
+    int obs;             // which observable of fns[b]
 };
+static_assert(sizeof(CircuitArgs) <= 4096, "kernel arguments of the classic size");
 // the kernel's shape for a call, from circuit_plan (false: the call does not fit it)
 struct CircuitPlan {
     int c, Tl, a, km, nt, teams, resident;

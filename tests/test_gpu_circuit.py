@@ -117,3 +117,27 @@ def test_ising_turnaround_over_odd_and_even_groups(plan):
         Er, dgr, dbr = O.ising_energy_grad(n, O.ising(e, w, h), np.array([0.5, 0.8]), np.array(beta))
         assert abs(E - Er) <= 1e-5 * scale
         assert np.max(np.abs(np.concatenate([dg - dgr, db - dbr]))) <= 1e-5 * scale
+
+
+@pytest.mark.parametrize("n,prec", [(5, "c64"), (10, "c128"), (13, "c64"), (16, "c64"), (20, "c64"), (20, "c128")])
+def test_plans_take_turns_on_one_workspace(n, prec):
+    """Two plans used one after the other on one buffer: a call depends on nothing
+    that another plan's set-up or call left there, to the last bit."""
+    import ctypes
+
+    from paper_2410_22247_gb300 import _native as N
+    a = [W.random_angles(2, 60 + k) for k in range(3)]
+    gs, bs = np.array([x[0] for x in a]), np.array([x[1] for x in a])
+
+    def results(pl):
+        one, many = pl.grad(gs[0], bs[0], "red"), pl.grad_batch(gs, bs, "red")
+        return np.concatenate([np.ravel(x) for x in one + many])
+
+    plans = [_plan(*graph, 2, prec, batch=3) for graph in (W.cycle_graph(n), W.star_graph(n))]
+    alone = [results(pl) for pl in plans]
+    assert not np.array_equal(alone[0], alone[1])
+    buf = plans[0].workspace
+    N.check(N.aaqaoa_set_workspace(plans[1].handle, ctypes.c_void_p(buf.data_ptr()), buf.numel(), 3, 1),
+            "set_workspace")
+    for k in (0, 1, 0, 1):
+        assert np.array_equal(results(plans[k]), alone[k])

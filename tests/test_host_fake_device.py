@@ -1,0 +1,83 @@
+"""The host side of the library (plans, copies, error reports) on a CUDA runtime
+that runs on the host (fake_device.cpp): aaqaoa_host.cu compiled as C++ and
+linked with it. The fake runs queued work only when the host synchronises, so
+what a queued operation still needs then has to be there."""
+import ctypes
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+from paper_2410_22247_gb300 import _native as N
+from paper_2410_22247_gb300 import build as B
+from paper_2410_22247_gb300 import workloads as W
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    out = str(tmp_path_factory.mktemp("fake") / "libfake.so")
+    cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+    subprocess.check_call(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-Wl,-Bsymbolic", "-I",
+                           os.path.join(cuda, "include"), "-I", B.INCLUDE, "-I", B.CSRC, "-o", out,
+                           os.path.join(HERE, "fake_device.cpp"), "-x", "c++",
+                           os.path.join(B.CSRC, "aaqaoa_host.cu")])
+    lib = ctypes.CDLL(out)
+    for name, res, args in N._PROTOS:
+        if hasattr(lib, name):
+            getattr(lib, name).restype = res
+            getattr(lib, name).argtypes = args
+    return lib
+
+
+def _p(a):
+    return a.ctypes.data_as(ctypes.POINTER(ctypes.c_int32))
+
+
+class FakePlan:
+    """A plan of the fake library on a buffer of host memory (its own, or `buffer`)."""
+
+    def __init__(self, lib, graph, p, batch=1, grad=True, buffer=None):
+        n, e = graph
+        self.lib, self.p, self.m = lib, p, len(e)
+        e = np.ascontiguousarray(e, dtype=np.int32).reshape(-1)
+        self.h = ctypes.c_void_p()
+        assert lib.aaqaoa_prepare(n, self.m, _p(e), 0, None, None, None, p, 0, None, ctypes.byref(self.h)) == 0
+        size = ctypes.c_size_t()
+        assert lib.aaqaoa_workspace_bytes(self.h, batch, int(grad), ctypes.byref(size)) == 0
+        self.buffer = np.zeros(size.value + 256, dtype=np.uint8) if buffer is None else buffer
+        at = (self.buffer.ctypes.data + 255) & ~255
+        assert self.buffer.nbytes >= size.value + 256
+        assert lib.aaqaoa_set_workspace(self.h, ctypes.c_void_p(at), size.value, batch, int(grad)) == 0
+
+    def value(self, g, b):
+        return 1000.0 * self.m + np.sum(g) + 2.0 * np.sum(b)
+
+    def expect(self, g, b):
+        out = np.zeros(1)
+        rc = self.lib.aaqaoa_expect(self.h, g.ctypes.data, b.ctypes.data, 0, 0, out.ctypes.data)
+        return rc, out[0]
+
+    def expect_batch(self, g, b):
+        out = np.zeros(len(g))
+        rc = self.lib.aaqaoa_expect_batch(self.h, len(g), g.ctypes.data, b.ctypes.data, 0, out.ctypes.data)
+        return rc, out
+
+    def close(self):
+        self.lib.aaqaoa_destroy(self.h)
+
+
+@pytest.mark.parametrize("n", [10, 14, 18])
+def test_plans_may_take_turns_on_one_workspace(lib, n):
+    """A MaxCut plan keeps nothing in its workspace from one call to the next:
+    plans used one after the other may have the same one."""
+    a = FakePlan(lib, W.complete_graph(n), 2)
+    b = FakePlan(lib, W.cycle_graph(n), 2, buffer=a.buffer)
+    x, y = np.array([0.3, 0.2]), np.array([0.1, 0.4])
+    for pl in (a, b, a):
+        rc, E = pl.expect(x, y)
+        assert rc == 0 and abs(E - pl.value(x, y)) < 1e-9
+    a.close()
+    b.close()
