@@ -23,7 +23,9 @@
 #include <cstring>
 #include <algorithm>
 #include <map>
+#include <memory>
 #include <mutex>
+#include <new>
 #include <string>
 #include <vector>
 
@@ -163,6 +165,7 @@ struct aaqaoa_plan {
     double state_bytes() const { return (double)((size_t)1 << n) * (double)amp(); }
     double sym() const { return half() ? 2.0 : 1.0; }  // what a sum over the stored amplitudes counts
     int tiles() const { return small() ? 1 : 1 << (bits() - T()); }
+    std::unique_ptr<double[]> angles;  // gamma and beta of the host call in flight (upload_params)
     double *slot = nullptr;  // pinned result row of one-point host calls (HostSlots)
     bool forced = false;  // the caller set the pass plan (aaqaoa_set_pass_plan)
     bool fuse = true;  // fuse layer boundaries into one pass where the plan allows
@@ -1172,11 +1175,17 @@ int upload_params(aaqaoa_plan *pl, int B, const double *gamma, const double *bet
     if (!gamma || !beta)
         return fail(AAQAOA_ERR_INVALID_ARG, "gamma/beta is NULL");
     const size_t count = (size_t)B * pl->p, bytes = count * sizeof(double);
-    double both[1024];
-    if (2 * count <= sizeof both / sizeof both[0]) {  // one copy (pageable memory: staged before the call returns)
-        memcpy(both, gamma, bytes);
-        memcpy(both + count, beta, bytes);
-        CK(cudaMemcpyAsync(pl->d_params(), both, 2 * bytes, cudaMemcpyHostToDevice, pl->stream));
+    constexpr size_t STAGED = 1024;  // doubles
+    if (2 * count <= STAGED) {
+        // one copy, from memory that lives as long as the plan: the device may read
+        // the source as late as the call's synchronisation
+        if (!pl->angles)
+            pl->angles.reset(new (std::nothrow) double[STAGED]);
+        if (!pl->angles)
+            return fail(AAQAOA_ERR_INVALID_ARG, "out of host memory");
+        memcpy(pl->angles.get(), gamma, bytes);
+        memcpy(pl->angles.get() + count, beta, bytes);
+        CK(cudaMemcpyAsync(pl->d_params(), pl->angles.get(), 2 * bytes, cudaMemcpyHostToDevice, pl->stream));
         return AAQAOA_OK;
     }
     CK(cudaMemcpyAsync(pl->d_params(), gamma, bytes, cudaMemcpyHostToDevice, pl->stream));

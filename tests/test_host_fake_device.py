@@ -81,3 +81,18 @@ def test_plans_may_take_turns_on_one_workspace(lib, n):
         assert rc == 0 and abs(E - pl.value(x, y)) < 1e-9
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("n,batch", [(10, 4), (14, 4), (18, 4), (22, 1), (22, 3), (22, 300)])
+def test_copies_read_living_memory(lib, n, batch):
+    """The angles of a call, and what a plan puts into its workspace, may be read
+    by the device as late as the call's own synchronisation."""
+    before = lib.fake_changed_sources()
+    pl = FakePlan(lib, W.cycle_graph(n), 2, batch=min(batch, 4), grad=False)
+    rng = np.random.default_rng(n)
+    g, b = rng.uniform(0, 3, (batch, 2)), rng.uniform(0, 1, (batch, 2))
+    rc, E = pl.expect_batch(g, b) if batch > 1 else pl.expect(g[0], b[0])
+    assert rc == 0
+    assert np.allclose(E, [pl.value(g[k], b[k]) for k in range(batch)], rtol=0, atol=1e-9)
+    assert lib.fake_changed_sources() == before
+    pl.close()
