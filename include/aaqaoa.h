@@ -241,7 +241,8 @@ int aaqaoa_grad_batch(aaqaoa_plan *plan, int B, const double *gamma, const doubl
  * Device-pointer forms: the same computations with every argument already in
  * device memory. They only enqueue work on the plan's stream and return; the
  * results are valid once that stream has reached them. A device-side timeout
- * is reported by the next call of aaqaoa_sync().
+ * is reported by the next call of aaqaoa_sync(); until then a whole-circuit
+ * launch that gave up, or that finds the timeout unreported, leaves NaN.
  *
  * aaqaoa_expect_device: d_gamma, d_beta: B*p doubles; d_energy: B doubles
  *   (B <= the workspace's batch capacity). Fused aggregation.
@@ -407,7 +408,7 @@ int aaqaoa_multi_info(const aaqaoa_multi *multi, int *G, int *small_graphs, int 
 void aaqaoa_destroy_multi(aaqaoa_multi *multi);
 
 /*
- * aaqaoa_inject_fault -- test hook for the failure path of the tiled passes.
+ * aaqaoa_inject_fault -- test hook for the failure paths of bounded waits.
  * kind AAQAOA_FAULT_DROP_TILE: the next tiled pass that loads the statevector
  * leaves the first tile of one CTA unloaded, so that CTA's bounded wait
  * (about one second) runs out; the call returns AAQAOA_ERR_TIMEOUT, its
@@ -415,8 +416,13 @@ void aaqaoa_destroy_multi(aaqaoa_multi *multi);
  * faults: the wait is the same bounded wait every pass uses. kind 0 clears a
  * pending fault. Plans with n <= the tile size have no tiled pass
  * (AAQAOA_ERR_UNSUPPORTED).
+ * kind AAQAOA_FAULT_DROP_ARRIVAL: in the next whole-circuit launch whose CTAs
+ * exchange through global memory and wait for one another, one CTA never
+ * arrives, so the others' bounded waits run out in the same way. Plans whose
+ * one-point energies take no such launch: AAQAOA_ERR_UNSUPPORTED.
  */
 #define AAQAOA_FAULT_DROP_TILE 1
+#define AAQAOA_FAULT_DROP_ARRIVAL 2
 int aaqaoa_inject_fault(aaqaoa_plan *plan, int kind);
 
 /*

@@ -285,8 +285,17 @@ __global__ void __launch_bounds__(512) k_circuit(const __grid_constant__ Circuit
         circ_cluster_sync();  // every CTA of the cluster runs before its memory is written
     else
         __syncthreads();
-    if (!CL && s_stop)
+    // A team that gives up leaves NaN in its point's row, not what an earlier call put
+    // there (each CTA that gives up writes it; no other result follows, since the
+    // last CTA to finish writes that and needs all of them).
+    auto give_up = [&](unsigned b) {
+        for (int r = tid; r < rows; r += nt)
+            A.out[(size_t)b * A.out_stride + r] = __longlong_as_double(0x7ff8000000000000ll);
+    };
+    if (!CL && s_stop) {
+        give_up(team);
         return;
+    }
 
     for (unsigned b = team; b < (unsigned)A.B; b += teams) {
         // cut functions. A graph per point reads all classes, so that no load waits
@@ -414,7 +423,8 @@ __global__ void __launch_bounds__(512) k_circuit(const __grid_constant__ Circuit
             __syncthreads();
             if (tid == 0) {
                 __threadfence();
-                atomicAdd(A.bar + b, 1u);
+                if (!(A.drop_arrival && X.rank == 0))
+                    atomicAdd(A.bar + b, 1u);
                 const long long t0 = clock64();
                 while (*reinterpret_cast<volatile unsigned *>(A.bar + b) < arrivals)
                     if (clock64() - t0 > WAIT_BUDGET_CYCLES) {
@@ -425,8 +435,10 @@ __global__ void __launch_bounds__(512) k_circuit(const __grid_constant__ Circuit
                 __threadfence();
             }
             __syncthreads();
-            if (s_stop)
+            if (s_stop) {
+                give_up(b);
                 return false;
+            }
 #pragma unroll 4
             for (uint32_t i = tid; i < NL; i += nt) {
                 const uint32_t y = circ_index(X, from ^ 1, i), x = cswz(i);

@@ -899,7 +899,7 @@ bool use_circuit(const aaqaoa_plan *pl, int B, bool grad, bool state, CircuitPla
         return false;
     if (pl->small())
         return true;
-    if (pl->forced || !pl->fuse || pl->inject || state)
+    if (pl->forced || !pl->fuse || pl->inject == AAQAOA_FAULT_DROP_TILE || state)
         return false;
     return q->cluster || ((size_t)B * (grad ? 1 + 2 * pl->p : 1) << q->c) <= pl->L.partial_count;
 }
@@ -963,6 +963,10 @@ int enqueue_circuit(aaqaoa_plan *pl, int B, const double *d_gamma, const double 
     a.err = pl->d_err();
     a.fns = pl->pt_dev;
     a.obs = obs;
+    if (pl->inject == AAQAOA_FAULT_DROP_ARRIVAL && q.c && !q.cluster) {
+        a.drop_arrival = 1;
+        pl->inject = 0;
+    }
     ProfScope ps_(pl, PK_SMALL, state ? (double)B * pl->state_bytes() : 0.0);
     CKL(launch_circuit(pl->c128, grad, a, q, pl->stream), "whole-circuit kernel");
     pl->launches++;
@@ -1051,10 +1055,13 @@ int circuit_host(aaqaoa_plan *pl, const double *gamma, const double *beta, int o
         return r;
     CK(cudaStreamSynchronize(pl->stream));
     memcpy(&first, pl->slot, sizeof first);
-    if (first == unset) {  // the launch gave up: its error flag says why
+    double head;
+    memcpy(&head, &first, sizeof head);
+    if (std::isnan(head)) {  // a launch that gave up: its error flag says why (or the angles were no numbers)
         if ((r = fetch_out(pl, 1, rows)))
             return r;
-        return fail(AAQAOA_ERR_CUDA, "the whole-circuit kernel left no result");
+        if (first == unset)
+            return fail(AAQAOA_ERR_CUDA, "the whole-circuit kernel left no result");
     }
     rows.assign(pl->slot, pl->slot + (grad ? pl->out_stride() : 1));
     return AAQAOA_OK;
@@ -2202,8 +2209,11 @@ int aaqaoa_inject_fault(aaqaoa_plan *pl, int kind)
 {
     if (!pl)
         return fail(AAQAOA_ERR_INVALID_ARG, "plan is NULL");
-    if (kind != 0 && kind != AAQAOA_FAULT_DROP_TILE)
+    if (kind != 0 && kind != AAQAOA_FAULT_DROP_TILE && kind != AAQAOA_FAULT_DROP_ARRIVAL)
         return fail(AAQAOA_ERR_INVALID_ARG, "fault kind %d unknown", kind);
+    CircuitPlan q;
+    if (kind == AAQAOA_FAULT_DROP_ARRIVAL && (pl->small() || !use_circuit(pl, 1, false, false, &q) || q.cluster || !q.c))
+        return fail(AAQAOA_ERR_UNSUPPORTED, "n=%d: no launch whose CTAs wait for one another", pl->n);
     if (kind == AAQAOA_FAULT_DROP_TILE && pl->small())
         return fail(AAQAOA_ERR_UNSUPPORTED, "n=%d runs in one CTA: no tiled pass to drop a tile from", pl->n);
     pl->inject = kind;

@@ -166,7 +166,8 @@ struct CircuitArgs {
     void *phi, *lam;     // c > 0: exchange buffers, 2^n amplitudes per point (two states' halves)
     double *partials;    // c > 0: [B][rows][2^c]
     unsigned *bar;       // c > 0: one arrival counter per point, zero between launches
-    int *err;
+    int *err;            // a team whose wait runs out sets it and leaves NaN in its row of `out`
+    int drop_arrival;    // test hook: a team's first CTA never arrives (bounded waits expire)
     CircuitFn fn[2];     // the cost and the observable, or
     const GraphFns *fns; // per point (device memory): point b is its own graph, fns[b]
     int obs;             // which observable of fns[b]

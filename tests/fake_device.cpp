@@ -166,13 +166,16 @@ int launch_circuit(bool, bool grad, const CircuitArgs &a, const CircuitPlan &q, 
     g_circuits++;
     g_queue.push_back([=] {
         const bool team = q.c && !q.cluster;
-        if (team && g_expire)
+        if (team && (g_expire || a.drop_arrival))
             *a.err = 1;
         if (team)
             g_expire = 0;
-        if (team && *a.err)
-            return;
         for (int b = 0; b < a.B; b++) {
+            if (team && *a.err) {
+                for (int r = 0; r < (grad ? 1 + 2 * a.p : 1); r++)
+                    a.out[(size_t)b * a.out_stride + r] = NAN;
+                continue;
+            }
             const double *g = a.gamma ? a.gamma + (size_t)b * a.p : a.ang;
             const double *be = a.gamma ? a.beta + (size_t)b * a.p : a.ang + a.p;
             double *row = a.out + (size_t)b * a.out_stride;

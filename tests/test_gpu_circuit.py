@@ -141,3 +141,44 @@ def test_plans_take_turns_on_one_workspace(n, prec):
             "set_workspace")
     for k in (0, 1, 0, 1):
         assert np.array_equal(results(plans[k]), alone[k])
+
+
+@pytest.mark.parametrize("n,prec", [(18, "c64"), (20, "c64"), (19, "c128")])
+def test_expired_wait_of_a_team_is_reported_and_the_plan_recovers(n, prec):
+    """One CTA of a team never arrives (a bounded wait of about a second): host calls
+    raise, device calls leave NaN instead of the previous results until the error
+    has been fetched, and the next call is right again."""
+    import torch
+
+    from paper_2410_22247_gb300 import _native as N
+    n, e = W.prufer_tree(n, 7)
+    g, b = W.random_angles(2, 9)
+    pl = _plan(n, e, 2, prec)
+    ref = O.energy_grad(n, e, g, b)
+    _check(pl.grad(g, b, "red"), ref, prec)
+    assert pl.launch_count() == 1
+    N.check(N.aaqaoa_inject_fault(pl.handle, N.AAQAOA_FAULT_DROP_ARRIVAL), "inject")
+    with pytest.raises(N.AAQAOAError, match="TIMEOUT"):
+        pl.grad(g, b, "red")
+    _check(pl.grad(g, b, "red"), ref, prec)
+    dg = torch.tensor(g, dtype=torch.float64, device="cuda")
+    db = torch.tensor(b, dtype=torch.float64, device="cuda")
+    out = torch.empty(5, dtype=torch.float64, device="cuda")
+    pl.grad_device(dg, db, out, "red")
+    N.check(N.aaqaoa_inject_fault(pl.handle, N.AAQAOA_FAULT_DROP_ARRIVAL), "inject")
+    for _ in range(2):
+        pl.grad_device(dg, db, out, "red")
+        assert torch.isnan(out).all()
+    with pytest.raises(N.AAQAOAError, match="TIMEOUT"):
+        pl.sync()
+    pl.grad_device(dg, db, out, "red")
+    pl.sync()
+    row = out.cpu().numpy()
+    _check((row[0], row[1:3], row[3:]), ref, prec)
+
+
+@pytest.mark.parametrize("n", [5, 10, 16])
+def test_no_team_to_drop_an_arrival_from(n):
+    from paper_2410_22247_gb300 import _native as N
+    pl = _plan(*W.cycle_graph(n), 1, "c64")
+    assert N.aaqaoa_inject_fault(pl.handle, N.AAQAOA_FAULT_DROP_ARRIVAL) == -6

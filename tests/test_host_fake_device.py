@@ -65,6 +65,15 @@ class FakePlan:
         rc = self.lib.aaqaoa_expect_batch(self.h, len(g), g.ctypes.data, b.ctypes.data, 0, out.ctypes.data)
         return rc, out
 
+    def grad(self, g, b):
+        out, dg, db = np.zeros(1), np.zeros(self.p), np.zeros(self.p)
+        rc = self.lib.aaqaoa_grad(self.h, g.ctypes.data, b.ctypes.data, 0, out.ctypes.data, dg.ctypes.data,
+                                  db.ctypes.data)
+        return rc, out[0]
+
+    def expect_device(self, g, b, out):
+        return self.lib.aaqaoa_expect_device(self.h, 1, g.ctypes.data, b.ctypes.data, 0, out.ctypes.data)
+
     def close(self):
         self.lib.aaqaoa_destroy(self.h)
 
@@ -96,3 +105,44 @@ def test_copies_read_living_memory(lib, n, batch):
     assert np.allclose(E, [pl.value(g[k], b[k]) for k in range(batch)], rtol=0, atol=1e-9)
     assert lib.fake_changed_sources() == before
     pl.close()
+
+
+TIMEOUT = -5
+
+
+def test_a_team_that_gives_up_is_reported(lib):
+    """The expired wait of a team (n = 18): host calls return TIMEOUT and the plan
+    recovers; device calls leave NaN until the error has been fetched."""
+    pl = FakePlan(lib, W.cycle_graph(18), 2)
+    x, y = np.array([0.3, 0.2]), np.array([0.1, 0.4])
+    for call in (pl.expect, pl.grad):
+        assert lib.aaqaoa_inject_fault(pl.h, N.AAQAOA_FAULT_DROP_ARRIVAL) == 0
+        assert call(x, y)[0] == TIMEOUT
+        rc, E = call(x, y)
+        assert rc == 0 and abs(E - pl.value(x, y)) < 1e-9
+    out = np.zeros(1)
+    assert lib.aaqaoa_inject_fault(pl.h, N.AAQAOA_FAULT_DROP_ARRIVAL) == 0
+    for _ in range(2):
+        out[0] = 7.0
+        assert pl.expect_device(x, y, out) == 0
+        lib.cudaStreamSynchronize(None)
+        assert np.isnan(out[0])
+    assert lib.aaqaoa_sync(pl.h) == TIMEOUT
+    assert pl.expect_device(x, y, out) == 0 and lib.aaqaoa_sync(pl.h) == 0
+    assert abs(out[0] - pl.value(x, y)) < 1e-9
+    pl.close()
+
+
+def test_angles_that_are_no_numbers_give_no_number(lib):
+    for n in (10, 18):
+        pl = FakePlan(lib, W.cycle_graph(n), 1)
+        rc, E = pl.expect(np.array([np.nan]), np.array([0.1]))
+        assert rc == 0 and np.isnan(E)
+        pl.close()
+
+
+def test_drop_arrival_needs_a_team(lib):
+    for n in (4, 10, 16, 22):
+        pl = FakePlan(lib, W.cycle_graph(n), 1)
+        assert lib.aaqaoa_inject_fault(pl.h, N.AAQAOA_FAULT_DROP_ARRIVAL) == -6
+        pl.close()
