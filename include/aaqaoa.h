@@ -241,7 +241,8 @@ int aaqaoa_grad_batch(aaqaoa_plan *plan, int B, const double *gamma, const doubl
  * Device-pointer forms: the same computations with every argument already in
  * device memory. They only enqueue work on the plan's stream and return; the
  * results are valid once that stream has reached them. A device-side timeout
- * is reported by the next call of aaqaoa_sync(); until then a whole-circuit
+ * is reported by the next call that waits for the plan (aaqaoa_sync() or an
+ * energy or gradient with host pointers); until then a whole-circuit
  * launch that gave up, or that finds the timeout unreported, leaves NaN.
  *
  * aaqaoa_expect_device: d_gamma, d_beta: B*p doubles; d_energy: B doubles
@@ -420,9 +421,12 @@ void aaqaoa_destroy_multi(aaqaoa_multi *multi);
  * exchange through global memory and wait for one another, one CTA never
  * arrives, so the others' bounded waits run out in the same way. Plans whose
  * one-point energies take no such launch: AAQAOA_ERR_UNSUPPORTED.
+ * kind AAQAOA_FAULT_UNREPORTED: sets the plan's device error flag at once, as
+ * the expired wait of a device call that no call has reported yet.
  */
 #define AAQAOA_FAULT_DROP_TILE 1
 #define AAQAOA_FAULT_DROP_ARRIVAL 2
+#define AAQAOA_FAULT_UNREPORTED 3
 int aaqaoa_inject_fault(aaqaoa_plan *plan, int kind);
 
 /*

@@ -23,6 +23,7 @@ AAQAOA_AGG_SINGLEPASS = 2
 AAQAOA_AGG_PERORBIT = AAQAOA_AGG_SINGLEPASS
 AAQAOA_FAULT_DROP_TILE = 1
 AAQAOA_FAULT_DROP_ARRIVAL = 2
+AAQAOA_FAULT_UNREPORTED = 3
 AAQAOA_OK = 0
 ERRORS = {
     -1: "AAQAOA_ERR_INVALID_ARG", -2: "AAQAOA_ERR_BAD_ORBITS", -3: "AAQAOA_ERR_WORKSPACE",

@@ -277,10 +277,15 @@ __global__ void __launch_bounds__(512) k_circuit(const __grid_constant__ Circuit
     X.off = 0;
     const unsigned team = blockIdx.x >> c, teams = gridDim.x >> c;
 
-    // (a team's wait gave up in an earlier launch whose error was not fetched yet:
-    // its counters are not at zero)
-    if (tid == 0)
-        s_stop = !CL && c && *reinterpret_cast<volatile int *>(A.err) ? 1 : 0;
+    // The error flag of earlier launches that was not fetched yet. A team stops (its
+    // counters are not at zero); a host call that reads no other word back gets it.
+    const bool stops = !CL && c;
+    int pending = 0;
+    if (tid == 0) {
+        if (stops || (A.err_out && X.rank == 0))
+            pending = *reinterpret_cast<volatile int *>(A.err);
+        s_stop = stops && pending ? 1 : 0;
+    }
     if (CL)
         circ_cluster_sync();  // every CTA of the cluster runs before its memory is written
     else
@@ -572,6 +577,8 @@ __global__ void __launch_bounds__(512) k_circuit(const __grid_constant__ Circuit
         }
 
         // -------------------------------------------------- the results
+        if (A.err_out && tid == 0 && X.rank == 0)
+            *A.err_out = pending;
         // sums over the stored half count twice; dE/dgamma and dE/dbeta are
         // 2 Im of theirs. A team's CTAs are added in rank order.
         double *part = CL ? nullptr : A.partials + (((size_t)b * rows) << c);

@@ -943,7 +943,7 @@ CircuitArgs circuit_args(const aaqaoa_plan *pl, int B, const CircuitPlan &q, int
 // point (h_angles: gamma, then beta) go by value.
 int enqueue_circuit(aaqaoa_plan *pl, int B, const double *d_gamma, const double *d_beta, int obs, bool grad, bool state,
                     const CircuitPlan &q, double *out = nullptr, int stride = 0, const double *h_gamma = nullptr,
-                    const double *h_beta = nullptr)
+                    const double *h_beta = nullptr, int *err_out = nullptr)
 {
     (void)cudaGetLastError();
     CircuitArgs a = circuit_args(pl, B, q, obs);
@@ -961,6 +961,7 @@ int enqueue_circuit(aaqaoa_plan *pl, int B, const double *d_gamma, const double 
     a.partials = pl->d_partials();
     a.bar = pl->d_team_bar();
     a.err = pl->d_err();
+    a.err_out = err_out;
     a.fns = pl->pt_dev;
     a.obs = obs;
     if (pl->inject == AAQAOA_FAULT_DROP_ARRIVAL && q.c && !q.cluster) {
@@ -978,7 +979,8 @@ int enqueue_circuit(aaqaoa_plan *pl, int B, const double *d_gamma, const double 
 // by the first such call); without a free row a call copies its results back.
 class HostSlots {
   public:
-    static constexpr int COUNT = 64, ROW = 256;  // doubles per row: 1 + 2 * 64 results and spare
+    static constexpr int COUNT = 64, ROW = 256;  // doubles per row: 1 + 2 * 64 results and spare,
+    static constexpr int FLAG = ROW - 1;         // the last one the error flag
     static double *take()
     {
         std::lock_guard<std::mutex> lock(mutex());
@@ -1047,17 +1049,22 @@ int circuit_host(aaqaoa_plan *pl, const double *gamma, const double *beta, int o
     const unsigned long long unset = 0x7ff8aa90a0000001ull;  // no result has these bits
     unsigned long long first = unset;
     memcpy(pl->slot, &unset, sizeof unset);
+    int *const flag = reinterpret_cast<int *>(pl->slot + HostSlots::FLAG);
+    *flag = 0;
     if (!pl->small())
         pl->state_valid = false;  // the exchange buffers are the stored state's
     int r = enqueue_circuit(pl, 1, nullptr, nullptr, obs, grad, false, q, static_cast<double *>(d_row),
-                            pl->out_stride(), gamma, beta);
+                            pl->out_stride(), gamma, beta,
+                            reinterpret_cast<int *>(static_cast<double *>(d_row) + HostSlots::FLAG));
     if (r)
         return r;
     CK(cudaStreamSynchronize(pl->stream));
     memcpy(&first, pl->slot, sizeof first);
     double head;
     memcpy(&head, &first, sizeof head);
-    if (std::isnan(head)) {  // a launch that gave up: its error flag says why (or the angles were no numbers)
+    // a launch that gave up (its error flag says why; or the angles were no numbers),
+    // or an earlier device call's error that no call has fetched
+    if (std::isnan(head) || *flag) {
         if ((r = fetch_out(pl, 1, rows)))
             return r;
         if (first == unset)
@@ -2209,8 +2216,14 @@ int aaqaoa_inject_fault(aaqaoa_plan *pl, int kind)
 {
     if (!pl)
         return fail(AAQAOA_ERR_INVALID_ARG, "plan is NULL");
-    if (kind != 0 && kind != AAQAOA_FAULT_DROP_TILE && kind != AAQAOA_FAULT_DROP_ARRIVAL)
+    if (kind < 0 || kind > AAQAOA_FAULT_UNREPORTED)
         return fail(AAQAOA_ERR_INVALID_ARG, "fault kind %d unknown", kind);
+    if (kind == AAQAOA_FAULT_UNREPORTED) {
+        if (!pl->ws)
+            return fail(AAQAOA_ERR_WORKSPACE, "no workspace set (aaqaoa_set_workspace)");
+        CK(cudaMemsetAsync(pl->d_err(), 1, 1, pl->stream));  // the flag's low byte
+        return AAQAOA_OK;
+    }
     CircuitPlan q;
     if (kind == AAQAOA_FAULT_DROP_ARRIVAL && (pl->small() || !use_circuit(pl, 1, false, false, &q) || q.cluster || !q.c))
         return fail(AAQAOA_ERR_UNSUPPORTED, "n=%d: no launch whose CTAs wait for one another", pl->n);

@@ -167,6 +167,7 @@ struct CircuitArgs {
     double *partials;    // c > 0: [B][rows][2^c]
     unsigned *bar;       // c > 0: one arrival counter per point, zero between launches
     int *err;            // a team whose wait runs out sets it and leaves NaN in its row of `out`
+    int *err_out;        // also store the error flag as this launch finds it (or null)
     int drop_arrival;    // test hook: a team's first CTA never arrives (bounded waits expire)
     CircuitFn fn[2];     // the cost and the observable, or
     const GraphFns *fns; // per point (device memory): point b is its own graph, fns[b]

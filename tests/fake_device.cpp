@@ -170,6 +170,8 @@ int launch_circuit(bool, bool grad, const CircuitArgs &a, const CircuitPlan &q, 
             *a.err = 1;
         if (team)
             g_expire = 0;
+        if (a.err_out)
+            *a.err_out = *a.err;
         for (int b = 0; b < a.B; b++) {
             if (team && *a.err) {
                 for (int r = 0; r < (grad ? 1 + 2 * a.p : 1); r++)

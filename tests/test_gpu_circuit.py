@@ -182,3 +182,19 @@ def test_no_team_to_drop_an_arrival_from(n):
     from paper_2410_22247_gb300 import _native as N
     pl = _plan(*W.cycle_graph(n), 1, "c64")
     assert N.aaqaoa_inject_fault(pl.handle, N.AAQAOA_FAULT_DROP_ARRIVAL) == -6
+
+
+@pytest.mark.parametrize("n,prec", [(4, "c64"), (8, "c64"), (10, "c128"), (16, "c64"), (20, "c64"), (22, "c64")])
+def test_unreported_timeout_reaches_the_next_host_call(n, prec):
+    """The error flag of an earlier device call, through every form of a one-point
+    host call: one CTA, a cluster, a team, the passes."""
+    from paper_2410_22247_gb300 import _native as N
+    n, e = W.cycle_graph(n)
+    g, b = W.random_angles(1, 3)
+    pl = _plan(n, e, 1, prec)
+    for call in (lambda: pl.expect(g, b, "red"), lambda: pl.grad(g, b, "red")[0]):
+        want = call()
+        N.check(N.aaqaoa_inject_fault(pl.handle, N.AAQAOA_FAULT_UNREPORTED), "inject")
+        with pytest.raises(N.AAQAOAError, match="TIMEOUT"):
+            call()
+        assert call() == want

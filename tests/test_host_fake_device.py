@@ -146,3 +146,47 @@ def test_drop_arrival_needs_a_team(lib):
         pl = FakePlan(lib, W.cycle_graph(n), 1)
         assert lib.aaqaoa_inject_fault(pl.h, N.AAQAOA_FAULT_DROP_ARRIVAL) == -6
         pl.close()
+
+
+@pytest.mark.parametrize("n", [4, 10, 14, 18, 22])
+def test_an_unreported_timeout_reaches_the_next_host_call(lib, n):
+    """A device call's expired wait is reported by whichever call waits next, a
+    one-point energy or gradient among them; the one after that is right."""
+    pl = FakePlan(lib, W.cycle_graph(n), 2)
+    x, y = np.array([0.3, 0.2]), np.array([0.1, 0.4])
+    for call in (pl.expect, pl.grad):
+        assert lib.aaqaoa_inject_fault(pl.h, N.AAQAOA_FAULT_UNREPORTED) == 0
+        assert call(x, y)[0] == TIMEOUT
+        rc, E = call(x, y)
+        assert rc == 0 and (n == 4 or abs(E - pl.value(x, y)) < 1e-9)
+    pl.close()
+
+
+def test_host_calls_without_a_pinned_row(lib):
+    """Plans beyond the 64 that hold a pinned row copy their results back."""
+    x, y = np.array([0.3]), np.array([0.1])
+    plans = [FakePlan(lib, W.cycle_graph(6 + k % 4), 1, grad=False) for k in range(70)]
+    for pl in plans:
+        rc, E = pl.expect(x, y)
+        assert rc == 0 and abs(E - pl.value(x, y)) < 1e-9
+    for pl in plans[64:]:
+        assert lib.aaqaoa_inject_fault(pl.h, N.AAQAOA_FAULT_UNREPORTED) == 0
+        assert pl.expect(x, y)[0] == TIMEOUT
+    for pl in plans:
+        pl.close()
+
+
+@pytest.mark.parametrize("n", [10, 14, 18])
+def test_device_results_over_their_angles(lib, n):
+    """A result row that overlaps the angles is written only when they have been read."""
+    for at in range(0, 6):
+        buf = np.zeros(12)
+        buf[2:4], buf[4:6] = [0.3, 0.2], [0.1, 0.4]
+        pl = FakePlan(lib, W.cycle_graph(n), 2)
+        g, b = buf[2:4], buf[4:6]
+        want = pl.value(g, b)
+        out = buf[at:at + 5]
+        assert lib.aaqaoa_grad_device(pl.h, g.ctypes.data, b.ctypes.data, 0, out.ctypes.data) == 0
+        assert lib.aaqaoa_sync(pl.h) == 0
+        assert abs(out[0] - want) < 1e-9 and np.allclose(out[1:], [0.3, 0.2, 0.1, 0.4])
+        pl.close()
