@@ -338,9 +338,9 @@ __global__ void __launch_bounds__(512) k_circuit(const __grid_constant__ Circuit
         // follows once those are known.
         double2 z0 = make_double2(1.0, 0.0);
         if (A.resident && warp < p && lane < tab_len)
-            z0 = phase_sincos<R>(gam[warp] * (double)lane);
+            z0 = phase_sincos(gam[warp] * (double)lane);
         for (int l = nt - 1 - tid; l < p; l += nt) {
-            const double2 z = phase_sincos<double>(bet[l]);
+            const double2 z = phase_sincos(bet[l]);
             const bool sh = fabs(z.y) > fabs(z.x);  // rotate by beta - pi/2 (see rot)
             double t, f;
             mix_ratio<R>(sh ? -z.x : z.y, sh ? z.y : z.x, t, f);
@@ -370,7 +370,7 @@ __global__ void __launch_bounds__(512) k_circuit(const __grid_constant__ Circuit
         if (A.resident) {
             for (int l = warp; l < p; l += nw)
                 for (int i = lane; i < tab_len; i += 32) {
-                    const double2 z = l == warp && i == lane ? z0 : phase_sincos<R>(gam[l] * (double)i);
+                    const double2 z = l == warp && i == lane ? z0 : phase_sincos(gam[l] * (double)i);
                     entry(l, i, z, tabs + (size_t)2 * l * tab_len);
                 }
             __syncthreads();
@@ -380,7 +380,7 @@ __global__ void __launch_bounds__(512) k_circuit(const __grid_constant__ Circuit
                 return tabs + (size_t)2 * l * tab_len;
             __syncthreads();
             for (int i = tid; i < tab_len; i += nt)
-                entry(l, i, phase_sincos<R>(gam[l] * (double)i), tabs);
+                entry(l, i, phase_sincos(gam[l] * (double)i), tabs);
             __syncthreads();
             return tabs;
         };

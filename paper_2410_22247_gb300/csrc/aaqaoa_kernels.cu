@@ -446,7 +446,7 @@ __global__ void __launch_bounds__(256) k_params(int B, int p, int tab_len, int n
     const long long i0 = (long long)blockIdx.x * 256, i = i0 + threadIdx.x, N = (long long)B * p * tab_len;
     const long long BP = (long long)B * p;
     auto rotation = [&](long long bl, double &c, double &s, double &t, double &f) -> bool {  // |sin| > |cos|
-        const double2 z = phase_sincos<double>(beta[bl]);
+        const double2 z = phase_sincos(beta[bl]);
         c = z.x;
         s = z.y;
         const bool sh = fabs(s) > fabs(c);
@@ -474,7 +474,7 @@ __global__ void __launch_bounds__(256) k_params(int B, int p, int tab_len, int n
     __syncthreads();
     if (i < N) {
         const long long bl = i / tab_len;
-        const double2 z = phase_sincos<R>(gamma[bl] * (double)(i - bl * tab_len));
+        const double2 z = phase_sincos(gamma[bl] * (double)(i - bl * tab_len));
         const double fs = bl % p ? s_fs[bl - bl0] : 1.0, fb = s_fb[bl - bl0];
         if (kinds & 1)
             tab[i] = mkc<C>((R)z.x, (R)(-z.y));

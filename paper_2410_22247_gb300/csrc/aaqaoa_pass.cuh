@@ -42,6 +42,7 @@
 #include <type_traits>
 
 #include "aaqaoa_internal.h"
+#include "aaqaoa_trig.h"
 
 namespace aaq {
 
@@ -165,47 +166,6 @@ __device__ __forceinline__ void dot_acc(C &acc, const C &u, const C &v)
         acc.x = fma(u.x, v.x, acc.x);
         acc.y = fma(u.y, v.y, acc.y);
     }
-}
-
-// cos x, sin x in FP64 for the phase tables, by reduction to |r| <= pi/4 (x -
-// k pi/2 with pi/2 in two parts, fused) and the Taylor series there: the
-// library's function costs 3 us at the head of a launch. float: a relative
-// error below 1e-10, rounded once to the table's precision; double: 1e-16.
-template <typename R>
-__device__ __noinline__ double2 phase_sincos(double x)  // (cos, sin)
-{
-    const double k = rint(x * 0.63661977236758134308);
-    if (!(fabs(k) < 1e9)) {
-        double sn, cn;
-        sincos(x, &sn, &cn);
-        return make_double2(cn, sn);
-    }
-    double r = fma(k, -1.5707963267948965580, x);
-    r = fma(k, -6.1232339957367660359e-17, r);
-    const double s = r * r;
-    double ps, pc;
-    if constexpr (std::is_same<R, float>::value) {
-        ps = fma(s, -1.0 / 39916800.0, 1.0 / 362880.0);
-        pc = fma(s, 1.0 / 479001600.0, -1.0 / 3628800.0);
-    } else {
-        ps = fma(s, -1.0 / 1307674368000.0, 1.0 / 6227020800.0);
-        pc = fma(s, 1.0 / 20922789888000.0, -1.0 / 87178291200.0);
-        ps = fma(ps, s, -1.0 / 39916800.0);
-        pc = fma(pc, s, 1.0 / 479001600.0);
-        ps = fma(ps, s, 1.0 / 362880.0);
-        pc = fma(pc, s, -1.0 / 3628800.0);
-    }
-    ps = fma(ps, s, -1.0 / 5040.0);
-    pc = fma(pc, s, 1.0 / 40320.0);
-    ps = fma(ps, s, 1.0 / 120.0);
-    pc = fma(pc, s, -1.0 / 720.0);
-    ps = fma(ps, s, -1.0 / 6.0);
-    pc = fma(pc, s, 1.0 / 24.0);
-    pc = fma(pc, s, -0.5);
-    const double sr = fma(r * s, ps, r), cr = fma(s, pc, 1.0);
-    const int q = (int)(long long)k & 3;
-    const double a = (q & 1) ? cr : sr, b = (q & 1) ? sr : cr;
-    return make_double2(((q + 1) & 2) ? -b : b, (q & 2) ? -a : a);
 }
 
 // The rotation of one mixer layer from (cos, sin) of its angle: u / v = t, the
