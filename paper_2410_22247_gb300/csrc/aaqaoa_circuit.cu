@@ -342,16 +342,11 @@ __global__ void __launch_bounds__(512) k_circuit(const __grid_constant__ Circuit
         for (int l = nt - 1 - tid; l < p; l += nt) {
             const double2 z = phase_sincos(bet[l]);
             const bool sh = fabs(z.y) > fabs(z.x);  // rotate by beta - pi/2 (see rot)
-            double t, f;
-            mix_ratio<R>(sh ? -z.x : z.y, sh ? z.y : z.x, t, f);
-            const double fi = sh ? -f : f;
-            double fn = 1.0, q = f;
-            for (int k = n; k; k >>= 1) {
-                if (k & 1)
-                    fn *= q;
-                q *= q;
-            }
-            lay[l] = CircLayer{f, fi, fn, (sh && (n & 1)) ? -fn : fn, t};
+            double t;
+            MixFactor m;
+            mix_ratio<R>(sh ? -z.x : z.y, sh ? z.y : z.x, t, m);
+            const double fn = mix_power<R>(m, n);
+            lay[l] = CircLayer{m.f, sh ? -m.f : m.f, fn, (sh && (n & 1)) ? -fn : fn, t};
         }
         // cut values of the tile's states in both layouts
         if (fresh)

@@ -445,7 +445,7 @@ __global__ void __launch_bounds__(256) k_params(int B, int p, int tab_len, int n
     __shared__ double s_fs[258], s_fb[258];
     const long long i0 = (long long)blockIdx.x * 256, i = i0 + threadIdx.x, N = (long long)B * p * tab_len;
     const long long BP = (long long)B * p;
-    auto rotation = [&](long long bl, double &c, double &s, double &t, double &f) -> bool {  // |sin| > |cos|
+    auto rotation = [&](long long bl, double &c, double &s, double &t, MixFactor &f) -> bool {  // |sin| > |cos|
         const double2 z = phase_sincos(beta[bl]);
         c = z.x;
         s = z.y;
@@ -458,14 +458,10 @@ __global__ void __launch_bounds__(256) k_params(int B, int p, int tab_len, int n
     for (long long bl = bl0 - 1 + threadIdx.x; bl <= bl1; bl += 256) {
         if (bl < 0 || bl0 >= BP)
             continue;
-        double c, s, t, f;
+        double c, s, t;
+        MixFactor f;
         const bool sh = rotation(bl, c, s, t, f);
-        double fn = 1.0, q = f;
-        for (int k = n; k; k >>= 1) {
-            if (k & 1)
-                fn *= q;
-            q *= q;
-        }
+        const double fn = mix_power<R>(f, n);
         if (bl < bl1)
             s_fs[bl - bl0 + 1] = fn;  // for the next layer's entries
         if (bl >= bl0)
@@ -488,16 +484,17 @@ __global__ void __launch_bounds__(256) k_params(int B, int p, int tab_len, int n
         out[k] = 0.0;
     for (long long bl = step - 1 - i; bl < BP; bl += step) {  // (the last blocks: the first ones have tables)
         MixRow &r = rows[bl];
-        double c, s, t, f;
+        double c, s, t;
+        MixFactor f;
         rotation(bl, c, s, t, f);
         r.c = c;
         r.s = s;
         r.t = t;
-        r.f = f;
-        double q = 1.0;
+        r.f = f.f;
+        MixPower q;
         for (int k = 0; k <= n; k++) {
-            r.pw[k] = q;
-            q *= f;
+            r.pw[k] = q.value();
+            q.times<R>(f);
         }
     }
 }

@@ -168,21 +168,6 @@ __device__ __forceinline__ void dot_acc(C &acc, const C &u, const C &v)
     }
 }
 
-// The rotation of one mixer layer from (cos, sin) of its angle: u / v = t, the
-// ratio the butterflies use (rounded to the amplitude type), and f, the factor one
-// butterfly with that t drops: 1 / sqrt(1 + t^2) with v's sign, to first order in
-// the rounding error t v - u. f and t belong together: with f = cos beta the norm
-// drifts by the rounding of t in every butterfly.
-template <typename R>
-__device__ __forceinline__ void mix_ratio(double u, double v, double &t, double &f)
-{
-    if constexpr (std::is_same<R, float>::value)
-        t = (double)((float)u / (float)v);
-    else
-        t = u / v;
-    f = v - v * (u * fma(t, v, -u));
-}
-
 // Im(conj(l) f)
 template <typename C>
 __device__ __forceinline__ auto im_conj_mul(C l, C f) -> decltype(l.x) { return l.x * f.y - l.y * f.x; }

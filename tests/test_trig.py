@@ -55,6 +55,36 @@ def test_host_form_of_no_number(probe):
     assert np.isnan(_host(probe, np.array([np.nan, np.inf, -np.inf]))).all()
 
 
+@pytest.mark.parametrize("real", ["float", "double"])
+def test_dropped_factor_and_its_powers(probe, real):
+    """f = 1 / sqrt(1 + t^2) for the rounded t, and f^k, k <= 34. Double: f^k right to
+    one rounding (2^-53 relative; f in two parts, products with their errors: the
+    rest is below 2^-90). Float: t is off by three roundings to float, 3 2^-24,
+    and f to second order in that, below 2^-45."""
+    mp = pytest.importorskip("mpmath")
+    n = 34
+    rng = np.random.default_rng(11)
+    angles = np.concatenate([rng.uniform(-np.pi, np.pi, 300), [0.0, np.pi / 4, -np.pi / 4, 1e-9, np.pi / 2, 3.0]])
+    worst = 0.0
+    with mp.workprec(250):
+        for a in angles:
+            u, v = float(np.sin(a)), float(np.cos(a))
+            if abs(u) > abs(v):
+                u, v = -v, u
+            t, f = ctypes.c_double(), np.zeros(2)
+            sq, ch = np.zeros(n + 1), np.zeros(n + 1)
+            P = lambda x: ctypes.c_void_p(x.ctypes.data)
+            probe.probe_mix(ctypes.c_double(u), ctypes.c_double(v), int(real == "float"), n, ctypes.byref(t), P(f),
+                            P(sq), P(ch))
+            exact = (1 if v > 0 else -1) / mp.sqrt(1 + mp.mpf(t.value) ** 2)
+            for k in range(n + 1):
+                for x in (sq[k], ch[k]):
+                    err = float(abs(mp.mpf(float(x)) / exact ** k - 1))
+                    worst = max(worst, err / (2.0 ** -53 * (1 + 1e-6) if real == "double"
+                                              else k * 2.0 ** -45 + 2.0 ** -53))
+    assert worst <= 1.0
+
+
 @pytest.mark.gpu
 def test_device_form_is_the_host_form(probe):
     torch = pytest.importorskip("torch")
