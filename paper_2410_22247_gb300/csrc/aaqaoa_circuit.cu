@@ -39,6 +39,27 @@ constexpr int CIRC_MAXN = CIRCUIT_MASKS;  // row length of the neighbour masks
 
 __device__ __forceinline__ uint32_t cswz(uint32_t i) { return i ^ ((i >> 4) & 15u); }
 
+// A thread's sum of terms in the amplitude type. complex64: a float and the
+// rounding errors of its additions (TwoSum), 48 bits, so that a term costs six
+// FP32 operations and no FP64 one: the FP64 unit takes 16 cycles per warp, and
+// three such additions per register stage were 1.2 us of a 33 us gradient at
+// n = 10. Sums over threads are FP64.
+template <typename R> struct CircSum {
+    double v = 0.0;
+    __device__ __forceinline__ void add(double x) { v += x; }
+    __device__ __forceinline__ double value() const { return v; }
+};
+template <> struct CircSum<float> {
+    float hi = 0.f, lo = 0.f;
+    __device__ __forceinline__ void add(float x)
+    {
+        const float t = __fadd_rn(hi, x), z = __fsub_rn(t, hi);
+        lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(t, z)), __fsub_rn(x, z)));
+        hi = t;
+    }
+    __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
+};
+
 struct CircLayer {  // one layer's mixer: rotation t, dropped factor f, f^n; of the inverse: -t, fi, fi^n
     double f, fi, fn, fin;
     double t;
@@ -79,18 +100,17 @@ __device__ __forceinline__ uint32_t circ_index(const CircCtx &X, int high, uint3
 // runs the same code (a launch meets it cold).
 template <typename R> struct CircMix {
     R run;
-    double acc;
+    CircSum<R> acc;
 };
 template <typename R, int NV, int K, bool MIR>
 __device__ __noinline__ CircMix<R> circ_stage(uint32_t off, int Tl, int q0, int pair, R sg0, R t, R f, R run,
-                                              double acc)
+                                              CircSum<R> acc)
 {
     using C = typename CT<R>::T;
     C *phi = reinterpret_cast<C *>(circ_smem) + off, *lam = phi + ((size_t)1 << Tl);
     constexpr int RB = K + (MIR ? 1 : 0), NR = 1 << RB, H = 1 << K;
     const uint32_t items = 1u << (Tl - RB), full = (1u << Tl) - 1u, gm = (uint32_t)(H - 1) << q0;
     R sc = run;
-    double sum = 0.0;
     for (uint32_t it = threadIdx.x; it < items; it += blockDim.x) {
         const uint32_t i = ((it >> q0) << (q0 + K)) | (it & ((1u << q0) - 1u));
         const uint32_t s0 = cswz(i), s1 = MIR ? cswz(i ^ full ^ gm) : 0u;
@@ -103,7 +123,6 @@ __device__ __noinline__ CircMix<R> circ_stage(uint32_t off, int Tl, int q0, int 
                 l[r] = lam[x];
         }
         sc = run;
-        R gb = 0;
 #pragma unroll
         for (int k = 0; k < K; k++) {
             C ipp[2], ipn[2];
@@ -124,7 +143,7 @@ __device__ __noinline__ CircMix<R> circ_stage(uint32_t off, int Tl, int q0, int 
             if constexpr (NV == 2) {
                 const R q = ((ipp[0].x + ipp[0].y) + (ipp[1].x + ipp[1].y)) -
                             ((ipn[0].x + ipn[0].y) + (ipn[1].x + ipn[1].y));
-                gb = fma(q, sc * sc, gb);
+                acc.add(q * (sc * sc));
             }
             sc *= f;
         }
@@ -132,11 +151,9 @@ __device__ __noinline__ CircMix<R> circ_stage(uint32_t off, int Tl, int q0, int 
             const R sg = (__popc(i) & 1) ? -sg0 : sg0;
             const R q = sg * mix_mirror<R, NV, RB, NV == 1>(pair, sg * t, a, l);
             if constexpr (NV == 2)
-                gb = fma(q, sc * sc, gb);
+                acc.add(q * (sc * sc));
             sc *= f;
         }
-        if constexpr (NV == 2)
-            sum += (double)gb;
 #pragma unroll
         for (int r = 0; r < NR; r++) {
             const uint32_t x = (MIR && r >= H ? s1 : s0) ^ cswz((uint32_t)(r & (H - 1)) << q0);
@@ -149,7 +166,7 @@ __device__ __noinline__ CircMix<R> circ_stage(uint32_t off, int Tl, int q0, int 
 #pragma unroll
     for (int k = 0; k < RB; k++)  // (threads without an item too)
         run *= f;
-    return CircMix<R>{run, acc + sum};
+    return CircMix<R>{run, acc};
 }
 
 // The mixer's part in one layout: local bits q0..q1-1, and vertex n - 1 if
@@ -480,7 +497,7 @@ __global__ void __launch_bounds__(512) k_circuit(const __grid_constant__ Circuit
                         return;
                     high ^= 1;
                 }
-                circ_mix<R, 1>(X, high ? hq0 : 0, high ? hq1 : Tl, high || c == 0, t, f, CircMix<R>{(R)1, 0.0});
+                circ_mix<R, 1>(X, high ? hq0 : 0, high ? hq1 : Tl, high || c == 0, t, f, CircMix<R>{(R)1, {}});
             }
         }
 
@@ -488,11 +505,10 @@ __global__ void __launch_bounds__(512) k_circuit(const __grid_constant__ Circuit
         {
             C *phi = vec + X.off, *lam = phi + NL;
             const R fn = (R)lay[p - 1].fn;
-            double e = 0.0;
+            CircSum<R> es;
             for (uint32_t i0 = 4u * tid; i0 < NL; i0 += 4u * nt) {
                 const int4 o4 = circ_cuts(s_obs, s_ow, Ko, m, circ_index(X, high, i0));
                 const int ov[4] = {o4.x, o4.y, o4.z, o4.w};
-                R es = 0;
 #pragma unroll
                 for (int j = 0; j < 4; j++) {
                     const uint32_t x = cswz(i0 + j);
@@ -500,14 +516,14 @@ __global__ void __launch_bounds__(512) k_circuit(const __grid_constant__ Circuit
                     v.x *= fn;
                     v.y *= fn;
                     const R o = (R)ov[j];
-                    es += (v.x * v.x + v.y * v.y) * o;
+                    es.add((v.x * v.x + v.y * v.y) * o);
                     if (GRAD || A.state)
                         phi[x] = v;
                     if (GRAD)
                         lam[x] = mkc<C>(v.x * o, v.y * o);
                 }
-                e += (double)es;
             }
+            double e = es.value();
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1)
                 e += __shfl_xor_sync(0xffffffffu, e, o);
@@ -533,7 +549,7 @@ __global__ void __launch_bounds__(512) k_circuit(const __grid_constant__ Circuit
         if constexpr (GRAD) {
             for (int l = p - 1; l >= 0; l--) {
                 const R t = (R)-lay[l].t, f = (R)lay[l].fi;
-                CircMix<R> M{(R)1, 0.0};
+                CircMix<R> M{(R)1, {}};
                 for (int part = 0; part < (c ? 2 : 1); part++) {
                     if (part) {
                         if (!exchange(high, true))
@@ -545,19 +561,19 @@ __global__ void __launch_bounds__(512) k_circuit(const __grid_constant__ Circuit
                 // dE/dgamma (both vectors carry 1/f^n) and the inverse cost phase
                 C *phi = vec + X.off, *lam = phi + NL;
                 const C *T = l > 0 ? layer_table(l) + tab_len : nullptr;
-                R g = 0;
+                CircSum<R> g;
                 for (uint32_t i = tid; i < NL; i += nt) {
                     const uint32_t x = cswz(i);
                     const int cv = cval[(size_t)high * NL + i];
                     const C u = phi[x], v = lam[x];
-                    g = fma((R)cv, im_conj_mul(v, u), g);
+                    g.add((R)cv * im_conj_mul(v, u));
                     if (l > 0) {
                         const C z = T[cv];
                         phi[x] = cmul(u, z);
                         lam[x] = cmul(v, z);
                     }
                 }
-                double gb = M.acc, gg = (double)g * (lay[l].fn * lay[l].fn);
+                double gb = M.acc.value(), gg = g.value() * (lay[l].fn * lay[l].fn);
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) {
                     gg += __shfl_xor_sync(0xffffffffu, gg, o);
