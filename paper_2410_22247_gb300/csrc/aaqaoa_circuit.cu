@@ -292,7 +292,7 @@ __global__ void __launch_bounds__(512) k_circuit(const __grid_constant__ Circuit
     X.km = A.km;
     X.pair = (m & 1) ? 1 : 2;
     X.off = 0;
-    const unsigned team = blockIdx.x >> c, teams = gridDim.x >> c;
+    const unsigned b = blockIdx.x >> c;  // the team's point
 
     // The error flag of earlier launches that was not fetched yet. A team stops (its
     // counters are not at zero); a host call that reads no other word back gets it.
@@ -310,330 +310,318 @@ __global__ void __launch_bounds__(512) k_circuit(const __grid_constant__ Circuit
     // A team that gives up leaves NaN in its point's row, not what an earlier call put
     // there (each CTA that gives up writes it; no other result follows, since the
     // last CTA to finish writes that and needs all of them).
-    auto give_up = [&](unsigned b) {
+    auto give_up = [&] {
         for (int r = tid; r < rows; r += nt)
             A.out[(size_t)b * A.out_stride + r] = __longlong_as_double(0x7ff8000000000000ll);
     };
     if (!CL && s_stop) {
-        give_up(team);
+        give_up();
         return;
     }
 
-    for (unsigned b = team; b < (unsigned)A.B; b += teams) {
-        // cut functions. A graph per point reads all classes, so that no load waits
-        // for their number; one graph's are launch constants, only those in use (a
-        // constant read by lane-dependent index costs one access per lane).
-        const bool fresh = b == team || A.fns;
-        const GraphFns *const pt = A.fns ? A.fns + b : nullptr;
-        const int Kc = pt ? pt->cost.K : A.fn[0].K, Ko = pt ? pt->obs[A.obs].K : A.fn[1].K;
-        if (fresh) {
-            if (pt) {
-                const CutFn &cost = pt->cost, &obs = pt->obs[A.obs];
-                for (int i = tid; i < MAXK * CIRC_MAXN; i += nt) {
-                    const int k = i / CIRC_MAXN, u = i % CIRC_MAXN;
-                    s_cost[i] = u < n ? (uint32_t)cost.nbr[k][u] : 0u;
-                    s_obs[i] = u < n ? (uint32_t)obs.nbr[k][u] : 0u;
-                }
-                if (tid < MAXK) {
-                    s_cw[tid] = cost.w[tid];
-                    s_ow[tid] = obs.w[tid];
-                }
-            } else {
-                for (int i = tid; i < (Kc + Ko) * CIRC_MAXN; i += nt) {
-                    const int e = i >= Kc * CIRC_MAXN, j = e ? i - Kc * CIRC_MAXN : i;
-                    (e ? s_obs : s_cost)[j] = A.fn[e].nbr[j / CIRC_MAXN][j % CIRC_MAXN];
-                }
-                for (int k = tid; k < 2 * MAXK; k += nt)
-                    (k < MAXK ? s_cw : s_ow)[k % MAXK] = A.fn[k / MAXK].w[k % MAXK];
+    // cut functions. A graph per point reads all classes, so that no load waits
+    // for their number; one graph's are launch constants, only those in use (a
+    // constant read by lane-dependent index costs one access per lane).
+    const GraphFns *const pt = A.fns ? A.fns + b : nullptr;
+    const int Kc = pt ? pt->cost.K : A.fn[0].K, Ko = pt ? pt->obs[A.obs].K : A.fn[1].K;
+    if (pt) {
+        const CutFn &cost = pt->cost, &obs = pt->obs[A.obs];
+        for (int i = tid; i < MAXK * CIRC_MAXN; i += nt) {
+            const int k = i / CIRC_MAXN, u = i % CIRC_MAXN;
+            s_cost[i] = u < n ? (uint32_t)cost.nbr[k][u] : 0u;
+            s_obs[i] = u < n ? (uint32_t)obs.nbr[k][u] : 0u;
+        }
+        if (tid < MAXK) {
+            s_cw[tid] = cost.w[tid];
+            s_ow[tid] = obs.w[tid];
+        }
+    } else {
+        for (int i = tid; i < (Kc + Ko) * CIRC_MAXN; i += nt) {
+            const int e = i >= Kc * CIRC_MAXN, j = e ? i - Kc * CIRC_MAXN : i;
+            (e ? s_obs : s_cost)[j] = A.fn[e].nbr[j / CIRC_MAXN][j % CIRC_MAXN];
+        }
+        for (int k = tid; k < 2 * MAXK; k += nt)
+            (k < MAXK ? s_cw : s_ow)[k % MAXK] = A.fn[k / MAXK].w[k % MAXK];
+    }
+    __syncthreads();
+    const double *gam = A.gamma ? A.gamma + (size_t)b * p : A.ang, *bet = A.gamma ? A.beta + (size_t)b * p : A.ang + p;
+    // ------------------------------------------------ angles, tables
+    // Warps take layers, lanes table entries; the first entry of a lane is
+    // computed beside the mixer's angles (the last warps), its scale
+    // follows once those are known.
+    double2 z0 = make_double2(1.0, 0.0);
+    if (A.resident && warp < p && lane < tab_len)
+        z0 = phase_sincos(gam[warp] * (double)lane);
+    for (int l = nt - 1 - tid; l < p; l += nt) {
+        const double2 z = phase_sincos(bet[l]);
+        const bool sh = fabs(z.y) > fabs(z.x);  // rotate by beta - pi/2 (see rot)
+        double t;
+        MixFactor m;
+        mix_ratio<R>(sh ? -z.x : z.y, sh ? z.y : z.x, t, m);
+        const double fn = mix_power<R>(m, n);
+        lay[l] = CircLayer{m.f, sh ? -m.f : m.f, fn, (sh && (n & 1)) ? -fn : fn, t};
+    }
+    // cut values of the tile's states in both layouts
+    for (int h = 0; h < (c > 0 ? 2 : 1); h++)
+        for (uint32_t i = 4u * tid; i < NL; i += 4u * nt) {
+            const int4 v = circ_cuts(s_cost, s_cw, Kc, m, circ_index(X, h, i));
+            *reinterpret_cast<uint2 *>(cval + (size_t)h * NL + i) =
+                make_uint2((uint32_t)v.x | ((uint32_t)v.y << 16), (uint32_t)v.z | ((uint32_t)v.w << 16));
+        }
+    __syncthreads();
+    auto entry = [&](int l, int c0, double2 z, C *dst) {  // [0] forward, [1] inverse
+        const double fs = l > 0 ? lay[l - 1].fn : 1.0, fb = lay[l].fin;
+        dst[c0] = mkc<C>((R)(z.x * fs), (R)(-z.y * fs));
+        dst[tab_len + c0] = mkc<C>((R)(z.x * fb), (R)(z.y * fb));
+    };
+    if (A.resident) {
+        for (int l = warp; l < p; l += nw)
+            for (int i = lane; i < tab_len; i += 32) {
+                const double2 z = l == warp && i == lane ? z0 : phase_sincos(gam[l] * (double)i);
+                entry(l, i, z, tabs + (size_t)2 * l * tab_len);
             }
-            __syncthreads();
-        }
-        const double *gam = A.gamma ? A.gamma + (size_t)b * p : A.ang, *bet = A.gamma ? A.beta + (size_t)b * p : A.ang + p;
-        // ------------------------------------------------ angles, tables
-        // Warps take layers, lanes table entries; the first entry of a lane is
-        // computed beside the mixer's angles (the last warps), its scale
-        // follows once those are known.
-        double2 z0 = make_double2(1.0, 0.0);
-        if (A.resident && warp < p && lane < tab_len)
-            z0 = phase_sincos(gam[warp] * (double)lane);
-        for (int l = nt - 1 - tid; l < p; l += nt) {
-            const double2 z = phase_sincos(bet[l]);
-            const bool sh = fabs(z.y) > fabs(z.x);  // rotate by beta - pi/2 (see rot)
-            double t;
-            MixFactor m;
-            mix_ratio<R>(sh ? -z.x : z.y, sh ? z.y : z.x, t, m);
-            const double fn = mix_power<R>(m, n);
-            lay[l] = CircLayer{m.f, sh ? -m.f : m.f, fn, (sh && (n & 1)) ? -fn : fn, t};
-        }
-        // cut values of the tile's states in both layouts
-        if (fresh)
-            for (int h = 0; h < (c > 0 ? 2 : 1); h++)
-                for (uint32_t i = 4u * tid; i < NL; i += 4u * nt) {
-                    const int4 v = circ_cuts(s_cost, s_cw, Kc, m, circ_index(X, h, i));
-                    *reinterpret_cast<uint2 *>(cval + (size_t)h * NL + i) =
-                        make_uint2((uint32_t)v.x | ((uint32_t)v.y << 16), (uint32_t)v.z | ((uint32_t)v.w << 16));
-                }
         __syncthreads();
-        auto entry = [&](int l, int c0, double2 z, C *dst) {  // [0] forward, [1] inverse
-            const double fs = l > 0 ? lay[l - 1].fn : 1.0, fb = lay[l].fin;
-            dst[c0] = mkc<C>((R)(z.x * fs), (R)(-z.y * fs));
-            dst[tab_len + c0] = mkc<C>((R)(z.x * fb), (R)(z.y * fb));
-        };
-        if (A.resident) {
-            for (int l = warp; l < p; l += nw)
-                for (int i = lane; i < tab_len; i += 32) {
-                    const double2 z = l == warp && i == lane ? z0 : phase_sincos(gam[l] * (double)i);
-                    entry(l, i, z, tabs + (size_t)2 * l * tab_len);
-                }
-            __syncthreads();
-        }
-        auto layer_table = [&](int l) -> const C * {
-            if (A.resident)
-                return tabs + (size_t)2 * l * tab_len;
-            __syncthreads();
-            for (int i = tid; i < tab_len; i += nt)
-                entry(l, i, phase_sincos(gam[l] * (double)i), tabs);
-            __syncthreads();
-            return tabs;
-        };
+    }
+    auto layer_table = [&](int l) -> const C * {
+        if (A.resident)
+            return tabs + (size_t)2 * l * tab_len;
+        __syncthreads();
+        for (int i = tid; i < tab_len; i += nt)
+            entry(l, i, phase_sincos(gam[l] * (double)i), tabs);
+        __syncthreads();
+        return tabs;
+    };
 
-        // exchange of the tiles between the layouts (all CTAs of the team)
-        C *xphi = c && !CL ? reinterpret_cast<C *>(A.phi) + ((size_t)b << n) : nullptr;
-        C *xlam = c && !CL && GRAD ? reinterpret_cast<C *>(A.lam) + ((size_t)b << n) : nullptr;
-        unsigned arrivals = 0;
-        int parity = 0;
-        auto exchange = [&](int from, bool both) -> bool {
-            C *phi = vec + X.off, *lam = phi + NL;
-            if constexpr (CL) {  // every amplitude straight to its place in the other layout
-                X.off ^= (uint32_t)NV * NL;
-                const uint32_t dst = smem_u32(vec + X.off), amask = (1u << X.a) - 1u, fm = (2u << c) - 1u;
-#pragma unroll 4
-                for (uint32_t i = tid; i < NL; i += nt) {
-                    const uint32_t y = circ_index(X, from, i), x = cswz(i);
-                    uint32_t r, j;
-                    if (from) {
-                        r = y >> Tl;
-                        j = y & (NL - 1u);
-                    } else {
-                        const uint32_t f = (y >> X.a) & fm, P = f >> c;
-                        r = P ? ~f & (fm >> 1) : f;
-                        j = (P << (Tl - 1)) | ((y >> (X.a + c + 1)) << X.a) | (y & amask);
-                    }
-                    const uint32_t at = circ_map(dst + cswz(j) * (uint32_t)sizeof(C), r);
-                    circ_st(at, phi[x]);
-                    if (GRAD && both)
-                        circ_st(at + NL * (uint32_t)sizeof(C), lam[x]);
-                }
-                circ_cluster_sync();
-                return true;
-            }
-            C *bp = xphi + ((size_t)parity << m), *bl = xlam + ((size_t)parity << m);
-            parity ^= 1;
+    // exchange of the tiles between the layouts (all CTAs of the team)
+    C *xphi = c && !CL ? reinterpret_cast<C *>(A.phi) + ((size_t)b << n) : nullptr;
+    C *xlam = c && !CL && GRAD ? reinterpret_cast<C *>(A.lam) + ((size_t)b << n) : nullptr;
+    unsigned arrivals = 0;
+    int parity = 0;
+    auto exchange = [&](int from, bool both) -> bool {
+        C *phi = vec + X.off, *lam = phi + NL;
+        if constexpr (CL) {  // every amplitude straight to its place in the other layout
+            X.off ^= (uint32_t)NV * NL;
+            const uint32_t dst = smem_u32(vec + X.off), amask = (1u << X.a) - 1u, fm = (2u << c) - 1u;
 #pragma unroll 4
             for (uint32_t i = tid; i < NL; i += nt) {
                 const uint32_t y = circ_index(X, from, i), x = cswz(i);
-                __stcg(bp + y, phi[x]);
+                uint32_t r, j;
+                if (from) {
+                    r = y >> Tl;
+                    j = y & (NL - 1u);
+                } else {
+                    const uint32_t f = (y >> X.a) & fm, P = f >> c;
+                    r = P ? ~f & (fm >> 1) : f;
+                    j = (P << (Tl - 1)) | ((y >> (X.a + c + 1)) << X.a) | (y & amask);
+                }
+                const uint32_t at = circ_map(dst + cswz(j) * (uint32_t)sizeof(C), r);
+                circ_st(at, phi[x]);
                 if (GRAD && both)
-                    __stcg(bl + y, lam[x]);
+                    circ_st(at + NL * (uint32_t)sizeof(C), lam[x]);
             }
-            arrivals += 1u << c;
-            __syncthreads();
-            if (tid == 0) {
-                __threadfence();
-                if (!(A.drop_arrival && X.rank == 0))
-                    atomicAdd(A.bar + b, 1u);
-                const long long t0 = clock64();
-                while (*reinterpret_cast<volatile unsigned *>(A.bar + b) < arrivals)
-                    if (clock64() - t0 > WAIT_BUDGET_CYCLES) {
-                        atomicExch(A.err, 1);
-                        s_stop = 1;
-                        break;
-                    }
-                __threadfence();
-            }
-            __syncthreads();
-            if (s_stop) {
-                give_up(b);
-                return false;
-            }
-#pragma unroll 4
-            for (uint32_t i = tid; i < NL; i += nt) {
-                const uint32_t y = circ_index(X, from ^ 1, i), x = cswz(i);
-                phi[x] = __ldcg(bp + y);
-                if (GRAD && both)
-                    lam[x] = __ldcg(bl + y);
-            }
-            __syncthreads();
+            circ_cluster_sync();
             return true;
-        };
-        const int hq0 = Tl - 1 - c, hq1 = Tl - 1;  // the high layout's bits
-
-        // ------------------------------------------------ forward sweep
-        int high = 0;
-        {
-            C *phi = vec + X.off;
-            const C *T = layer_table(0);
-            const R amp0 = (R)A.amp0;
-            for (uint32_t i = tid; i < NL; i += nt) {  // 2^(-n/2) i^|y| times the first cost phase
-                const C z = T[cval[i]];
-                phi[cswz(i)] = circ_turn(mkc<C>(amp0 * z.x, amp0 * z.y), __popc(circ_index(X, 0, i)));
-            }
+        }
+        C *bp = xphi + ((size_t)parity << m), *bl = xlam + ((size_t)parity << m);
+        parity ^= 1;
+#pragma unroll 4
+        for (uint32_t i = tid; i < NL; i += nt) {
+            const uint32_t y = circ_index(X, from, i), x = cswz(i);
+            __stcg(bp + y, phi[x]);
+            if (GRAD && both)
+                __stcg(bl + y, lam[x]);
+        }
+        arrivals += 1u << c;
+        __syncthreads();
+        if (tid == 0) {
+            __threadfence();
+            if (!(A.drop_arrival && X.rank == 0))
+                atomicAdd(A.bar + b, 1u);
+            const long long t0 = clock64();
+            while (*reinterpret_cast<volatile unsigned *>(A.bar + b) < arrivals)
+                if (clock64() - t0 > WAIT_BUDGET_CYCLES) {
+                    atomicExch(A.err, 1);
+                    s_stop = 1;
+                    break;
+                }
+            __threadfence();
         }
         __syncthreads();
-        for (int l = 0; l < p; l++) {
-            if (l > 0) {
-                C *phi = vec + X.off;
-                const C *T = layer_table(l);
-                for (uint32_t i = tid; i < NL; i += nt) {
-                    const uint32_t x = cswz(i);
-                    phi[x] = cmul(phi[x], T[cval[(size_t)high * NL + i]]);
-                }
-                __syncthreads();
+        if (s_stop) {
+            give_up();
+            return false;
+        }
+#pragma unroll 4
+        for (uint32_t i = tid; i < NL; i += nt) {
+            const uint32_t y = circ_index(X, from ^ 1, i), x = cswz(i);
+            phi[x] = __ldcg(bp + y);
+            if (GRAD && both)
+                lam[x] = __ldcg(bl + y);
+        }
+        __syncthreads();
+        return true;
+    };
+    const int hq0 = Tl - 1 - c, hq1 = Tl - 1;  // the high layout's bits
+
+    // ------------------------------------------------ forward sweep
+    int high = 0;
+    {
+        C *phi = vec + X.off;
+        const C *T = layer_table(0);
+        const R amp0 = (R)A.amp0;
+        for (uint32_t i = tid; i < NL; i += nt) {  // 2^(-n/2) i^|y| times the first cost phase
+            const C z = T[cval[i]];
+            phi[cswz(i)] = circ_turn(mkc<C>(amp0 * z.x, amp0 * z.y), __popc(circ_index(X, 0, i)));
+        }
+    }
+    __syncthreads();
+    for (int l = 0; l < p; l++) {
+        if (l > 0) {
+            C *phi = vec + X.off;
+            const C *T = layer_table(l);
+            for (uint32_t i = tid; i < NL; i += nt) {
+                const uint32_t x = cswz(i);
+                phi[x] = cmul(phi[x], T[cval[(size_t)high * NL + i]]);
             }
-            const R t = (R)lay[l].t, f = (R)lay[l].f;
+            __syncthreads();
+        }
+        const R t = (R)lay[l].t, f = (R)lay[l].f;
+        for (int part = 0; part < (c ? 2 : 1); part++) {
+            if (part) {
+                if (!exchange(high, false))
+                    return;
+                high ^= 1;
+            }
+            circ_mix<R, 1>(X, high ? hq0 : 0, high ? hq1 : Tl, high || c == 0, t, f, CircMix<R>{(R)1, {}});
+        }
+    }
+
+    // ------------------------------ energy, lambda = O phi, the state
+    {
+        C *phi = vec + X.off, *lam = phi + NL;
+        const R fn = (R)lay[p - 1].fn;
+        CircSum<R> es;
+        for (uint32_t i0 = 4u * tid; i0 < NL; i0 += 4u * nt) {
+            const int4 o4 = circ_cuts(s_obs, s_ow, Ko, m, circ_index(X, high, i0));
+            const int ov[4] = {o4.x, o4.y, o4.z, o4.w};
+#pragma unroll
+            for (int j = 0; j < 4; j++) {
+                const uint32_t x = cswz(i0 + j);
+                C v = phi[x];
+                v.x *= fn;
+                v.y *= fn;
+                const R o = (R)ov[j];
+                es.add((v.x * v.x + v.y * v.y) * o);
+                if (GRAD || A.state)
+                    phi[x] = v;
+                if (GRAD)
+                    lam[x] = mkc<C>(v.x * o, v.y * o);
+            }
+        }
+        double e = es.value();
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+            e += __shfl_xor_sync(0xffffffffu, e, o);
+        if (lane == 0)
+            red[warp] = e;
+    }
+    __syncthreads();
+    if (A.state) {  // psi(x) = (-i)^(nK) i^(-|x|) psi~(x) and psi(~x) = psi(x)
+        int K = 0;
+        for (int l = 0; l < p; l++)
+            K += lay[l].fi == lay[l].f ? 0 : 1;
+        const C *phi = vec + X.off;
+        C *dst = reinterpret_cast<C *>(A.state) + ((size_t)b << n);
+        for (uint32_t i = tid; i < NL; i += nt) {
+            const uint32_t y = circ_index(X, high, i);
+            const C v = circ_turn(phi[cswz(i)], 4 * CIRC_MAXN - ((n * K) & 3) - __popc(y));
+            dst[y] = v;
+            dst[(2u << m) - 1u - y] = v;
+        }
+    }
+
+    // ------------------------------------------------- adjoint sweep
+    if constexpr (GRAD) {
+        for (int l = p - 1; l >= 0; l--) {
+            const R t = (R)-lay[l].t, f = (R)lay[l].fi;
+            CircMix<R> M{(R)1, {}};
             for (int part = 0; part < (c ? 2 : 1); part++) {
                 if (part) {
-                    if (!exchange(high, false))
+                    if (!exchange(high, true))
                         return;
                     high ^= 1;
                 }
-                circ_mix<R, 1>(X, high ? hq0 : 0, high ? hq1 : Tl, high || c == 0, t, f, CircMix<R>{(R)1, {}});
+                M = circ_mix<R, NV>(X, high ? hq0 : 0, high ? hq1 : Tl, high || c == 0, t, f, M);
             }
-        }
-
-        // ------------------------------ energy, lambda = O phi, the state
-        {
+            // dE/dgamma (both vectors carry 1/f^n) and the inverse cost phase
             C *phi = vec + X.off, *lam = phi + NL;
-            const R fn = (R)lay[p - 1].fn;
-            CircSum<R> es;
-            for (uint32_t i0 = 4u * tid; i0 < NL; i0 += 4u * nt) {
-                const int4 o4 = circ_cuts(s_obs, s_ow, Ko, m, circ_index(X, high, i0));
-                const int ov[4] = {o4.x, o4.y, o4.z, o4.w};
-#pragma unroll
-                for (int j = 0; j < 4; j++) {
-                    const uint32_t x = cswz(i0 + j);
-                    C v = phi[x];
-                    v.x *= fn;
-                    v.y *= fn;
-                    const R o = (R)ov[j];
-                    es.add((v.x * v.x + v.y * v.y) * o);
-                    if (GRAD || A.state)
-                        phi[x] = v;
-                    if (GRAD)
-                        lam[x] = mkc<C>(v.x * o, v.y * o);
-                }
-            }
-            double e = es.value();
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1)
-                e += __shfl_xor_sync(0xffffffffu, e, o);
-            if (lane == 0)
-                red[warp] = e;
-        }
-        __syncthreads();
-        if (A.state) {  // psi(x) = (-i)^(nK) i^(-|x|) psi~(x) and psi(~x) = psi(x)
-            int K = 0;
-            for (int l = 0; l < p; l++)
-                K += lay[l].fi == lay[l].f ? 0 : 1;
-            const C *phi = vec + X.off;
-            C *dst = reinterpret_cast<C *>(A.state) + ((size_t)b << n);
+            const C *T = l > 0 ? layer_table(l) + tab_len : nullptr;
+            CircSum<R> g;
             for (uint32_t i = tid; i < NL; i += nt) {
-                const uint32_t y = circ_index(X, high, i);
-                const C v = circ_turn(phi[cswz(i)], 4 * CIRC_MAXN - ((n * K) & 3) - __popc(y));
-                dst[y] = v;
-                dst[(2u << m) - 1u - y] = v;
+                const uint32_t x = cswz(i);
+                const int cv = cval[(size_t)high * NL + i];
+                const C u = phi[x], v = lam[x];
+                g.add((R)cv * im_conj_mul(v, u));
+                if (l > 0) {
+                    const C z = T[cv];
+                    phi[x] = cmul(u, z);
+                    lam[x] = cmul(v, z);
+                }
             }
-        }
-
-        // ------------------------------------------------- adjoint sweep
-        if constexpr (GRAD) {
-            for (int l = p - 1; l >= 0; l--) {
-                const R t = (R)-lay[l].t, f = (R)lay[l].fi;
-                CircMix<R> M{(R)1, {}};
-                for (int part = 0; part < (c ? 2 : 1); part++) {
-                    if (part) {
-                        if (!exchange(high, true))
-                            return;
-                        high ^= 1;
-                    }
-                    M = circ_mix<R, NV>(X, high ? hq0 : 0, high ? hq1 : Tl, high || c == 0, t, f, M);
-                }
-                // dE/dgamma (both vectors carry 1/f^n) and the inverse cost phase
-                C *phi = vec + X.off, *lam = phi + NL;
-                const C *T = l > 0 ? layer_table(l) + tab_len : nullptr;
-                CircSum<R> g;
-                for (uint32_t i = tid; i < NL; i += nt) {
-                    const uint32_t x = cswz(i);
-                    const int cv = cval[(size_t)high * NL + i];
-                    const C u = phi[x], v = lam[x];
-                    g.add((R)cv * im_conj_mul(v, u));
-                    if (l > 0) {
-                        const C z = T[cv];
-                        phi[x] = cmul(u, z);
-                        lam[x] = cmul(v, z);
-                    }
-                }
-                double gb = M.acc.value(), gg = g.value() * (lay[l].fn * lay[l].fn);
+            double gb = M.acc.value(), gg = g.value() * (lay[l].fn * lay[l].fn);
 #pragma unroll
-                for (int o = 16; o > 0; o >>= 1) {
-                    gg += __shfl_xor_sync(0xffffffffu, gg, o);
-                    gb += __shfl_xor_sync(0xffffffffu, gb, o);
-                }
-                if (lane == 0) {
-                    red[(1 + l) * nw + warp] = gg;
-                    red[(1 + p + l) * nw + warp] = gb;
-                }
-                __syncthreads();
+            for (int o = 16; o > 0; o >>= 1) {
+                gg += __shfl_xor_sync(0xffffffffu, gg, o);
+                gb += __shfl_xor_sync(0xffffffffu, gb, o);
             }
+            if (lane == 0) {
+                red[(1 + l) * nw + warp] = gg;
+                red[(1 + p + l) * nw + warp] = gb;
+            }
+            __syncthreads();
         }
+    }
 
-        // -------------------------------------------------- the results
-        if (A.err_out && tid == 0 && X.rank == 0)
-            *A.err_out = pending;
-        // sums over the stored half count twice; dE/dgamma and dE/dbeta are
-        // 2 Im of theirs. A team's CTAs are added in rank order.
-        double *part = CL ? nullptr : A.partials + (((size_t)b * rows) << c);
-        for (int r = tid; r < rows; r += nt) {
-            double s = 0.0;
-            for (int w = 0; w < nw; w++)
-                s += red[r * nw + w];
-            if (c == 0)
+    // -------------------------------------------------- the results
+    if (A.err_out && tid == 0 && X.rank == 0)
+        *A.err_out = pending;
+    // sums over the stored half count twice; dE/dgamma and dE/dbeta are
+    // 2 Im of theirs. A team's CTAs are added in rank order.
+    double *part = CL ? nullptr : A.partials + (((size_t)b * rows) << c);
+    for (int r = tid; r < rows; r += nt) {
+        double s = 0.0;
+        for (int w = 0; w < nw; w++)
+            s += red[r * nw + w];
+        if (c == 0)
+            A.out[(size_t)b * A.out_stride + r] = (r ? 4.0 : 2.0) * s;
+        else if (CL)
+            circ_st(circ_map(smem_u32(xred + ((size_t)r << c) + X.rank), 0), s);
+        else
+            __stcg(part + ((size_t)r << c) + X.rank, s);
+    }
+    if (c) {
+        bool mine = X.rank == 0;
+        if constexpr (CL) {
+            circ_cluster_sync();
+        } else {
+            __syncthreads();
+            if (tid == 0) {
+                __threadfence();
+                s_last = atomicAdd(A.bar + b, 1u) == arrivals + (1u << c) - 1u;
+                __threadfence();
+            }
+            __syncthreads();
+            mine = s_last;
+        }
+        if (mine) {
+            for (int r = tid; r < rows; r += nt) {
+                double s = 0.0;
+                for (int k = 0; k < (1 << c); k++)
+                    s += CL ? xred[((size_t)r << c) + k] : __ldcg(part + ((size_t)r << c) + k);
                 A.out[(size_t)b * A.out_stride + r] = (r ? 4.0 : 2.0) * s;
-            else if (CL)
-                circ_st(circ_map(smem_u32(xred + ((size_t)r << c) + X.rank), 0), s);
-            else
-                __stcg(part + ((size_t)r << c) + X.rank, s);
-        }
-        if (c) {
-            bool mine = X.rank == 0;
-            if constexpr (CL) {
-                circ_cluster_sync();
-            } else {
-                __syncthreads();
-                if (tid == 0) {
-                    __threadfence();
-                    s_last = atomicAdd(A.bar + b, 1u) == arrivals + (1u << c) - 1u;
-                    __threadfence();
-                }
-                __syncthreads();
-                mine = s_last;
             }
-            if (mine) {
-                for (int r = tid; r < rows; r += nt) {
-                    double s = 0.0;
-                    for (int k = 0; k < (1 << c); k++)
-                        s += CL ? xred[((size_t)r << c) + k] : __ldcg(part + ((size_t)r << c) + k);
-                    A.out[(size_t)b * A.out_stride + r] = (r ? 4.0 : 2.0) * s;
-                }
-                if (!CL && tid == 0)
-                    A.bar[b] = 0u;  // every CTA is past its waits
-            }
-        }
-        if (b + teams < (unsigned)A.B) {  // the next point reuses the shared memory
-            if (CL)
-                circ_cluster_sync();
-            else
-                __syncthreads();
+            if (!CL && tid == 0)
+                A.bar[b] = 0u;  // every CTA is past its waits
         }
     }
 }
@@ -677,7 +665,6 @@ static bool circuit_shape(bool c128, bool grad, int n, int p, int tab_len, int B
     }
     if (q->resident < 0)
         return false;
-    q->teams = B;
     if (c && !q->cluster) {  // the CTAs of a team wait for one another: all are resident
         if (B > (device_sms() >> c) || B > CIRCUIT_MAX_POINTS)
             return false;
@@ -747,7 +734,7 @@ static int launch_circuit_t(const CircuitArgs &a, const CircuitPlan &q, cudaStre
         at[0].id = cudaLaunchAttributeCooperative;
         at[0].val.cooperative = 1;
     }
-    cfg.gridDim = dim3((unsigned)q.teams << q.c);
+    cfg.gridDim = dim3((unsigned)a.B << q.c);
     cfg.blockDim = dim3(q.nt);
     cfg.dynamicSmemBytes = q.smem;
     cfg.stream = st;

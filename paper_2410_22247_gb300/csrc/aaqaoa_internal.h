@@ -176,7 +176,7 @@ struct CircuitArgs {
 static_assert(sizeof(CircuitArgs) <= 4096, "kernel arguments of the classic size");
 // the kernel's shape for a call, from circuit_plan (false: the call does not fit it)
 struct CircuitPlan {
-    int c, Tl, a, km, nt, teams, resident;
+    int c, Tl, a, km, nt, resident;
     int cluster;         // the 2^c CTAs are a cluster; else they exchange through global memory
     size_t smem;
 };
