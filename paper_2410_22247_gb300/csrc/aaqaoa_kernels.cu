@@ -835,12 +835,11 @@ template <> struct LaneSum<float> {
         const float e = __fadd_rn(__fsub_rn(a, __fsub_rn(t, z)), __fsub_rn(b, z));
         return {t, __fadd_rn(__fadd_rn(la, lb), e)};
     }
-    // sums of chunks: the rounded parts in FP64, the rounding errors (2^-24 of
-    // them) in float
-    __device__ __forceinline__ void add_to(double &a, float &b, bool neg) const
+    // sums of chunks in FP64
+    __device__ __forceinline__ void add_to(double &a, bool neg) const
     {
-        a += (double)(neg ? -hi : hi);
-        b += neg ? -lo : lo;
+        const double v = (double)hi + (double)lo;
+        a += neg ? -v : v;
     }
 };
 template <> struct LaneSum<double> {
@@ -850,7 +849,7 @@ template <> struct LaneSum<double> {
     {
         return {(neg ? -v : v) + __shfl_xor_sync(0xffffffffu, v, o)};
     }
-    __device__ __forceinline__ void add_to(double &a, float &, bool neg) const { a += neg ? -v : v; }
+    __device__ __forceinline__ void add_to(double &a, bool neg) const { a += neg ? -v : v; }
 };
 
 template <typename R>
@@ -925,7 +924,6 @@ __global__ void __launch_bounds__(256, std::is_same<R, float>::value ? 2 : 1) k_
             }
         }
         double acc[2] = {0.0, 0.0}, pacc[PAIRS];
-        float accl[2] = {0.f, 0.f};
 #pragma unroll
         for (int i = 0; i < PAIRS; i++)
             pacc[i] = 0.0;
@@ -975,12 +973,12 @@ __global__ void __launch_bounds__(256, std::is_same<R, float>::value ? 2 : 1) k_
 #pragma unroll
             for (int q = 0; q < 2; q++)
                 if (idx[q] >= 0)
-                    vals[warp][idx[q]].add_to(acc[q], accl[q], __popcll((ch << 10) & cmask[q]) & 1);
+                    vals[warp][idx[q]].add_to(acc[q], __popcll((ch << 10) & cmask[q]) & 1);
         }
 #pragma unroll
         for (int q = 0; q < 2; q++)
             if (idx[q] >= 0)
-                wsum[lane + 32 * q][warp] = acc[q] + (double)accl[q];
+                wsum[lane + 32 * q][warp] = acc[q];
 #pragma unroll
         for (int i = 0; i < PAIRS; i++)
             if ((needp >> i) & 1) {
