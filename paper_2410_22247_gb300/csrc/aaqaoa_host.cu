@@ -168,6 +168,7 @@ struct aaqaoa_plan {
     std::unique_ptr<double[]> angles;  // gamma and beta of the host call in flight (upload_params)
     double *slot = nullptr;  // pinned result row of one-point host calls (HostSlots)
     bool forced = false;  // the caller set the pass plan (aaqaoa_set_pass_plan)
+    std::array<int, 4> tuned{};  // the plan that aaqaoa_autotune returned (zeros: none)
     bool fuse = true;  // fuse layer boundaries into one pass where the plan allows
     int *err_shared = nullptr;  // set when the plan is part of a multi-graph batch
     const GraphFns *pt_dev = nullptr;  // set for a group of same-n graphs: point b is graph b
@@ -1607,7 +1608,9 @@ int aaqaoa_set_workspace(aaqaoa_plan *pl, void *device_ptr, size_t bytes, int ba
 // ------------------------------------------------- pass plans, autotune
 // A layer's qubits per pass (the low pass's qubit count L and the number K of
 // high passes) for the forward (nv = 1) and the two-vector adjoint (nv = 2)
-// passes. 0 selects the default of build_passes().
+// passes. 0 selects the default of build_passes(). A gradient's forward passes are
+// the forward's if the caller asks for others than the default (forced), else
+// those that follow the adjoint (gradient_passes).
 static int set_layers(aaqaoa_plan *pl, const int plan4[4], bool forced = false)
 {
     if (pl->small())
@@ -1618,6 +1621,8 @@ static int set_layers(aaqaoa_plan *pl, const int plan4[4], bool forced = false)
         pass_geometry(pl->c128, nv, &T, &CB, &HB);
         const int L2 = low_two_stage_bits(pl->c128, nv);
         default_layer(pl->n, T, CB, HB, L2, &L, &K, nv == 2);
+        if (nv == 1)
+            forced = forced && ((plan4[0] > 0 && plan4[0] != L) || (plan4[1] > 0 && plan4[1] != K));
         if (plan4[2 * (nv - 1)] > 0)
             L = plan4[2 * (nv - 1)];
         if (plan4[2 * (nv - 1) + 1] > 0)
@@ -1653,7 +1658,8 @@ int aaqaoa_set_pass_plan(aaqaoa_plan *pl, int fwd_low, int fwd_high, int bwd_low
     if (fwd_low < 0 || fwd_high < 0 || bwd_low < 0 || bwd_high < 0)
         return fail(AAQAOA_ERR_INVALID_ARG, "negative pass-plan entry");
     const int plan4[4] = {fwd_low, fwd_high, bwd_low, bwd_high};
-    const bool forced = fwd_low || fwd_high || bwd_low || bwd_high;
+    const bool forced = (fwd_low || fwd_high || bwd_low || bwd_high) &&
+                        !std::equal(plan4, plan4 + 4, pl->tuned.begin());
     const int r = set_layers(pl, plan4, forced);
     if (!r)
         pl->forced = forced;
@@ -1767,7 +1773,8 @@ int aaqaoa_autotune(aaqaoa_plan *pl, int *plan4)
         return fail(AAQAOA_ERR_WORKSPACE, "no workspace set (aaqaoa_set_workspace)");
     int r = AAQAOA_OK;
     const char *env = std::getenv("AAQAOA_AUTOTUNE");
-    if (!pl->small() && !(env && env[0] == '0')) {
+    const bool tune = !pl->small() && !(env && env[0] == '0');
+    if (tune) {
         int dev = 0;
         cudaGetDevice(&dev);
         const TuneKey key{dev, pl->c128 ? 1 : 0, pl->n, pl->p, pl->cap, pl->ws_grad ? 1 : 0, plan_fuses(pl) ? 1 : 0};
@@ -1825,9 +1832,18 @@ int aaqaoa_autotune(aaqaoa_plan *pl, int *plan4)
             plan_tune_cache()[key] = best;
         }
     }
-    if (!r && plan4)
-        r = aaqaoa_get_pass_plan(pl, plan4);
-    return r;
+    int now[4] = {0, 0, 0, 0};
+    if (!r)
+        r = aaqaoa_get_pass_plan(pl, now);
+    if (r)
+        return r;
+    if (tune)
+        pl->forced = false;
+    if (!pl->forced)
+        std::copy(now, now + 4, pl->tuned.begin());
+    if (plan4)
+        std::copy(now, now + 4, plan4);
+    return AAQAOA_OK;
 }
 
 int aaqaoa_set_stream(aaqaoa_plan *pl, void *stream)

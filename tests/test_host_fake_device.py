@@ -52,6 +52,16 @@ class FakePlan:
         assert self.buffer.nbytes >= size.value + 256
         assert lib.aaqaoa_set_workspace(self.h, ctypes.c_void_p(at), size.value, batch, int(grad)) == 0
 
+    @classmethod
+    def unbacked(cls, lib, graph, p):
+        """A plan without a workspace (schedules only)."""
+        self = cls.__new__(cls)
+        n, e = graph
+        self.lib, self.p, self.m, self.h = lib, p, len(e), ctypes.c_void_p()
+        e = np.ascontiguousarray(e, dtype=np.int32).reshape(-1)
+        assert lib.aaqaoa_prepare(n, self.m, _p(e), 0, None, None, None, p, 0, None, ctypes.byref(self.h)) == 0
+        return self
+
     def value(self, g, b):
         return 1000.0 * self.m + np.sum(g) + 2.0 * np.sum(b)
 
@@ -190,3 +200,51 @@ def test_device_results_over_their_angles(lib, n):
         assert lib.aaqaoa_sync(pl.h) == 0
         assert abs(out[0] - want) < 1e-9 and np.allclose(out[1:], [0.3, 0.2, 0.1, 0.4])
         pl.close()
+
+
+def _schedules(pl):
+    out = []
+    for mode in (0, 1, 2):
+        rows, cnt = np.zeros((64, 5), dtype=np.int32), ctypes.c_int()
+        assert pl.lib.aaqaoa_get_schedule(pl.h, mode, _p(rows), 64, ctypes.byref(cnt)) == 0
+        out.append(rows[:cnt.value].tolist())
+    return out
+
+
+@pytest.mark.parametrize("n", [14, 18, 20, 22, 24, 27, 30])
+def test_a_tuned_plan_set_again_changes_nothing(lib, n):
+    """set_pass_plan(*autotune()) leaves the calls as they were: one launch up to 20
+    qubits, the gradient's own forward passes above; so does the default written
+    out above 20 qubits. Other plans run as written."""
+    pl = FakePlan(lib, W.cycle_graph(n), 2) if n < 26 else FakePlan.unbacked(lib, W.cycle_graph(n), 2)
+    x, y = np.array([0.3, 0.2]), np.array([0.1, 0.4])
+
+    def launches():
+        if n > 20:
+            return 0
+        before = lib.fake_circuit_launches()
+        assert pl.expect(x, y)[0] == 0
+        return lib.fake_circuit_launches() - before
+
+    plan4 = np.zeros(4, dtype=np.int32)
+    if n < 26:
+        before = _schedules(pl)
+        assert lib.aaqaoa_set_pass_plan(pl.h, 9, 0, 0, 0) in (0, -1)  # (what it was before does not matter)
+        assert lib.aaqaoa_autotune(pl.h, _p(plan4)) == 0
+        tuned = _schedules(pl)
+        assert launches() == (1 if n <= 20 else 0)
+        assert lib.aaqaoa_set_pass_plan(pl.h, *[int(v) for v in plan4]) == 0
+        assert _schedules(pl) == tuned and launches() == (1 if n <= 20 else 0)
+        assert lib.aaqaoa_set_pass_plan(pl.h, 0, 0, 0, 0) == 0
+        assert _schedules(pl) == before
+    else:
+        before = _schedules(pl)
+    other = FakePlan.unbacked(lib, W.cycle_graph(n), 2)
+    assert lib.aaqaoa_get_pass_plan(other.h, _p(plan4)) == 0
+    assert lib.aaqaoa_set_pass_plan(other.h, *[int(v) for v in plan4]) == 0
+    if n > 20:
+        assert _schedules(other) == before
+    if n in (18, 20):
+        assert lib.aaqaoa_set_pass_plan(pl.h, 9, 2, 8, 2) == 0 and launches() == 0
+    other.close()
+    pl.close()
