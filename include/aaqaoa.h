@@ -593,8 +593,9 @@ int aaqaoa_stats(aaqaoa_plan *plan, aaqaoa_stats_t *out);
  * order: per launch its kind (as above), flags (bit 0: the pass carries
  * cut-function work -- phase, lambda = O phi, energy, dE/dgamma, inverse
  * phase; bit 1: a fused layer boundary; bit 2: the cluster low pass; bit 3:
- * the turnaround pass of a gradient evaluation), event duration (ms) and
- * bytes, counted as above. kind, flags, ms, bytes: host arrays of at least max entries, each may
+ * the turnaround pass of a gradient evaluation; bit 4: the launch works on the
+ * stored half of the statevectors and moves half of its bytes), event duration
+ * (ms) and bytes, counted as above. kind, flags, ms, bytes: host arrays of at least max entries, each may
  * be NULL. *count (host int) receives the number of records, also when it
  * exceeds max. Synchronises the plan's stream. INVALID_ARG for a NULL plan
  * or count, or max < 0.

@@ -212,7 +212,9 @@ class Plan:
         """The launches recorded since profiling was enabled
         (aaqaoa_profile_enable), in order: dicts of kind (0 forward pass,
         1 adjoint pass, 2 whole circuit, 3 aggregation, 4 parameter tables),
-        cut_work, fused, cluster, turnaround, ms and bytes."""
+        cut_work, fused, cluster, turnaround, ms, bytes (of whole
+        statevectors) and moved, the bytes that the launch loads and stores
+        (half of them for the tiled passes of MaxCut plans)."""
         cnt = ctypes.c_int()
         N.check(N.aaqaoa_profile_launches(self.handle, 0, ctypes.byref(cnt), None, None, None, None),
                 "aaqaoa_profile_launches")
@@ -226,7 +228,8 @@ class Plan:
                                           _ptr(by, ctypes.c_double)), "aaqaoa_profile_launches")
         return [{"kind": int(kind[i]), "cut_work": bool(flags[i] & 1), "fused": bool(flags[i] & 2),
                  "cluster": bool(flags[i] & 4), "turnaround": bool(flags[i] & 8),
-                 "ms": float(ms[i]), "bytes": float(by[i])} for i in range(n)]
+                 "ms": float(ms[i]), "bytes": float(by[i]),
+                 "moved": float(by[i]) * (0.5 if flags[i] & 16 else 1.0)} for i in range(n)]
 
     def autotune(self):
         """Time the candidate pass plans and keep the fastest; returns pass_plan()."""

@@ -142,7 +142,7 @@ struct aaqaoa_plan {
     bool prof = false;
     struct ProfRec {
         int kind;
-        int flags;  // bit 0: cut-function work, bit 1: fused layer boundary
+        int flags;  // as aaqaoa_profile_launches
         double bytes;
         cudaEvent_t a, b;
     };
@@ -229,7 +229,7 @@ struct ProfScope {
         if (pl->prof) {
             cudaEvent_t b = prof_event(pl);
             cudaEventRecord(b, pl->stream);
-            pl->prof_recs.push_back({kind, flags, bytes, a, b});
+            pl->prof_recs.push_back({kind, flags | (bytes > 0 && pl->half() ? 16 : 0), bytes, a, b});
         }
     }
 };

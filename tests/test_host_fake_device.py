@@ -45,12 +45,15 @@ class FakePlan:
         e = np.ascontiguousarray(e, dtype=np.int32).reshape(-1)
         self.h = ctypes.c_void_p()
         assert lib.aaqaoa_prepare(n, self.m, _p(e), 0, None, None, None, p, 0, None, ctypes.byref(self.h)) == 0
+        self.back(batch, grad, buffer)
+
+    def back(self, batch, grad, buffer=None):
         size = ctypes.c_size_t()
-        assert lib.aaqaoa_workspace_bytes(self.h, batch, int(grad), ctypes.byref(size)) == 0
+        assert self.lib.aaqaoa_workspace_bytes(self.h, batch, int(grad), ctypes.byref(size)) == 0
         self.buffer = np.zeros(size.value + 256, dtype=np.uint8) if buffer is None else buffer
         at = (self.buffer.ctypes.data + 255) & ~255
         assert self.buffer.nbytes >= size.value + 256
-        assert lib.aaqaoa_set_workspace(self.h, ctypes.c_void_p(at), size.value, batch, int(grad)) == 0
+        assert self.lib.aaqaoa_set_workspace(self.h, ctypes.c_void_p(at), size.value, batch, int(grad)) == 0
 
     @classmethod
     def unbacked(cls, lib, graph, p):
@@ -247,4 +250,33 @@ def test_a_tuned_plan_set_again_changes_nothing(lib, n):
     if n in (18, 20):
         assert lib.aaqaoa_set_pass_plan(pl.h, 9, 2, 8, 2) == 0 and launches() == 0
     other.close()
+    pl.close()
+
+
+@pytest.mark.parametrize("n,fields", [(22, None), (22, True), (18, None)])
+def test_launch_records_tell_halves_from_whole_states(lib, n, fields):
+    """Passes of a MaxCut plan move half of the bytes that their records count
+    (bit 4 of the flags); those of an Ising plan, with the whole state, all."""
+    x, y = np.array([0.3, 0.2]), np.array([0.1, 0.4])
+    e = np.ascontiguousarray(W.cycle_graph(n)[1], dtype=np.int32).reshape(-1)
+    if fields:
+        pl = FakePlan.unbacked(lib, W.cycle_graph(n), 2)
+        lib.aaqaoa_destroy(pl.h)
+        F = lambda a: a.ctypes.data_as(ctypes.POINTER(ctypes.c_double))
+        w, h = np.ones(len(e) // 2), np.ones(n)
+        pl.h = ctypes.c_void_p()
+        assert lib.aaqaoa_prepare_ising(n, len(e) // 2, _p(e), F(w), F(h), 0, None, None, None, 0, None, None, None, 2,
+                                        0, None, ctypes.byref(pl.h)) == 0
+        pl.back(1, False)
+    else:
+        pl = FakePlan(lib, W.cycle_graph(n), 2, grad=False)
+        assert lib.aaqaoa_set_pass_plan(pl.h, 9, 2 if n > 18 else 1, 0, 0) == 0
+    assert lib.aaqaoa_profile_enable(pl.h, 1) == 0
+    assert pl.expect(x, y)[0] == 0
+    cnt, flags, by = ctypes.c_int(), np.zeros(32, dtype=np.int32), np.zeros(32)
+    assert lib.aaqaoa_profile_launches(pl.h, 32, ctypes.byref(cnt), None, _p(flags), None,
+                                       by.ctypes.data_as(ctypes.POINTER(ctypes.c_double))) == 0
+    states = by[:cnt.value] > 0
+    assert states.sum() >= 2
+    assert ((flags[:cnt.value] & 16 != 0) == (states & (not fields))).all()
     pl.close()
