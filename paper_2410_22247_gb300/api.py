@@ -423,8 +423,8 @@ def _autograd_function():
         @staticmethod
         def backward(ctx, grad_out):
             (out,) = ctx.saved_tensors
-            d = grad_out * out[1:]  # both gradients in one product
-            return d[:ctx.p], d[ctx.p:], None, None
+            # (a tensor each: halves of one product would share its storage and version counter)
+            return grad_out * out[1:1 + ctx.p], grad_out * out[1 + ctx.p:], None, None
 
     return AAQAOAFunction
 
