@@ -171,6 +171,7 @@ struct aaqaoa_plan {
     std::array<int, 4> tuned{};  // the plan that aaqaoa_autotune returned (zeros: none)
     bool fuse = true;  // fuse layer boundaries into one pass where the plan allows
     int *err_shared = nullptr;  // set when the plan is part of a multi-graph batch
+    bool stateless = false;  // group of one-CTA graphs of a batch: no state is ever stored
     const GraphFns *pt_dev = nullptr;  // set for a group of same-n graphs: point b is graph b
     int *d_err() const { return err_shared ? err_shared : reinterpret_cast<int *>(ws + L.ctrl); }
     unsigned *d_counter_pass() const { return reinterpret_cast<unsigned *>(ws + L.ctrl + 8); }
@@ -265,12 +266,14 @@ Layout layout(const aaqaoa_plan *pl, int batch, bool grad)
     L.zz = off;
     off = align256(off + (size_t)(pl->m > 0 ? pl->m : 1) * sizeof(double));
     L.samp = off;
-    off = align256(off + (sample_chunk_count(pl->n) + 32 + 2 * (size_t)AAQAOA_SAMPLE_MAX) * sizeof(double) +
+    if (!pl->stateless)
+        off = align256(off + (sample_chunk_count(pl->n) + 32 + 2 * (size_t)AAQAOA_SAMPLE_MAX) * sizeof(double) +
                    (size_t)AAQAOA_SAMPLE_MAX * sizeof(int));
     L.ising = off;
     off = align256(off + (pl->ising ? 3 * sizeof(IsingFn) : 0));
     L.phi = off;
-    off = align256(off + B * ((size_t)1 << pl->n) * pl->amp());
+    if (!pl->stateless)
+        off = align256(off + B * ((size_t)1 << pl->n) * pl->amp());
     L.lam = off;
     if (grad && !pl->small())
         off = align256(off + B * ((size_t)1 << pl->n) * pl->amp());
@@ -2786,6 +2789,8 @@ int aaqaoa_prepare_multi(int G, const aaqaoa_graph_desc *graphs, int p, unsigned
             aaqaoa_destroy_multi(m);
             return r;
         }
+        // (always one whole-circuit launch, which stores nothing: see use_circuit)
+        g.pl->stateless = g.pl->small();
         for (int gi : g.members)  // tables long enough for every member's cut values
             g.pl->wsum = std::max(g.pl->wsum, m->plans[gi]->wsum);
         m->order.insert(m->order.end(), g.members.begin(), g.members.end());

@@ -280,3 +280,17 @@ def test_launch_records_tell_halves_from_whole_states(lib, n, fields):
     assert states.sum() >= 2
     assert ((flags[:cnt.value] & 16 != 0) == (states & (not fields))).all()
     pl.close()
+
+
+@pytest.mark.parametrize("n,flags", [(13, 0), (12, 1), (5, 0)])
+def test_a_batch_of_small_graphs_stores_no_states(lib, n, flags):
+    """Graphs that run in one CTA or cluster need their functions, angles and results
+    in a batch's workspace, and no statevector each."""
+    G = 400
+    e = np.ascontiguousarray(W.cycle_graph(n)[1], dtype=np.int32).reshape(-1)
+    desc = (N.GraphDesc * G)(*[N.GraphDesc(n, len(e) // 2, _p(e), 0, None, None, None) for _ in range(G)])
+    h, size = ctypes.c_void_p(), ctypes.c_size_t()
+    assert lib.aaqaoa_prepare_multi(G, desc, 2, flags, None, ctypes.byref(h)) == 0
+    assert lib.aaqaoa_multi_workspace_bytes(h, ctypes.byref(size)) == 0
+    assert size.value < G * (12 << 10) + (1 << 20)
+    lib.aaqaoa_destroy_multi(h)
