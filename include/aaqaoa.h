@@ -437,9 +437,8 @@ int aaqaoa_inject_fault(aaqaoa_plan *plan, int kind);
  * enough for the whole-circuit kernel).
  *
  * aaqaoa_get_pass_plan: plan4 (host, 4 ints) receives the current plan. (Without
- *   forward entries set here that differ from the default, the forward sweep of a
- *   gradient may use other groups than an energy's, chosen to end on the
- *   adjoint's last: aaqaoa_get_schedule.)
+ *   a plan set here, the forward sweep of a gradient may use other groups than
+ *   an energy's, chosen to end on the adjoint's last: aaqaoa_get_schedule.)
  * aaqaoa_set_pass_plan: 0 keeps the default for that entry (the fewest high
  *   passes; a two-register-stage low pass when they can take the rest).
  *   For complex64 plans the adjoint's low pass may span 14 qubits (bwd_low =
@@ -452,8 +451,9 @@ int aaqaoa_inject_fault(aaqaoa_plan *plan, int kind);
  *   MaxCut energies and gradients of up to 20 qubits run as one whole-circuit
  *   launch where that is faster; a plan set here (any non-zero entry), like
  *   layer fusion switched off, makes them run the tiled passes. Setting what
- *   aaqaoa_autotune returned for this plan restores what it left; a new plan that
- *   is given another one's tuned entries takes its passes as written here.
+ *   aaqaoa_autotune returned for this plan restores what it left, and above 20
+ *   qubits the default written out in full is the default; a new plan that is
+ *   given another one's tuned entries takes its passes as written here.
  *   Rebuilds the workspace's tensor maps; the stored state becomes invalid.
  * aaqaoa_autotune: times each candidate (the fewest and one more high pass,
  *   each with the full and the two-stage low pass, and for the complex64

@@ -1612,8 +1612,8 @@ int aaqaoa_set_workspace(aaqaoa_plan *pl, void *device_ptr, size_t bytes, int ba
 // A layer's qubits per pass (the low pass's qubit count L and the number K of
 // high passes) for the forward (nv = 1) and the two-vector adjoint (nv = 2)
 // passes. 0 selects the default of build_passes(). A gradient's forward passes are
-// the forward's if the caller asks for others than the default (forced), else
-// those that follow the adjoint (gradient_passes).
+// an energy's if the caller asks for a plan of its own (forced), else those that
+// follow the adjoint (gradient_passes).
 static int set_layers(aaqaoa_plan *pl, const int plan4[4], bool forced = false)
 {
     if (pl->small())
@@ -1624,8 +1624,6 @@ static int set_layers(aaqaoa_plan *pl, const int plan4[4], bool forced = false)
         pass_geometry(pl->c128, nv, &T, &CB, &HB);
         const int L2 = low_two_stage_bits(pl->c128, nv);
         default_layer(pl->n, T, CB, HB, L2, &L, &K, nv == 2);
-        if (nv == 1)
-            forced = forced && ((plan4[0] > 0 && plan4[0] != L) || (plan4[1] > 0 && plan4[1] != K));
         if (plan4[2 * (nv - 1)] > 0)
             L = plan4[2 * (nv - 1)];
         if (plan4[2 * (nv - 1) + 1] > 0)
@@ -1661,8 +1659,16 @@ int aaqaoa_set_pass_plan(aaqaoa_plan *pl, int fwd_low, int fwd_high, int bwd_low
     if (fwd_low < 0 || fwd_high < 0 || bwd_low < 0 || bwd_high < 0)
         return fail(AAQAOA_ERR_INVALID_ARG, "negative pass-plan entry");
     const int plan4[4] = {fwd_low, fwd_high, bwd_low, bwd_high};
+    // not a plan of the caller's own: what autotune returned; the default (up to 20
+    // qubits that asks for the passes)
+    int own[4] = {0, 0, 0, 0};
+    for (int nv = 1; nv <= 2 && pl->n > CIRCUIT_MAX_QUBITS; nv++) {
+        int T, CB, HB;
+        pass_geometry(pl->c128, nv, &T, &CB, &HB);
+        default_layer(pl->n, T, CB, HB, low_two_stage_bits(pl->c128, nv), &own[2 * nv - 2], &own[2 * nv - 1], nv == 2);
+    }
     const bool forced = (fwd_low || fwd_high || bwd_low || bwd_high) &&
-                        !std::equal(plan4, plan4 + 4, pl->tuned.begin());
+                        !std::equal(plan4, plan4 + 4, pl->tuned.begin()) && !std::equal(plan4, plan4 + 4, own);
     const int r = set_layers(pl, plan4, forced);
     if (!r)
         pl->forced = forced;
