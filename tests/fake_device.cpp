@@ -21,6 +21,7 @@ std::vector<std::function<void()>> g_queue;
 int g_changed = 0;    // sources of queued copies that changed before the copy ran
 int g_expire = 0;     // the next launch with a bounded wait finds it expired
 int g_circuits = 0;   // whole-circuit launches
+int g_lose = 0;       // the next whole-circuit launch writes nothing
 int g_no_pinned = 0;  // cudaHostAlloc fails
 
 __attribute__((noinline)) void clobber_stack()
@@ -56,6 +57,7 @@ extern "C" {
 int fake_changed_sources() { return g_changed; }
 void fake_expire_next_wait() { g_expire = 1; }
 int fake_circuit_launches() { return g_circuits; }
+void fake_lose_next_launch() { g_lose = 1; }
 void fake_no_pinned_memory(int on) { g_no_pinned = on; }
 
 cudaError_t cudaGetLastError() { return cudaSuccess; }
@@ -165,6 +167,10 @@ int launch_circuit(bool, bool grad, const CircuitArgs &a, const CircuitPlan &q, 
 {
     g_circuits++;
     g_queue.push_back([=] {
+        if (g_lose) {
+            g_lose = 0;
+            return;
+        }
         const bool team = q.c && !q.cluster;
         if (team && (g_expire || a.drop_arrival))
             *a.err = 1;

@@ -198,3 +198,34 @@ def test_unreported_timeout_reaches_the_next_host_call(n, prec):
         with pytest.raises(N.AAQAOAError, match="TIMEOUT"):
             call()
         assert call() == want
+
+
+@pytest.mark.parametrize("n,prec", [(4, "c64"), (10, "c64"), (12, "c128"), (16, "c64"), (18, "c64"), (20, "c128"),
+                                    (22, "c64")])
+def test_device_calls_replay_from_a_captured_graph(n, prec):
+    """A gradient call captured into the caller's CUDA graph reads the angles of the
+    replay: one CTA, a cluster, a team (a cooperative launch), the passes."""
+    import torch
+    from paper_2410_22247_gb300.api import Plan
+    n, e = W.cycle_graph(n)
+    st = torch.cuda.Stream()
+    with torch.cuda.stream(st):
+        pl = Plan(n, e, 2, orbits=ORB.edge_orbits(n, e), precision=prec, stream=st)
+        dg = torch.zeros(2, dtype=torch.float64, device="cuda")
+        db = torch.zeros(2, dtype=torch.float64, device="cuda")
+        out = torch.zeros(5, dtype=torch.float64, device="cuda")
+        pl.grad_device(dg, db, out, "red")
+        pl.sync()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=st):
+        pl.grad_device(dg, db, out, "red")
+    for seed in (2, 3):
+        g, b = W.random_angles(2, seed)
+        dg.copy_(torch.tensor(g))
+        db.copy_(torch.tensor(b))
+        torch.cuda.synchronize()
+        graph.replay()
+        torch.cuda.synchronize()
+        pl.sync()
+        row = out.cpu().numpy()
+        _check((row[0], row[1:3], row[3:]), O.energy_grad(n, e, g, b), prec)

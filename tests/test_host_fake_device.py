@@ -294,3 +294,18 @@ def test_a_batch_of_small_graphs_stores_no_states(lib, n, flags):
     assert lib.aaqaoa_multi_workspace_bytes(h, ctypes.byref(size)) == 0
     assert size.value < G * (12 << 10) + (1 << 20)
     lib.aaqaoa_destroy_multi(h)
+
+
+@pytest.mark.parametrize("n", [10, 14, 18])
+def test_a_launch_without_a_result_is_an_error(lib, n):
+    """A one-point host call whose pinned row stays unwritten does not return the row
+    of the call before."""
+    pl = FakePlan(lib, W.cycle_graph(n), 1)
+    x, y = np.array([0.3]), np.array([0.1])
+    assert pl.expect(x, y)[0] == 0
+    for call in (pl.expect, pl.grad):
+        lib.fake_lose_next_launch()
+        assert call(x, y)[0] == -4
+        rc, E = call(x, y)
+        assert rc == 0 and abs(E - pl.value(x, y)) < 1e-9
+    pl.close()
