@@ -20,6 +20,7 @@ own GPU (independent evaluations, no collective on the data path) and
 from __future__ import annotations
 
 import argparse
+import ctypes
 import json
 import math
 import os
