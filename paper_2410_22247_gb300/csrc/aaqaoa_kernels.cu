@@ -820,7 +820,7 @@ __global__ void __launch_bounds__(256) k_agg_fused(const __grid_constant__ AggAr
 // so that a chunk costs one FP64 addition per term and warp, each term owned
 // by a lane, instead of one per term and lane: 42 terms at n = 28 took 2.3 ms
 // of selects and FP64 additions against 0.16 ms of memory time, and take 0.4.
-// One term reads the state at 5.4-6.0 TB/s (n = 28, 30). The lanes'
+// One term reads the stored half at 5.3-5.8 TB/s (n = 28, 30). The lanes'
 // sums carry their rounding errors along (float pairs, TwoSum), as the FP64
 // sums over lanes did.
 template <typename R> struct LaneSum;
@@ -835,12 +835,21 @@ template <> struct LaneSum<float> {
         const float e = __fadd_rn(__fsub_rn(a, __fsub_rn(t, z)), __fsub_rn(b, z));
         return {t, __fadd_rn(__fadd_rn(la, lb), e)};
     }
-    // sums of chunks in FP64
-    __device__ __forceinline__ void add_to(double &a, bool neg) const
-    {
-        const double v = (double)hi + (double)lo;
-        a += neg ? -v : v;
-    }
+    // sums of chunks: the rounded parts in FP64, the rounding errors (2^-24 of
+    // them) in a pair of floats, 2^-72 of the sum (adding them in FP64, two more
+    // FP64 operations a chunk: a read for one term at n = 28 0.219 ms, this 0.202)
+    struct Sum {
+        double a = 0.0;
+        float l = 0.f, e = 0.f;
+        __device__ __forceinline__ void add(const LaneSum &v, bool neg)
+        {
+            const float x = neg ? -v.lo : v.lo, t = __fadd_rn(l, x), z = __fsub_rn(t, l);
+            a += (double)(neg ? -v.hi : v.hi);
+            e = __fadd_rn(e, __fadd_rn(__fsub_rn(l, __fsub_rn(t, z)), __fsub_rn(x, z)));
+            l = t;
+        }
+        __device__ __forceinline__ double value() const { return a + ((double)l + (double)e); }
+    };
 };
 template <> struct LaneSum<double> {
     double v;
@@ -849,7 +858,11 @@ template <> struct LaneSum<double> {
     {
         return {(neg ? -v : v) + __shfl_xor_sync(0xffffffffu, v, o)};
     }
-    __device__ __forceinline__ void add_to(double &a, bool neg) const { a += neg ? -v : v; }
+    struct Sum {
+        double a = 0.0;
+        __device__ __forceinline__ void add(const LaneSum &x, bool neg) { a += neg ? -x.v : x.v; }
+        __device__ __forceinline__ double value() const { return a; }
+    };
 };
 
 template <typename R>
@@ -923,7 +936,8 @@ __global__ void __launch_bounds__(256, std::is_same<R, float>::value ? 2 : 1) k_
                 cmask[t >> 5] = cm;
             }
         }
-        double acc[2] = {0.0, 0.0}, pacc[PAIRS];
+        typename LS::Sum acc[2];
+        double pacc[PAIRS];
 #pragma unroll
         for (int i = 0; i < PAIRS; i++)
             pacc[i] = 0.0;
@@ -973,12 +987,12 @@ __global__ void __launch_bounds__(256, std::is_same<R, float>::value ? 2 : 1) k_
 #pragma unroll
             for (int q = 0; q < 2; q++)
                 if (idx[q] >= 0)
-                    vals[warp][idx[q]].add_to(acc[q], __popcll((ch << 10) & cmask[q]) & 1);
+                    acc[q].add(vals[warp][idx[q]], __popcll((ch << 10) & cmask[q]) & 1);
         }
 #pragma unroll
         for (int q = 0; q < 2; q++)
             if (idx[q] >= 0)
-                wsum[lane + 32 * q][warp] = acc[q];
+                wsum[lane + 32 * q][warp] = acc[q].value();
 #pragma unroll
         for (int i = 0; i < PAIRS; i++)
             if ((needp >> i) & 1) {
