@@ -2,7 +2,8 @@
 
 Workload (one "step" = one evaluation of the whole hot path): the star S_29
 (n = 30 qubits, 29 edges, one edge orbit of weight 29), p = 2 layers,
-complex64 amplitudes with FP64 reductions, observable H_red, energy and the
+complex64 amplitudes (a thread sums the few products of a register stage in
+single precision, everything beyond in FP64), observable H_red, energy and the
 adjoint gradient with respect to all 2p angles. The stored half of the statevector (4.3 GB) is
 far larger than L2, so no flush is needed between steps.
 
