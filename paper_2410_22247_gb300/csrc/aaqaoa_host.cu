@@ -992,11 +992,17 @@ class HostSlots {
         if (!s.tried) {
             s.tried = true;
             void *p = nullptr;
+            // (another thread may be capturing a graph in the global mode, which an
+            // allocation made here in that mode would invalidate)
+            cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+            const bool relaxed = cudaThreadExchangeStreamCaptureMode(&mode) == cudaSuccess;
             if (cudaHostAlloc(&p, sizeof(double) * COUNT * ROW, cudaHostAllocPortable | cudaHostAllocMapped) ==
                 cudaSuccess)
                 s.base = static_cast<double *>(p);
             else
                 (void)cudaGetLastError();
+            if (relaxed)
+                cudaThreadExchangeStreamCaptureMode(&mode);
         }
         if (!s.base || !~s.used)
             return nullptr;

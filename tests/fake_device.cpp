@@ -9,6 +9,7 @@
 #include <cmath>
 #include <cstring>
 #include <functional>
+#include <utility>
 #include <vector>
 
 #include "aaqaoa_internal.h"
@@ -23,6 +24,8 @@ int g_expire = 0;     // the next launch with a bounded wait finds it expired
 int g_circuits = 0;   // whole-circuit launches
 int g_lose = 0;       // the next whole-circuit launch writes nothing
 int g_no_pinned = 0;  // cudaHostAlloc fails
+cudaStreamCaptureMode g_mode = cudaStreamCaptureModeGlobal;  // this thread's
+int g_unsafe = 0;     // allocations that would invalidate another thread's global capture
 
 __attribute__((noinline)) void clobber_stack()
 {
@@ -59,6 +62,8 @@ void fake_expire_next_wait() { g_expire = 1; }
 int fake_circuit_launches() { return g_circuits; }
 void fake_lose_next_launch() { g_lose = 1; }
 void fake_no_pinned_memory(int on) { g_no_pinned = on; }
+int fake_unsafe_allocations() { return g_unsafe; }
+int fake_capture_mode() { return (int)g_mode; }
 
 cudaError_t cudaGetLastError() { return cudaSuccess; }
 const char *cudaGetErrorName(cudaError_t) { return "fake"; }
@@ -111,9 +116,16 @@ cudaError_t cudaMemsetAsync(void *dst, int v, size_t n, cudaStream_t)
 cudaError_t cudaStreamSynchronize(cudaStream_t) { run_queue(); return cudaSuccess; }
 cudaError_t cudaHostAlloc(void **p, size_t n, unsigned)
 {
+    if (g_mode != cudaStreamCaptureModeRelaxed)
+        g_unsafe++;
     if (g_no_pinned)
         return cudaErrorMemoryAllocation;
     *p = calloc(1, n);
+    return cudaSuccess;
+}
+cudaError_t cudaThreadExchangeStreamCaptureMode(cudaStreamCaptureMode *m)
+{
+    std::swap(*m, g_mode);
     return cudaSuccess;
 }
 cudaError_t cudaHostGetDevicePointer(void **d, void *h, unsigned) { *d = h; return cudaSuccess; }

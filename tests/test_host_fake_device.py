@@ -189,6 +189,16 @@ def test_host_calls_without_a_pinned_row(lib):
         pl.close()
 
 
+def test_the_pinned_rows_leave_captures_of_other_threads_alone(lib):
+    """The block of pinned rows is made in the relaxed capture mode (any other
+    would end a global-mode capture in another thread), which is then put back."""
+    pl = FakePlan(lib, W.cycle_graph(10), 1)
+    mode = lib.fake_capture_mode()
+    rc, _ = pl.expect(np.array([0.3]), np.array([0.1]))
+    assert rc == 0 and lib.fake_unsafe_allocations() == 0 and lib.fake_capture_mode() == mode == 0
+    pl.close()
+
+
 @pytest.mark.parametrize("n", [10, 14, 18])
 def test_device_results_over_their_angles(lib, n):
     """A result row that overlaps the angles is written only when they have been read."""
